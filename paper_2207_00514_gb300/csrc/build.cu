@@ -418,15 +418,15 @@ void launch_gather(Problem &P, const uint32_t *perm) {
 // k_build_local: one thread per leaf chunk climbs the splits between two of
 // its CTA's chunks, with the CTA's shared keys' delta values, boxes and
 // arrival counts in shared memory (block-scope acquire-release adds).  A
-// split at the CTA's edge ends the climb in global memory: the thread leaves
-// its far end in split_far, adds a device-scope acquire-release arrival, and
-// the second arriver lists the split.  A split inside the CTA that only one
-// child reached (the other spans CTAs) passes that child's far end to global
-// memory at the end.
+// split at the CTA's edge ends the climb in global memory: the thread
+// exchanges its arrival entry (device scope, acquire-release) and the second
+// arriver lists the split.  A split inside the CTA that only one child
+// reached (the other spans CTAs) passes that child's entry to global memory
+// at the end.
 // k_build_up: one thread per listed split builds it and climbs on in global
 // memory; a child's box comes from its record (the union of the record's two
 // child boxes) or from its points (a leaf).
-// Each split gets exactly two arrivals; the counters start at zero.
+// Each split gets exactly two arrivals; the entries start at zero.
 // The child labels are the round-0 ones (a one-point chunk k: label k;
 // otherwise several components, kInvalid); a caller with other labels
 // rewrites them (A5).
@@ -536,12 +536,23 @@ __device__ __forceinline__ void write_node(NodeRec *nodes, uint2 *__restrict__ n
   idmin = min(minL, minR);
 }
 
-// Arrival counters with acquire-release order: the first arriver's stores
-// (its box and far end) are released by its add, and the second arriver's
-// add acquires them, so no separate fences are needed around the add.
-__device__ __forceinline__ uint32_t add_acq_rel_gpu(uint32_t *p, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+// A split's arrival entry: 0 until a child arrives, then that child's far end
+// and outer delta (the leading bits its far end's key shares with the key
+// beyond it), so the second arriver learns from its own exchange the parent's
+// whole range and both deltas that say where the parent hangs: no load of
+// either before the sibling's box.  Acquire-release order: the first arriver's
+// stores (its record) are released by its exchange and acquired by the
+// second's.  (With a counter, the far end and the deltas' keys loaded after
+// it, a level above the CTAs took four dependent round trips instead of two:
+// k_build_up 131 -> 78 us at 200,000 halo points, 644 -> 418 us at 37M.)
+__device__ __forceinline__ uint64_t pack_arrival(uint32_t far, int outer_delta) {
+  return (1ull << 63) | ((uint64_t)(uint32_t)(outer_delta + 1) << 32) | (uint64_t)far;
+}
+__device__ __forceinline__ uint32_t arrival_far(uint64_t a) { return (uint32_t)a; }
+__device__ __forceinline__ int arrival_delta(uint64_t a) { return (int)((a >> 32) & 0x7fffffffu) - 1; }
+__device__ __forceinline__ uint64_t exch_acq_rel_gpu(uint64_t *p, uint64_t v) {
+  uint64_t old;
+  asm volatile("atom.acq_rel.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
   return old;
 }
 __device__ __forceinline__ uint32_t add_acq_rel_cta_shared(uint32_t *p, uint32_t v) {
@@ -551,11 +562,17 @@ __device__ __forceinline__ uint32_t add_acq_rel_cta_shared(uint32_t *p, uint32_t
   return old;
 }
 
+// A split both of whose children k_build_local finished: the split, the
+// parent's range, and the deltas outside it (+ 1, the left one in the low half).
+__device__ __forceinline__ uint4 ready_entry(uint32_t ps, uint32_t L, uint32_t R, int dl, int dr) {
+  return make_uint4(ps, L, R, (uint32_t)(dl + 1) | ((uint32_t)(dr + 1) << 16));
+}
+
 __global__ void __launch_bounds__(kRefitBlock) k_build_local(
     const uint64_t *__restrict__ keys, const uint64_t *__restrict__ keys_hi,
     const float4 *__restrict__ pts, int64_t n, int64_t nc, int leaf, NodeRec *nodes,
-    uint2 *__restrict__ nlabels, uint2 *__restrict__ range, uint2 *split_far, uint32_t *arrivals,
-    uint32_t *__restrict__ ready, uint32_t *ready_count, uint32_t capacity, uint32_t *status) {
+    uint2 *__restrict__ nlabels, uint2 *__restrict__ range, uint64_t *arrivals,
+    uint4 *__restrict__ ready, uint32_t *ready_count, uint32_t capacity, uint32_t *status) {
   __shared__ int s_delta[kRefitBlock + 1];     // delta(first - 1 + t)
   __shared__ float s_box[kRefitBlock][2][6];   // both child boxes of each split inside the CTA
   __shared__ uint32_t s_min[kRefitBlock][2];   // their smallest original ids
@@ -581,10 +598,14 @@ __global__ void __launch_bounds__(kRefitBlock) k_build_local(
       const uint32_t far = side == 0 ? (uint32_t)l : (uint32_t)r;
       if ((int64_t)ps < first || (int64_t)ps >= last) {
         // a split at the CTA's edge: its other child lies (partly) in another CTA
-        reinterpret_cast<uint32_t *>(split_far + ps)[side] = far;
-        if ((add_acq_rel_gpu(arrivals + ps, 1u) & 1u) != 0u) {  // second: list it
+        const int dl = s_delta[l - first], dr = s_delta[r - first + 1];
+        const uint64_t sib = exch_acq_rel_gpu(arrivals + ps, pack_arrival(far, side == 0 ? dl : dr));
+        if (sib != 0u) {  // second: list it
           const uint32_t at = atomicAdd(ready_count, 1u);
-          if (at < capacity) ready[at] = ps;
+          if (at < capacity)
+            ready[at] = side == 0
+                            ? ready_entry(ps, (uint32_t)l, arrival_far(sib), dl, arrival_delta(sib))
+                            : ready_entry(ps, arrival_far(sib), (uint32_t)r, arrival_delta(sib), dr);
           else atomicOr(status, kErrChain);  // cannot happen (see launch_build_tree)
         }
         break;
@@ -623,41 +644,39 @@ __global__ void __launch_bounds__(kRefitBlock) k_build_local(
   }
   __syncthreads();
   // a split inside the CTA that one child reached: the other spans CTAs and
-  // arrives in k_build_up, which finds this one's far end in split_far
+  // arrives in k_build_up
   const int64_t s = first + threadIdx.x;
   if (s < last && s_arrive[threadIdx.x] == 1u) {
     const int side = s_far[threadIdx.x][0] != kInvalid ? 0 : 1;
-    reinterpret_cast<uint32_t *>(split_far + s)[side] = s_far[threadIdx.x][side];
-    arrivals[s] = 1u;
+    const uint32_t far = s_far[threadIdx.x][side];
+    arrivals[s] = pack_arrival(far, s_delta[(int64_t)far - first + side]);
   }
 }
 
 __global__ void __launch_bounds__(kRefitUpBlock) k_build_up(
-    const uint64_t *__restrict__ keys, const uint64_t *__restrict__ keys_hi,
     const float4 *__restrict__ pts, int64_t n, int64_t nc, int leaf, NodeRec *nodes,
-    uint2 *__restrict__ nlabels, uint2 *__restrict__ range, uint2 *split_far, uint32_t *arrivals,
-    const uint32_t *__restrict__ ready, const uint32_t *ready_count, uint32_t capacity,
+    uint2 *__restrict__ nlabels, uint2 *__restrict__ range, uint64_t *arrivals,
+    const uint4 *__restrict__ ready, const uint32_t *ready_count, uint32_t capacity,
     uint32_t *status) {
   const uint32_t count = min(*ready_count, capacity);
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < count; t += gridDim.x * blockDim.x) {
-    // a split both of whose children k_build_local finished
-    uint32_t ps = __ldg(ready + t);
-    const uint2 fe = __ldcg(split_far + ps);
-    if (fe.x > ps || fe.y <= ps || (int64_t)fe.y >= nc) {  // cannot happen: both children arrived
+    const uint4 e = __ldg(ready + t);
+    uint32_t ps = e.x;
+    if (e.y > ps || e.z <= ps || (int64_t)e.z >= nc) {  // cannot happen: both children arrived
       atomicOr(status, kErrChain);
       continue;
     }
     float box[6], sib[6];
     uint32_t idmin, sibmin;
-    child_box(pts, n, leaf, nodes, ps, fe.x == ps, box, idmin);
-    child_box(pts, n, leaf, nodes, ps + 1u, fe.y == ps + 1u, sib, sibmin);
-    int64_t L = fe.x, R = fe.y;
+    child_box(pts, n, leaf, nodes, ps, e.y == ps, box, idmin);
+    child_box(pts, n, leaf, nodes, ps + 1u, e.z == ps + 1u, sib, sibmin);
+    int64_t L = e.y, R = e.z;
+    int dl = (int)(e.w & 0xffffu) - 1, dr = (int)(e.w >> 16) - 1;
     int side = 0;  // the child whose box is in `box`
     while (true) {
       uint32_t ps2;
       int side2;
-      const bool up = parent_split(L, R, nc, prefix_delta(keys, keys_hi, nc, leaf, L - 1, L),
-                                   prefix_delta(keys, keys_hi, nc, leaf, R, R + 1), ps2, side2);
+      const bool up = parent_split(L, R, nc, dl, dr, ps2, side2);
       const uint32_t idx = node_index(L, R, !up, side2);
       if (side == 0)
         write_node(nodes, nlabels, range, idx, (uint32_t)L, ps, (uint32_t)R, box, sib, idmin, sibmin, n,
@@ -666,13 +685,13 @@ __global__ void __launch_bounds__(kRefitUpBlock) k_build_up(
         write_node(nodes, nlabels, range, idx, (uint32_t)L, ps, (uint32_t)R, sib, box, sibmin, idmin, n,
                    leaf, box, idmin);
       if (!up) break;
-      // arrive at the parent's split; the record just written is released with the add
+      // arrive at the parent's split; the record just written is released with the exchange
       ps = ps2;
       side = side2;
-      const uint32_t far = side == 0 ? (uint32_t)L : (uint32_t)R;
-      reinterpret_cast<uint32_t *>(split_far + ps)[side] = far;
-      if ((add_acq_rel_gpu(arrivals + ps, 1u) & 1u) == 0u) break;  // first: the sibling carries on
-      const uint32_t sibfar = __ldcg(reinterpret_cast<const uint32_t *>(split_far + ps) + (side ^ 1));
+      const uint64_t other = exch_acq_rel_gpu(
+          arrivals + ps, pack_arrival(side == 0 ? (uint32_t)L : (uint32_t)R, side == 0 ? dl : dr));
+      if (other == 0u) break;  // first: the sibling carries on
+      const uint32_t sibfar = arrival_far(other);
       if (side == 0 ? (sibfar <= ps || (int64_t)sibfar >= nc) : sibfar > ps) {  // cannot happen
         atomicOr(status, kErrChain);
         break;
@@ -680,8 +699,13 @@ __global__ void __launch_bounds__(kRefitUpBlock) k_build_up(
       const uint32_t sidx = side == 0 ? ps + 1u : ps;  // the sibling's index or leaf chunk
       const bool sleaf = side == 0 ? sibfar == ps + 1u : sibfar == ps;
       child_box(pts, n, leaf, nodes, sidx, sleaf, sib, sibmin);
-      if (side == 0) R = sibfar;
-      else L = sibfar;
+      if (side == 0) {
+        R = sibfar;
+        dr = arrival_delta(other);
+      } else {
+        L = sibfar;
+        dl = arrival_delta(other);
+      }
     }
   }
 }
@@ -689,21 +713,21 @@ __global__ void __launch_bounds__(kRefitUpBlock) k_build_up(
 void launch_build_tree(Problem &P) {
   // A listed split has both children inside CTAs of k_build_local but lies at
   // the edge of one, so it is the boundary between two: fewer listed splits
-  // than k_build_local has CTAs.  list_buf[1] (n entries) is free until the
-  // rounds.
-  uint32_t *ready = P.list_buf[1];
+  // than k_build_local has CTAs, so n / 4 entries are room enough.  list_buf[1]
+  // (n words) is free until the rounds.
+  uint4 *ready = reinterpret_cast<uint4 *>(P.list_buf[1]);
+  const uint32_t capacity = (uint32_t)(P.n / 4);
   uint32_t *ready_count = P.counters + kRefitReadyCounter;
-  uint2 *split_far = P.split_far;
   cudaMemsetAsync(ready_count, 0, sizeof(uint32_t), P.stream);
   const int64_t ctas = grid_for(P.nc, kRefitBlock);
   k_build_local<<<(unsigned)ctas, kRefitBlock, 0, P.stream>>>(
-      P.keys[0] /*sorted*/, P.code_hi, P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels, P.range, split_far,
-      P.arrivals, ready, ready_count, (uint32_t)P.n, P.counters + 1);
+      P.keys[0] /*sorted*/, P.code_hi, P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels, P.range,
+      P.arrivals, ready, ready_count, capacity, P.counters + 1);
   int64_t g = ctas / kRefitUpBlock + 1;
   if (g > (int64_t)sm_count() * 16) g = (int64_t)sm_count() * 16;
-  k_build_up<<<(unsigned)g, kRefitUpBlock, 0, P.stream>>>(
-      P.keys[0], P.code_hi, P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels, P.range, split_far,
-      P.arrivals, ready, ready_count, (uint32_t)P.n, P.counters + 1);
+  k_build_up<<<(unsigned)g, kRefitUpBlock, 0, P.stream>>>(P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels,
+                                                          P.range, P.arrivals, ready, ready_count,
+                                                          capacity, P.counters + 1);
   P.launches += 2;
 }
 

@@ -257,9 +257,7 @@ struct Problem {
                                       // else nullptr; the sorted low words are keys[0]
   NodeRec *nodes = nullptr;       // nc-1 internal nodes
   uint2 *nlabels = nullptr;       // nc-1: child labels of each internal node (A5)
-  uint2 *split_far = nullptr;        // nc-1: per split of the build, the far end of the left
-                                     //      and of the right child that reached it
-  uint32_t *arrivals = nullptr;      // nc-1 arrival counters of the splits (parity = who is second)
+  uint64_t *arrivals = nullptr;      // nc-1: per split of the build, the child that arrived first (0: none)
   uint2 *range = nullptr;            // nc-1: each internal node's leaf-chunk range [first, last]
                                      //      and split (the last chunk of its left child), packed
                                      //      by pack_range (one end of the range is the node itself)
