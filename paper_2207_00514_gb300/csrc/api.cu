@@ -568,6 +568,9 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     stats->struct_size = sz;
   }
   if (n == 0) return EMST_OK;
+  // a small problem with nothing to choose or report: one launch
+  if (!offsets && !opt && !stats && !ex && n >= 2 && n <= kSmallMaxPoints)
+    return small_emst(points, n, dim, out, stream);
   int block = 0, carried = 1, count = 0, leaf_req = 0, mrd_k = 0, morton_bits = 0, traversal = 0;
   int refill = 0, chunk = 0, ignore_tuning = 0, use_graph = 0;
   const float *mlp_params = nullptr;

@@ -385,6 +385,10 @@ void launch_rerun_mark(Problem &P);
 void launch_log_samples(Problem &P, int round, bool carried);
 void launch_edge_gather(Problem &P, int64_t m, const uint32_t *order, emst_edge *out);
 
+// small.cu: the whole EMST of 2 <= n <= kSmallMaxPoints points in one cooperative launch.
+constexpr int kSmallMaxPoints = 32768;  // (why there: small.cu)
+int small_emst(const float *points, int64_t n, int dim, emst_edge *out, cudaStream_t stream);
+
 // tuning.cu: the tuned traversal parameters for this device, dimension, form
 // and size (0 in a field: no choice); false when the tuning file has none.
 struct TuneChoice {
