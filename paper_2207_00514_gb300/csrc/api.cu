@@ -178,6 +178,8 @@ size_t layout(Problem &P, char *base, bool copy_points, bool copy_edges) {
     P.mlp = c.take<float>(EMST_MLP_PARAMS);
   }
   if (P.want_logging) P.log_count = c.take<unsigned long long>(1);
+  P.near_j = P.want_near ? c.take<uint4>(n) : nullptr;
+  P.near_w = P.want_near ? c.take<float4>(n) : nullptr;
   P.seen = P.want_count ? c.take<uint32_t>((nc - 1 + 31) / 32) : nullptr;
   P.core2 = P.want_mrd ? c.take<float>(n) : nullptr;
   P.wide_hi = P.wide || P.auto_wide ? c.take<uint64_t>(n) : nullptr;
@@ -656,6 +658,9 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
   P.queue_chunk = chunk;
   P.block = block;
   P.want_count = count != 0;
+  // near lists: the plain form on one-point leaves, searched from the host loop
+  P.want_near = !learned && !logging && !P.want_mrd && !P.persistent && P.leaf == 1 && carried &&
+                use_graph != 1;
   if (logging) {
     P.log_feat = ex->log_feat;
     P.log_target = ex->log_target;
@@ -712,7 +717,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
       launch_core_knn(P, mrd_k);
       if (stats) cudaEventRecord(cev[1], stream);
     }
-    reset_round_state(P);
+    if (!P.near_j) reset_round_state(P);  // (the near lists' first round needs neither)
     // Boruvka rounds (Fig. 3 loop): each round at least halves the number of
     // components of every unfinished instance, so more than ceil(log2 n)
     // rounds (n: the largest instance) means something is wrong.
@@ -722,7 +727,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
       if (stats && rounds < 40)
         stats->components_per_round[rounds] = n - (int64_t)host_counters[0];
       if (rounds > 0) launch_node_labels(P);
-      else launch_upper_bounds(P);
+      else if (!P.near_j) launch_upper_bounds(P);
       if (learned || logging) launch_comp_sizes(P);
       if (logging) launch_log_samples(P, rounds, rounds > 0 && carried);
       if (stats && rounds < 40) {

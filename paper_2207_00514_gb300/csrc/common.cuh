@@ -231,6 +231,9 @@ struct Problem {
   uint32_t *seen = nullptr;          // count runs: bitmap of the internal nodes visited this round
   bool ties = true;                  // the search needs its tie rule (a run of > 32 equal
                                      // codes exists; set after the build, true when unknown)
+  bool want_near = false;            // set before layout(): carve the near lists
+  uint4 *near_j = nullptr;           // n: each point's nearest points, by curve index
+  float4 *near_w = nullptr;          // n: their weights
   const float *mlp = nullptr;
   float *pred_r = nullptr;
   float *r_used = nullptr;

@@ -9,6 +9,10 @@
 namespace emst {
 
 constexpr int kBlock = 256;
+// P.counters slots of a round
+constexpr uint32_t kActiveCounter = 50;  // listed queries
+constexpr uint32_t kActiveQueue = 51;    // list entries handed out
+constexpr uint32_t kActiveDone = 52;     // tiles of k_active_count finished
 
 // The weight of curve neighbours k and k + 1 (core2: the mutual reachability
 // weight, §4.5).
@@ -277,31 +281,34 @@ void launch_upper_bounds(Problem &P) {
 // One thread per point, or (list != nullptr) a grid-stride pass over the
 // listed points (the certification reruns of the learned radius).
 template <bool CARRIED, bool RADIUS_IN, bool COUNT, bool SEEDED, bool CHUNKS, bool LEARNED,
-          bool FIRST, bool MRD, bool TIES = true, bool LBT = true>
+          bool FIRST, bool MRD, bool TIES = true, bool LBT = true, bool KEPT = true>
 __global__ void __launch_bounds__(kTraverseMaxBlock, EMST_TRAVERSE_MIN_BLOCKS) k_traverse(TravArgs A, const uint32_t *__restrict__ list,
                                                      const uint32_t *__restrict__ list_count) {
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (list && A.queue) {
     // the next 32 entries for this warp, in list order, so the queries in
     // flight stay a window of the list (and of the curve) that L2 holds
-    const uint32_t count = *list_count;
-    const int lane = threadIdx.x & 31;
     for (;;) {
-      uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(A.queue, 32u);
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (base >= count) break;
-      if (base + lane < count)
-        traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT>(
-            A, __ldg(list + base + lane));
+      const uint32_t lane = threadIdx.x & 31;
+      uint32_t at = 0;
+      if (lane == 0) at = atomicAdd(A.queue, 32u);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      const uint32_t count = *list_count;
+      if (at >= count) break;
+      at += lane;
+      if (at < count)
+        traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT, KEPT>(
+            A, __ldg(list + at));
       __syncwarp();
     }
   } else if (list) {
     const int64_t count = *list_count;
     for (int64_t t = gid; t < count; t += (int64_t)gridDim.x * blockDim.x)
-      traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT>(A, __ldg(list + t));
+      traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT, KEPT>(
+          A, __ldg(list + t));
   } else if (gid < A.n) {
-    traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT>(A, gid);
+    traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT, KEPT>(
+        A, (uint32_t)gid);
   }
 }
 
@@ -451,7 +458,7 @@ static void launch_traverse_queue(Problem &P, const TravArgs &A, bool carried, b
 
 // ---------------------------------------------------------------------------
 // The queries of a round that need a search (rounds from kCompactFromRound
-// on, where many points skip theirs): a point whose lower bound exceeds its
+// on, where many points skip theirs; from round 1 on with near lists): a point whose lower bound exceeds its
 // component's cutoff as the round starts (upper bound, best so far) is
 // finished here exactly as traverse_one would finish it; the others are
 // listed in curve order (k_active_count flags them and counts them per tile,
@@ -472,16 +479,258 @@ static void launch_traverse_queue(Problem &P, const TravArgs &A, bool carried, b
 #define EMST_COMPACT_FROM_ROUND 2
 #endif
 constexpr int kCompactFromRound = EMST_COMPACT_FROM_ROUND;
-constexpr uint32_t kActiveCounter = 50;  // P.counters slot: listed queries
-constexpr uint32_t kActiveQueue = 51;    // P.counters slot: list entries handed out
-constexpr uint32_t kActiveDone = 52;     // P.counters slot: tiles of k_active_count finished
 #ifndef EMST_ORDERED_UNTIL_ROUND
 #define EMST_ORDERED_UNTIL_ROUND 6
 #endif
 constexpr int kOrderedUntilRound = EMST_ORDERED_UNTIL_ROUND;  // exact curve order before this round
-#ifndef EMST_LIST_QUEUE
-#define EMST_LIST_QUEUE 1
-#endif
+
+// ---------------------------------------------------------------------------
+// Near lists (the plain form on one-point leaves).  The first round looks for
+// every point's kNear nearest points by (w, original id) instead of one, with
+// the same search: it keeps the kNear best in registers and cuts off at the
+// last of them, and starts from the kNear-th smallest weight to its kNearSeed
+// curve neighbours on each side.  In the next rounds the first list entry that lies in another
+// component is the point's exact nearest one, with no search: the entries
+// before it are the only nearer points there are.  With four entries that
+// settles 92 % of the points in round 1 and 46 % in round 2 of a halo cloud;
+// the settled points' edges tighten the cutoffs before any search starts, and
+// a point whose list is used up has its last entry's weight as lower bound.
+// At 37M halo points the searches of rounds 1 / 2 / 3 fall from 32.4 / 24.7 /
+// 15.2M to 0.9 / 7.4 / 10.4M and the traversal from 29.3 to 22.8 ms (round 0
+// 6.6 -> 11.6, rounds 1-3 8.4 / 6.5 / 3.2 -> 1.4 / 2.5 / 2.4), the call from
+// 44.5 to 38 ms.  Bound, like the search it replaces, by the L1 data pipe and
+// divergence.  Lists read in rounds 1-2 / 1-3 / 1-4 / 1-5: 38.7 / 38.2 / 38.5
+// / 38.8 ms; kNearSeed 2 / 3 / 6: round 0 12.18 / 11.86 / 11.56 ms; 40 and 36
+// instead of 32 registers: 12.36 and 12.2 ms.
+// ---------------------------------------------------------------------------
+constexpr int kNear = 4;
+constexpr int kNearSeed = 6;
+constexpr int kNearRounds = 3;
+static_assert(kNearRounds < EMST_ORDERED_UNTIL_ROUND, "the ordered listing reads the settled points");
+
+// The candidate c at weight d <= w[kNear - 1] among the kNear best so far (w
+// ascending, ties by original id; kInvalid at +inf: empty).  Some lane of a
+// warp inserts at nearly every node it visits, so the case without a tie is a
+// fixed run of min / max and selects.
+__device__ __forceinline__ void near_insert(float (&w)[kNear], uint32_t (&j)[kNear], float d, uint32_t c,
+                                            const float4 *__restrict__ pts) {
+  bool before[kNear], tie = false;  // does c come before entry t?  (ascending in t)
+#pragma unroll
+  for (int t = 0; t < kNear; ++t) {
+    before[t] = d < w[t];
+    tie = tie || d == w[t];
+  }
+  if (tie) {
+    const uint32_t id = __float_as_uint(__ldg(&pts[c].w));
+#pragma unroll
+    for (int t = 0; t < kNear; ++t)
+      if (d == w[t]) before[t] = j[t] == kInvalid || id < __float_as_uint(__ldg(&pts[j[t]].w));
+    if (!before[kNear - 1]) return;
+  }
+#pragma unroll
+  for (int t = kNear - 1; t > 0; --t) {
+    w[t] = fmaxf(w[t - 1], fminf(w[t], d));
+    j[t] = before[t - 1] ? j[t - 1] : before[t] ? c : j[t];
+  }
+  w[0] = fminf(w[0], d);
+  j[0] = before[0] ? c : j[0];
+}
+
+constexpr int kNearBlock = 128;
+
+// The first round (every point its own component): the lists, and the first
+// entry's edge as the component's minimum (no other query offers to it).
+template <bool TIES, bool COUNT>
+__global__ void __launch_bounds__(kNearBlock, 16) k_near(TravArgs A) {
+  const float kInf = __int_as_float(0x7f800000);
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= A.n) return;
+  float w[kNear];
+  uint32_t j[kNear];
+#pragma unroll
+  for (int t = 0; t < kNear; ++t) {
+    w[t] = kInf;
+    j[t] = kInvalid;
+  }
+  uint32_t node = 0u;
+  int64_t lo = 0, hi = A.n;  // the instance's curve positions
+  if (A.inst_of) {
+    const uint32_t I = __ldg(A.inst_of + i);
+    node = __ldg(A.inst_root + I);
+    lo = __ldg(A.offsets + I);
+    hi = __ldg(A.offsets + I + 1);
+  }
+  const float4 p = __ldg(A.pts + i);
+  unsigned long long nvis = 0;
+  if (node != kInvalid) {  // (kInvalid: a one-point instance)
+    // a real kNear-th smallest weight: the cutoff to begin with (inclusive)
+    float c[kNear];
+#pragma unroll
+    for (int t = 0; t < kNear; ++t) c[t] = kInf;
+#pragma unroll
+    for (int o = 1; o <= kNearSeed; ++o) {
+#pragma unroll
+      for (int side = -1; side <= 1; side += 2) {
+        const int64_t k = i + side * o;
+        if (k < lo || k >= hi) continue;
+        const float4 q = __ldg(A.pts + k);
+        const float d = sq_dist(p.x, p.y, p.z, q.x, q.y, q.z);
+#pragma unroll
+        for (int t = kNear - 1; t > 0; --t) c[t] = fminf(fmaxf(c[t - 1], d), c[t]);
+        c[0] = fminf(c[0], d);
+      }
+    }
+    float radius = c[kNear - 1];
+    uint32_t st_node[kStackDepth];
+    float st_dist[kStackDepth];
+    int sp = 0;
+    while (true) {
+      if (COUNT) {
+        ++nvis;
+        if (A.seen) atomicOr(A.seen + (node >> 5), 1u << (node & 31));
+      }
+      float4 a, b, cc;
+      uint4 dd;
+      load_record(A.nodes + node, a, b, cc, dd);
+      const float dL = box_dist(p.x, p.y, p.z, a.x, a.y, a.z, a.w, b.x, b.y);
+      const float dR = box_dist(p.x, p.y, p.z, b.z, b.w, cc.x, cc.y, cc.z, cc.w);
+      bool okL = dL <= radius, okR = dR <= radius;
+      if (okL && (dd.x & kLeafBit)) {
+        if (dd.x != (kLeafBit | (uint32_t)i)) {
+          near_insert(w, j, dL, dd.x & ~kLeafBit, A.pts);
+          radius = fminf(radius, w[kNear - 1]);
+        }
+        okL = false;
+      }
+      if (okR && (dd.y & kLeafBit)) {
+        if (dd.y != (kLeafBit | (uint32_t)i) && dR <= radius) {
+          near_insert(w, j, dR, dd.y & ~kLeafBit, A.pts);
+          radius = fminf(radius, w[kNear - 1]);
+        }
+        okR = false;
+      }
+      okL = okL && dL <= radius;
+      okR = okR && dR <= radius;
+      // (a child that only ties a full list's last entry: see explore)
+      if (TIES && A.ties && j[kNear - 1] != kInvalid &&
+          ((okL && dL == w[kNear - 1]) || (okR && dR == w[kNear - 1]))) {
+        const uint32_t id = __float_as_uint(__ldg(&A.pts[j[kNear - 1]].w));
+        const uint2 mn = __ldg(reinterpret_cast<const uint2 *>(A.nodes + node) + 7);
+        if (dL == w[kNear - 1] && mn.x >= id) okL = false;
+        if (dR == w[kNear - 1] && mn.y >= id) okR = false;
+      }
+      if (okL && okR) {
+        if (sp >= kStackDepth) {
+          atomicOr(A.status, kErrStack);
+          break;
+        }
+        if (dL <= dR) { st_node[sp] = dd.y; st_dist[sp] = dR; node = dd.x; }
+        else { st_node[sp] = dd.x; st_dist[sp] = dL; node = dd.y; }
+        ++sp;
+        continue;
+      }
+      if (okL) { node = dd.x; continue; }
+      if (okR) { node = dd.y; continue; }
+      bool found = false;
+      while (sp > 0) {
+        --sp;
+        if (st_dist[sp] <= radius) { node = st_node[sp]; found = true; break; }
+      }
+      if (!found) break;
+    }
+    if (COUNT) {
+      atomicAdd(A.visits, nvis);
+      atomicAdd(A.queries, 1ull);
+    }
+  }
+  A.near_j[i] = make_uint4(j[0], j[1], j[2], j[3]);
+  A.near_w[i] = make_float4(w[0], w[1], w[2], w[3]);
+  A.res[i] = make_uint2(0u, kInvalid);
+  CompBest best;
+  best.key = kEmptyKey;
+  best.mx = kEmptyKey;
+  if (j[0] != kInvalid) {
+    const uint32_t oi = __float_as_uint(__ldg(&A.pts[i].w)), oj = __float_as_uint(__ldg(&A.pts[j[0]].w));
+    best.key = ((uint64_t)__float_as_uint(w[0]) << 32) | (uint64_t)(oi < oj ? oi : oj);
+    best.mx = ((uint64_t)(oi < oj ? oj : oi) << 32) | (uint64_t)j[0];
+  }
+  A.comp[i] = best;
+}
+static_assert(kNear == 4, "lists are stored as one 16-byte entry of ids and one of weights");
+
+// Rounds 1 to kNearRounds, before the listing: every point whose nearest
+// other-component point is known without a search -- the one found in an
+// earlier round while it still lies in another component (components only
+// grow, so it is still the nearest), else the first such entry of its list --
+// offers that edge and is marked in `settled` (bit i & 31 of word i >> 5).
+// The others keep a lower bound: their list's last weight, if above theirs.
+__global__ void __launch_bounds__(256) k_settle(const float4 *__restrict__ pts,
+                                                const uint32_t *__restrict__ labels,
+                                                const uint4 *__restrict__ near_j,
+                                                const float4 *__restrict__ near_w,
+                                                const uint32_t *__restrict__ bound, CompBest *comp,
+                                                uint2 *__restrict__ res, int64_t n,
+                                                uint32_t *__restrict__ settled, uint32_t *status) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  bool known = false;
+  uint32_t me = 0;
+  uint2 r = make_uint2(0u, kInvalid);
+  if (i < n) {
+    me = __ldg(labels + i);
+    r = res[i];
+    known = r.y != kInvalid && __ldg(labels + r.y) != me;
+    if (!known) {
+      const uint4 e = __ldg(near_j + i);
+      const uint32_t ids[4] = {e.x, e.y, e.z, e.w};
+      uint32_t lab[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) lab[t] = ids[t] != kInvalid ? __ldg(labels + ids[t]) : me;
+      const float4 wv = __ldg(near_w + i);
+      const uint32_t ws[4] = {__float_as_uint(wv.x), __float_as_uint(wv.y), __float_as_uint(wv.z),
+                              __float_as_uint(wv.w)};
+      uint2 now = make_uint2(max(r.x, ws[3]), kInvalid);
+#pragma unroll
+      for (int t = 3; t >= 0; --t)
+        if (lab[t] != me) {
+          now = make_uint2(ws[t], ids[t]);
+          known = true;
+        }
+      if (now.x != r.x || now.y != r.y) res[i] = now;
+      r = now;
+    }
+  }
+  const unsigned word = __ballot_sync(0xffffffffu, known);
+  if (lane == 0 && i < n) settled[i >> 5] = word;
+  // offers: the component of the warp's first such lane makes one, not 32
+  bool off = known && r.x <= __ldg(bound + me);
+  const unsigned m = __ballot_sync(0xffffffffu, off);
+  if (m == 0u) return;
+  const uint32_t first = __shfl_sync(0xffffffffu, me, __ffs(m) - 1);
+  const bool same = off && me == first;
+  const uint32_t w = __reduce_min_sync(0xffffffffu, same ? r.x : 0xffffffffu);
+  if (same && r.x != w) off = false;
+  if (off) offer_kept(comp + me, pts, r.x, i, r.y, labels, status);
+}
+
+// Which of a thread's N consecutive positions pass the skip test: lower bound
+// at or below the component's cutoff as it stands.  (No query of the round
+// runs during the listing kernels, so the entries are fixed and may come
+// through L1: in the last rounds every point reads one of a handful of them.)
+template <int N>
+__device__ __forceinline__ uint32_t open_points(const uint32_t *__restrict__ bound,
+                                                const CompBest *__restrict__ comp, int64_t i0, int64_t n,
+                                                const uint32_t (&lab)[N], const uint32_t (&lower)[N]) {
+  uint32_t open = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (i0 + j >= n) continue;
+    const uint32_t cw =
+        (uint32_t)(__ldg(reinterpret_cast<const unsigned long long *>(&comp[lab[j]].key)) >> 32);
+    if (lower[j] <= min(__ldg(bound + lab[j]), cw)) open |= 1u << j;
+  }
+  return open;
+}
 
 // The same with one atomic per warp of 128 positions (four per thread):
 // the list is in curve order only within each warp's positions, which costs
@@ -489,7 +738,8 @@ constexpr int kOrderedUntilRound = EMST_ORDERED_UNTIL_ROUND;  // exact curve ord
 // pass's scan when few are (rounds from kOrderedUntilRound on).
 __global__ void __launch_bounds__(256) k_active(const uint32_t *__restrict__ labels,
                                                 const uint32_t *__restrict__ bound,
-                                                const CompBest *comp, uint2 *__restrict__ res,
+                                                const CompBest *__restrict__ comp,
+                                                const uint2 *__restrict__ res,
                                                 int64_t n, uint32_t *__restrict__ list,
                                                 uint32_t *count) {
   const int lane = threadIdx.x & 31;
@@ -497,37 +747,22 @@ __global__ void __launch_bounds__(256) k_active(const uint32_t *__restrict__ lab
   uint32_t act = 0;
   if (i0 < n) {
     uint32_t lab[4];
-    uint2 prev[4];
+    uint32_t prev[4];  // lower bounds
     if (i0 + 4 <= n) {  // 16-byte loads (i0 is a multiple of 4; the arrays are 256-B aligned)
       const uint4 l4 = *reinterpret_cast<const uint4 *>(labels + i0);
       const uint4 ra = reinterpret_cast<const uint4 *>(res + i0)[0];
       const uint4 rb = reinterpret_cast<const uint4 *>(res + i0)[1];
       lab[0] = l4.x; lab[1] = l4.y; lab[2] = l4.z; lab[3] = l4.w;
-      prev[0] = make_uint2(ra.x, ra.y); prev[1] = make_uint2(ra.z, ra.w);
-      prev[2] = make_uint2(rb.x, rb.y); prev[3] = make_uint2(rb.z, rb.w);
+      prev[0] = ra.x; prev[1] = ra.z;
+      prev[2] = rb.x; prev[3] = rb.z;
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         lab[j] = i0 + j < n ? labels[i0 + j] : 0u;
-        prev[j] = i0 + j < n ? res[i0 + j] : make_uint2(0u, kInvalid);
+        prev[j] = i0 + j < n ? res[i0 + j].x : 0u;
       }
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (i0 + j >= n) continue;
-      float r = bound_to_radius(__ldg(bound + lab[j]));
-      // (no query of the round has run yet, so the entries are fixed during
-      // this kernel and may come through L1: in the last rounds every point
-      // reads one of a handful of them)
-      const uint32_t cw =
-          (uint32_t)(__ldg(reinterpret_cast<const unsigned long long *>(&comp[lab[j]].key)) >> 32);
-      r = fminf(r, bound_to_radius(cw));
-      if (__uint_as_float(prev[j].x) > r) {
-        if (prev[j].y != kInvalid) res[i0 + j] = make_uint2(prev[j].x, kInvalid);
-      } else {
-        act |= 1u << j;
-      }
-    }
+    act = open_points<4>(bound, comp, i0, n, lab, prev);
   }
   const uint32_t c = (uint32_t)__popc(act);
   uint32_t x = c;
@@ -554,9 +789,9 @@ constexpr int kActiveTile = kActiveThreads * 8;
 static_assert(kActiveThreads == kScanThreads, "block_exclusive_scan runs on a CTA of kScanThreads");
 
 __global__ void __launch_bounds__(kActiveThreads) k_active_count(
-    const uint32_t *__restrict__ labels, const uint32_t *__restrict__ bound, const CompBest *comp,
-    uint2 *__restrict__ res, int64_t n, uint8_t *__restrict__ flags, uint32_t *tile_total,
-    uint32_t *tile_prefix, uint32_t *done, uint32_t *count) {
+    const uint32_t *__restrict__ labels, const uint32_t *__restrict__ bound, const CompBest *__restrict__ comp,
+    const uint2 *__restrict__ res, const uint8_t *__restrict__ settled, int64_t n,
+    uint8_t *__restrict__ flags, uint32_t *tile_total, uint32_t *tile_prefix, uint32_t *done, uint32_t *count) {
   __shared__ uint32_t s_warp[kActiveThreads / 32];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -565,7 +800,7 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_count(
   uint32_t act = 0;
   if (i0 < n) {
     uint32_t lab[8];
-    uint2 prev[8];
+    uint32_t prev[8];  // lower bounds
     if (i0 + 8 <= n) {  // 16-byte loads (i0 is a multiple of 8; the arrays are 256-B aligned)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -575,32 +810,18 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_count(
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
         const uint4 r = reinterpret_cast<const uint4 *>(res + i0)[h];
-        prev[2 * h] = make_uint2(r.x, r.y);
-        prev[2 * h + 1] = make_uint2(r.z, r.w);
+        prev[2 * h] = r.x;
+        prev[2 * h + 1] = r.z;
       }
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         lab[j] = i0 + j < n ? labels[i0 + j] : 0u;
-        prev[j] = i0 + j < n ? res[i0 + j] : make_uint2(0u, kInvalid);
+        prev[j] = i0 + j < n ? res[i0 + j].x : 0u;
       }
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (i0 + j >= n) continue;
-      float r = bound_to_radius(__ldg(bound + lab[j]));
-      // (no query of the round has run yet, so the entries are fixed during
-      // this kernel and may come through L1: in the last rounds every point
-      // reads one of a handful of them)
-      const uint32_t cw =
-          (uint32_t)(__ldg(reinterpret_cast<const unsigned long long *>(&comp[lab[j]].key)) >> 32);
-      r = fminf(r, bound_to_radius(cw));
-      if (__uint_as_float(prev[j].x) > r) {
-        if (prev[j].y != kInvalid) res[i0 + j] = make_uint2(prev[j].x, kInvalid);
-      } else {
-        act |= 1u << j;
-      }
-    }
+    act = open_points<8>(bound, comp, i0, n, lab, prev);
+    if (settled) act &= ~(uint32_t)settled[t];
     flags[t] = (uint8_t)act;
   }
   const uint32_t wsum = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(act));
@@ -665,7 +886,9 @@ static void launch_trav(TravKernel k, int g, int block, cudaStream_t s, const Tr
 #ifndef EMST_LB_FROM_ROUND
 #define EMST_LB_FROM_ROUND 2
 #endif
-static bool track_lower_bounds(int round) { return round < 0 || round >= EMST_LB_FROM_ROUND; }
+static bool track_lower_bounds(const Problem &P, int round) {
+  return round < 0 || round >= EMST_LB_FROM_ROUND || P.near_j != nullptr;
+}
 
 void launch_traverse(Problem &P, bool carried, const float *radius_in, int block, bool count,
                      bool seeded, int learned_pass, bool first, int round) {
@@ -693,6 +916,8 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
   A.pred_r = P.pred_r;
   A.r_used = P.r_used;
   A.queue = nullptr;
+  A.near_j = P.near_j;
+  A.near_w = P.near_w;
   // learned_pass: 0 = plain, 1 = with the proposed radii, 2 = rerun of the
   // listed points with the plain cutoff
   // the persistent work-queue form serves the plain rounds on one-point leaves
@@ -704,7 +929,20 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
   const uint32_t *list_count = learned_pass == 2 ? P.counters + 13 : nullptr;
   int g = learned_pass == 2 ? sm_count() * 8 : grid_for(P.n, block);
   cudaStream_t s = P.stream;
-  if (carried && seeded && !radius_in && learned_pass == 0 && round >= kCompactFromRound) {
+  if (P.near_j && first) {
+    // the lists; no later step of the round needs the bounds or the minima cleared
+    if (P.ties) {
+      if (count) k_near<true, true><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
+      else k_near<true, false><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
+    } else {
+      if (count) k_near<false, true><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
+      else k_near<false, false><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
+    }
+    P.launches += 1;
+    return;
+  }
+  if (carried && seeded && !radius_in && learned_pass == 0 &&
+      round >= (P.near_j ? 1 : kCompactFromRound)) {
     // the queries that need a search, listed in curve order (vals[1] and
     // keys[1] are free during the rounds: the list, and the flags and tile
     // counts behind it)
@@ -714,10 +952,18 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     uint8_t *flags = reinterpret_cast<uint8_t *>(P.keys[1]);
     uint32_t *tile_total = reinterpret_cast<uint32_t *>(P.keys[1]) + tiles * (kActiveTile / 8 / 4);  // after the flags
     uint32_t *tile_prefix = tile_total + tiles;
+    uint8_t *settled = nullptr;
+    if (P.near_j && round <= kNearRounds) {
+      uint32_t *words = reinterpret_cast<uint32_t *>(P.keys[0]);  // free during the rounds
+      k_settle<<<grid_for(P.n, 256), 256, 0, s>>>(P.pts, P.labels, P.near_j, P.near_w, P.bound, P.comp, P.res,
+                                                  P.n, words, P.counters + 1);
+      P.launches += 1;
+      settled = reinterpret_cast<uint8_t *>(words);
+    }
     if (round < kOrderedUntilRound) {
       cudaMemsetAsync(P.counters + kActiveDone, 0, sizeof(uint32_t), s);
-      k_active_count<<<(unsigned)tiles, kActiveThreads, 0, s>>>(P.labels, P.bound, P.comp, P.res, P.n,
-                                                               flags, tile_total, tile_prefix,
+      k_active_count<<<(unsigned)tiles, kActiveThreads, 0, s>>>(P.labels, P.bound, P.comp, P.res, settled,
+                                                               P.n, flags, tile_total, tile_prefix,
                                                                P.counters + kActiveDone, active_count);
       k_active_write<<<(unsigned)tiles, kActiveThreads, 0, s>>>(flags, tile_prefix, P.n, active);
       P.launches += 2;
@@ -730,72 +976,57 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     list = active;
     list_count = active_count;
     g = sm_count() * (2048 / block);  // one resident wave
-#if EMST_LIST_QUEUE
     A.queue = P.counters + kActiveQueue;  // warps take the list in order
     cudaMemsetAsync(A.queue, 0, sizeof(uint32_t), s);
-#endif
   }
-#define EMST_TRAV2(C, R, K, S, H, L) launch_trav(k_traverse<C, R, K, S, H, L, false, false>, g, block, s, A, list, list_count)
-#define EMST_TRAV_FIRST(K, H) launch_trav(k_traverse<false, false, K, true, H, false, true, false>, g, block, s, A, list, list_count)
-#define EMST_TRAV_MRD(C, K, H) launch_trav(k_traverse<C, false, K, true, H, false, false, true>, g, block, s, A, list, list_count)
-#define EMST_TRAV_NOTIES(C, F, H) launch_trav(k_traverse<C, false, false, true, H, false, F, false, false>, g, block, s, A, list, list_count)
-#define EMST_TRAV_NOTIES_NOLB() launch_trav(k_traverse<true, false, false, true, false, false, false, false, false, false>, g, block, s, A, list, list_count)
-#define EMST_TRAV_NOLB(K) launch_trav(k_traverse<true, false, K, true, false, false, false, false, true, false>, g, block, s, A, list, list_count)
-  const bool lbt = track_lower_bounds(round);
-#define EMST_TRAV(C, R, K, S, L)                       \
-  do {                                                 \
-    if (P.leaf > 1) EMST_TRAV2(C, R, K, S, true, L);   \
-    else EMST_TRAV2(C, R, K, S, false, L);             \
+#define EMST_LAUNCH(...) launch_trav(k_traverse<__VA_ARGS__>, g, block, s, A, list, list_count)
+// a host flag as a template argument
+#define EMST_IF(flag, B, ...)       \
+  do {                              \
+    if (flag) {                     \
+      constexpr bool B = true;      \
+      __VA_ARGS__;                  \
+    } else {                        \
+      constexpr bool B = false;     \
+      __VA_ARGS__;                  \
+    }                               \
   } while (0)
-  if (!P.ties && !count && seeded && !radius_in && learned_pass == 0 && !P.core2) {
-    // the plain form on input without large groups of identical points
-    const bool h = P.leaf > 1;
-    if (carried) {
-      if (h) EMST_TRAV_NOTIES(true, false, true);
-      else if (lbt) EMST_TRAV_NOTIES(true, false, false);
-      else EMST_TRAV_NOTIES_NOLB();
-    }
-    else if (first) { if (h) EMST_TRAV_NOTIES(false, true, true); else EMST_TRAV_NOTIES(false, true, false); }
-    else { if (h) EMST_TRAV_NOTIES(false, false, true); else EMST_TRAV_NOTIES(false, false, false); }
-  } else if (radius_in) {
-    EMST_TRAV(false, true, false, false, false);
+  const bool h = P.leaf > 1;
+  // a tighter lower bound is tracked only over one-point leaves
+  const bool lbt = track_lower_bounds(P, round) || h;
+  // whether a query looks at the neighbour of an earlier round: not where
+  // k_settle did, not in the round after the first (every point's nearest
+  // neighbour has merged with it), and not over the list (from the fourth
+  // round on hardly any still stands, and the search loop is faster without)
+  const bool kept = !(learned_pass == 0 && !P.core2 && (A.queue || round == 1));
+  if (radius_in) {
+    EMST_IF(h, H, EMST_LAUNCH(false, true, false, false, H, false, false, false));
   } else if (!seeded) {
-    EMST_TRAV(false, false, false, false, false);
+    EMST_IF(h, H, EMST_LAUNCH(false, false, false, false, H, false, false, false));
   } else if (learned_pass == 1) {
-    if (carried) {
-      if (count) EMST_TRAV(true, false, true, true, true); else EMST_TRAV(true, false, false, true, true);
-    } else {
-      if (count) EMST_TRAV(false, false, true, true, true); else EMST_TRAV(false, false, false, true, true);
-    }
+    EMST_IF(h, H, EMST_IF(count, K, EMST_IF(carried, C, EMST_LAUNCH(C, false, K, true, H, true, false, false))));
   } else if (P.core2) {  // mutual reachability weights (the plain form's rounds)
-    const bool h = P.leaf > 1;
-    if (carried) {
-      if (count) { if (h) EMST_TRAV_MRD(true, true, true); else EMST_TRAV_MRD(true, true, false); }
-      else { if (h) EMST_TRAV_MRD(true, false, true); else EMST_TRAV_MRD(true, false, false); }
-    } else {
-      if (count) { if (h) EMST_TRAV_MRD(false, true, true); else EMST_TRAV_MRD(false, true, false); }
-      else { if (h) EMST_TRAV_MRD(false, false, true); else EMST_TRAV_MRD(false, false, false); }
-    }
+    if (carried)
+      EMST_IF(h, H, EMST_IF(count, K, EMST_IF(kept, T, EMST_LAUNCH(true, false, K, true, H, false, false, true, true, true, T))));
+    else
+      EMST_IF(h, H, EMST_IF(count, K, EMST_LAUNCH(false, false, K, true, H, false, false, true)));
+  } else if (!P.ties && !count && learned_pass == 0) {
+    // the plain form on input without large groups of identical points
+    if (carried)
+      EMST_IF(h, H, EMST_IF(lbt, L, EMST_IF(kept, T, EMST_LAUNCH(true, false, false, true, H, false, false, false, false, L, T))));
+    else if (first)  // labels are the curve indices
+      EMST_IF(h, H, EMST_LAUNCH(false, false, false, true, H, false, true, false, false));
+    else
+      EMST_IF(h, H, EMST_LAUNCH(false, false, false, true, H, false, false, false, false));
   } else if (carried) {
-    if (!lbt && P.leaf == 1) {
-      if (count) EMST_TRAV_NOLB(true); else EMST_TRAV_NOLB(false);
-    } else {
-      if (count) EMST_TRAV(true, false, true, true, false); else EMST_TRAV(true, false, false, true, false);
-    }
-  } else if (first) {  // the first round of the plain form: labels are the curve indices
-    if (P.leaf > 1) {
-      if (count) EMST_TRAV_FIRST(true, true); else EMST_TRAV_FIRST(false, true);
-    } else {
-      if (count) EMST_TRAV_FIRST(true, false); else EMST_TRAV_FIRST(false, false);
-    }
+    EMST_IF(h, H, EMST_IF(count, K, EMST_IF(lbt, L, EMST_IF(kept, T, EMST_LAUNCH(true, false, K, true, H, false, false, false, true, L, T)))));
+  } else if (first) {
+    EMST_IF(h, H, EMST_IF(count, K, EMST_LAUNCH(false, false, K, true, H, false, true, false)));
   } else {
-    if (count) EMST_TRAV(false, false, true, true, false); else EMST_TRAV(false, false, false, true, false);
+    EMST_IF(h, H, EMST_IF(count, K, EMST_LAUNCH(false, false, K, true, H, false, false, false)));
   }
-#undef EMST_TRAV
-#undef EMST_TRAV2
-#undef EMST_TRAV_FIRST
-#undef EMST_TRAV_MRD
-#undef EMST_TRAV_NOTIES
+#undef EMST_LAUNCH
+#undef EMST_IF
   P.launches += 1;
 }
 

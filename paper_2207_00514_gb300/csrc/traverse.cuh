@@ -354,6 +354,29 @@ __device__ __forceinline__ void offer_best(CompBest *c, uint32_t w_bits, uint32_
   atomicOr(status, kErrCas);
 }
 
+// A result (w, j) of an earlier round is the nearest point of another component
+// by (w, original id) at that time.  Components only grow, so the points of
+// other components are a subset of what they were then: while j is still one
+// of them, (w, j) is still their smallest and the query needs no search.  (From
+// the third round on most points that pass the skip test hold such a
+// neighbour: their component took another point's edge.)
+__device__ __forceinline__ bool keep_neighbour(const uint32_t *__restrict__ labels, const uint2 &res,
+                                               uint32_t me) {
+  return res.y != kInvalid && labels[res.y] != me;
+}
+
+// The kept edge's offer: its ids are loaded only if its weight can improve on
+// the component's minimum.
+__device__ __forceinline__ void offer_kept(CompBest *c, const float4 *__restrict__ pts,
+                                           uint32_t w_bits, int64_t i, uint32_t j,
+                                           const uint32_t *__restrict__ labels, uint32_t *status) {
+  const uint32_t cur =
+      (uint32_t)(__ldcg(reinterpret_cast<const unsigned long long *>(&c->key)) >> 32);
+  if (w_bits > cur) return;
+  offer_best(c, w_bits, __float_as_uint(__ldg(&pts[i].w)), __float_as_uint(__ldg(&pts[j].w)), labels, j,
+             status);
+}
+
 struct TravArgs {
   const float4 *pts;
   const NodeRec *nodes;
@@ -378,6 +401,8 @@ struct TravArgs {
   float *r_used;        // LEARNED: cutoff each query was exact within (+inf: skipped)
   uint32_t *queue;      // a listed launch: warps take 32 list entries at a time, in list
                         // order, from this counter (null: a grid-stride walk of the list)
+  uint4 *near_j;        // near lists (rounds.cu): curve indices and weights, or null
+  float4 *near_w;
 };
 
 // The first half of a query: its cutoff, and whether it needs a search at all.
@@ -473,11 +498,16 @@ __device__ __forceinline__ void finish_query(const TravArgs &A, int64_t i, Query
 }
 
 // One query, start to finish (the one-thread-per-point form): the same
-// steps as start_query + explore + finish_query, kept in one piece so the
-// point's record stays in registers through the search.
+// steps as start_query + explore + finish_query in one piece.  The kernel is
+// held to 32 registers, so nothing stays live through the search that can be
+// read again after it.
+// KEPT: a neighbour of an earlier round may still stand (keep_neighbour) and
+// settles the query; otherwise the caller has ruled that out (the listing
+// kernels settle those, and after the first round every neighbour has merged)
+// and the earlier result is only a lower bound.
 template <bool CARRIED, bool RADIUS_IN, bool COUNT, bool SEEDED, bool CHUNKS, bool LEARNED,
-          bool FIRST = false, bool MRD = false, bool TIES = true, bool LBT = true>
-__device__ __forceinline__ void traverse_one(const TravArgs &A, int64_t i) {
+          bool FIRST = false, bool MRD = false, bool TIES = true, bool LBT = true, bool KEPT = true>
+__device__ __forceinline__ void traverse_one(const TravArgs &A, uint32_t i) {
   const float kInf = __int_as_float(0x7f800000);
   const int64_t n = A.n;
   // Batched form: search only this point's instance (its subtree).
@@ -491,11 +521,7 @@ __device__ __forceinline__ void traverse_one(const TravArgs &A, int64_t i) {
       return;
     }
   }
-  const float4 p = A.pts[i];
   Query q;
-  q.px = p.x;
-  q.py = p.y;
-  q.pz = p.z;
   q.core = MRD ? __ldg(A.core2 + i) : 0.0f;
   q.me = A.labels[i];
   q.best = kInf;
@@ -504,7 +530,10 @@ __device__ __forceinline__ void traverse_one(const TravArgs &A, int64_t i) {
   if (RADIUS_IN) q.radius = A.radius_in[i];
   else q.radius = bound_to_radius(A.bound[q.me]);
   uint2 prev = make_uint2(0u, kInvalid);
-  if (CARRIED) prev = A.res[i];
+  if (CARRIED) {
+    if (KEPT) prev = A.res[i];
+    else prev.x = A.res[i].x;
+  }
   if (SEEDED) {
     // The component's best weight found so far this round: a real cross edge
     // of the component, so never below its minimum.
@@ -516,22 +545,33 @@ __device__ __forceinline__ void traverse_one(const TravArgs &A, int64_t i) {
     // component-level cutoff, this point cannot be an endpoint of the
     // component's minimum edge: skip the query.
     if (CARRIED && __uint_as_float(prev.x) > q.radius) {
-      // (the entry already reads so when it holds no neighbour: no write)
-      if (prev.y != kInvalid) A.res[i] = make_uint2(prev.x, kInvalid);
+      // (the entry stays: its neighbour may still serve a later round)
       if (LEARNED) A.r_used[i] = kInf;
       return;
     }
   }
-  // The previous round's neighbour, if still in another component, is a real
-  // cross edge of this point: a per-point cutoff.
-  if (CARRIED && prev.y != kInvalid && A.labels[prev.y] != q.me)
+  // The neighbour of an earlier round, if still in another component, is a
+  // real cross edge of this point: the plain form is done with it (see
+  // keep_neighbour), the learned form takes it as a per-point cutoff.
+  if (CARRIED && KEPT && keep_neighbour(A.labels, prev, q.me)) {
+    if (SEEDED && !LEARNED) {
+      offer_kept(A.comp + q.me, A.pts, prev.x, i, prev.y, A.labels, A.status);
+      return;
+    }
     q.radius = fminf(q.radius, __uint_as_float(prev.x));
+  }
   if (LEARNED) q.radius = fminf(q.radius, __ldg(A.pred_r + i));
   const float r0 = q.radius;  // the search is exact within this cutoff
   if (LEARNED) A.r_used[i] = r0;
   if (MRD && q.core > r0) {  // every weight from this point is at least its core distance
     A.res[i] = make_uint2(__float_as_uint(q.core), kInvalid);
     return;
+  }
+  {
+    const float4 p = A.pts[i];
+    q.px = p.x;
+    q.py = p.y;
+    q.pz = p.z;
   }
   uint32_t st_node[kStackDepth];
   float st_dist[kStackDepth];
@@ -559,23 +599,14 @@ __device__ __forceinline__ void traverse_one(const TravArgs &A, int64_t i) {
       atomicAdd(A.queries, (unsigned long long)__popc(mask));
     }
   }
-  if (SEEDED) {
-    // Report only the exact nearest neighbour within r0 (a seed beyond r0 is
-    // dropped); keep in res.x a lower bound for the next round: the found
-    // weight, or r0 when nothing lies within it.
-    const bool found = q.bj != kInvalid && q.best <= r0;
-    if (!found) q.bj = kInvalid;
-    float lb = found ? q.best : (r0 < kInf ? r0 : 0.0f);
-    // (LB, nothing found: q.best is that bound, above r0, or +inf when the
-    // search met no other component at all; r0 is kept then)
-    if (LB && !found && r0 < kInf && q.best < kInf) lb = q.best;
-    A.res[i] = make_uint2(__float_as_uint(lb), q.bj);
-  } else {
-    A.res[i] = make_uint2(__float_as_uint(q.best), q.bj);
-  }
+  // res.x is a lower bound for the next round: the found weight (never above
+  // r0), else the bound LB tracked (+inf when the search met no other
+  // component at all: there is none within this point's instance), else r0.
+  if (SEEDED && !LB && q.bj == kInvalid) q.best = r0 < kInf ? r0 : 0.0f;
+  A.res[i] = make_uint2(__float_as_uint(q.best), q.bj);
   if (q.bj != kInvalid) {
-    const uint32_t oi = __float_as_uint(p.w);
-    const uint32_t oj = q.bid != kInvalid ? q.bid : __float_as_uint(A.pts[q.bj].w);
+    const uint32_t oi = __float_as_uint(__ldg(&A.pts[i].w));
+    const uint32_t oj = q.bid != kInvalid ? q.bid : __float_as_uint(__ldg(&A.pts[q.bj].w));
     offer_best(A.comp + q.me, __float_as_uint(q.best), oi, oj, A.labels, q.bj, A.status);
   }
 }
