@@ -99,6 +99,61 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
+// The calling thread's mailbox: a page of mapped host memory into which a
+// call's kernels post the counters the host needs between rounds (post_mail in
+// rounds.cu), so that a round costs the host a wait on one word instead of a
+// copy and a stream synchronisation (about 10 us per round, which at a
+// million points is a tenth of the call).  One per host thread, freed with it;
+// a call uses it only while it runs, and its sequence numbers never repeat.
+namespace {
+struct Mailbox {
+  uint32_t *words = nullptr;  // kMailWords, then the sequence number of the last post
+  uint32_t seq = 0;
+  bool open() {
+    if (!words && cudaHostAlloc((void **)&words, 4096, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      words = nullptr;
+    }
+    if (words && seq == 0) std::memset(words, 0, 4096);
+    return words != nullptr;
+  }
+  ~Mailbox() {
+    if (words) cudaFreeHost(words);
+  }
+};
+thread_local Mailbox t_mailbox;
+
+// Waits for the post `P.mail_seq` and copies it; false when the stream ends
+// (or fails) without it.
+bool wait_mail(Problem &P, uint32_t *out) {
+  const uint32_t *flag = t_mailbox.words + kMailWords;
+  auto arrived = [&]() { return __atomic_load_n(flag, __ATOMIC_ACQUIRE) == P.mail_seq; };
+  for (;;) {
+    for (int k = 0; k < 4096; ++k)
+      if (arrived()) {
+        std::memcpy(out, t_mailbox.words, sizeof(uint32_t) * kMailWords);
+        return true;
+      }
+    const cudaError_t q = cudaStreamQuery(P.stream);
+    if (q == cudaErrorNotReady) continue;
+    if (q == cudaSuccess && arrived()) continue;
+    return false;
+  }
+}
+}  // namespace
+
+// The counters as the work on the stream so far leaves them (kMailWords).
+bool read_counters(Problem &P, uint32_t *out) {
+  if (P.mail) {
+    P.mail_seq = ++t_mailbox.seq;
+    launch_post_mail(P);
+    return cudaPeekAtLastError() == cudaSuccess && wait_mail(P, out);
+  }
+  return cudaMemcpyAsync(out, P.counters, sizeof(uint32_t) * kMailWords, cudaMemcpyDeviceToHost, P.stream) ==
+             cudaSuccess &&
+         cudaStreamSynchronize(P.stream) == cudaSuccess;
+}
+
 struct Carver {
   char *base;
   size_t off = 0;
@@ -129,9 +184,7 @@ size_t layout(Problem &P, char *base, bool copy_points, bool copy_edges) {
   const int64_t nc = P.nc;
   Carver c(base);
   P.counters = c.take<uint32_t>(64);
-  P.sort_hist = c.take<uint32_t>(8 * 256);
-  P.sort_tiles = sort_tiles_for(n);
-  P.sort_lookback = c.take<uint32_t>(256 * P.sort_tiles);
+  P.sort_state = c.take<uint32_t>(sort_state_words(n));
   P.pts = c.take<float4>(n);
   P.keys[0] = c.take<uint64_t>(n);
   P.keys[1] = c.take<uint64_t>(n);
@@ -250,35 +303,40 @@ static void build_order128(Problem &P) {
 
 // A1-A4: scene box, codes, sort, gather, hierarchy, refit.  With auto_wide
 // the 64-bit order is built first and its collisions counted (one host
-// read); when more than n/64 distinct points share their predecessor's code,
-// the order is rebuilt with 128-bit codes (§4.1's remedy for data the 64-bit
-// grid under-resolves).
-void run_build(Problem &P) {
+// read, which also says whether the input is finite and has large groups of
+// equal codes); when more than n/64 distinct points share their
+// predecessor's code, the order is rebuilt with 128-bit codes (§4.1's remedy
+// for data the 64-bit grid under-resolves).  True: `counters` holds the
+// build's counters (the caller need not read them).
+bool run_build(Problem &P, uint32_t *counters) {
   launch_scene_box(P);
   if (P.num_inst > 1) launch_instance_ids(P);
+  bool known = false;
   if (P.wide) {
     build_order128(P);
   } else {
     build_order64(P);
-    if (P.auto_wide) {
-      unsigned long long c = 0;
-      uint32_t status = 0;
-      cudaMemcpyAsync(&c, P.counters + 30, sizeof(c), cudaMemcpyDeviceToHost, P.stream);
-      cudaMemcpyAsync(&status, P.counters + 1, sizeof(status), cudaMemcpyDeviceToHost, P.stream);
-      if (cudaStreamSynchronize(P.stream) == cudaSuccess) {
-        P.code_collisions = (int64_t)c;
-        if (status == 0 && (int64_t)c * 64 > P.n) {
-          P.wide = true;
-          build_order128(P);
-        }
+    if (P.auto_wide && read_counters(P, counters)) {
+      P.code_collisions = (int64_t)counters[30] | ((int64_t)counters[31] << 32);
+      known = true;
+      if (counters[1] != 0) return known;
+      if (P.code_collisions * 64 > P.n) {
+        P.wide = true;
+        build_order128(P);
+        known = false;
       }
     }
   }
   if (P.n >= 2) {
-    cudaMemsetAsync(P.arrivals, 0, sizeof(uint64_t) * (size_t)(P.nc - 1), P.stream);
     launch_build_tree(P);
     if (P.num_inst > 1) launch_instance_roots(P);
   }
+  return known;
+}
+
+void run_build(Problem &P) {
+  uint32_t counters[kMailWords];
+  run_build(P, counters);
 }
 
 // One Boruvka round (the loop body of Fig. 3).  Round 0 takes its node labels
@@ -438,10 +496,10 @@ void reset_round_state(Problem &P) {
 
 // A12: the n-1 edges in (w, i, j) order into `out` (device).  w_bits: the
 // largest emitted weight's bits (counters[11]): the sort key needs
-// L + significant bits of it.
-int run_output(Problem &P, emst_edge *out, uint32_t w_bits) {
+// L + significant bits of it.  Leaves the call's final counters in `counters`.
+int run_output(Problem &P, emst_edge *out, uint32_t w_bits, uint32_t *counters) {
   const int64_t m = P.num_inst > 1 ? P.edges_expected : P.n - 1;
-  if (m <= 0) return EMST_OK;
+  if (m <= 0) return EMST_OK;  // (not called without edges)
   const int L = bits_for(P.n - 1);
   const int wb = w_bits ? 32 - __builtin_clz(w_bits) : 0;
   // fast path: one sort of a 64-bit key, then the runs of equal keys (the
@@ -450,9 +508,9 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits) {
   const int Lloc = P.num_inst > 1 ? bits_for(P.largest > 1 ? P.largest - 1 : 1) : L;
   const bool fast = P.num_inst == 1 || P.inst_bits + wb + Lloc <= 64;
   auto long_run_count = [&](uint32_t &c) {
-    return cudaMemcpyAsync(&c, P.counters + 10, sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                           P.stream) == cudaSuccess &&
-           cudaStreamSynchronize(P.stream) == cudaSuccess;
+    if (!read_counters(P, counters)) return false;
+    c = counters[10];
+    return true;
   };
   // fastest path (one instance, no group of identical points): the same key
   // sorted on w's bits only, stable, then every run of equal w (a handful of
@@ -461,14 +519,13 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits) {
   if (P.num_inst == 1 && !P.ties && wb > 0) {
     launch_edge_keys_wi(P, m, L);
     const int s = radix_sort_pairs(P, m, 0, (wb + 7) / 8, 0, L);
-    cudaMemsetAsync(P.counters + 10, 0, sizeof(uint32_t), P.stream);
+    // (the count of long runs is zero since the call's first kernel; the
+    // edges are written without waiting for it, and again below if need be)
     launch_edge_ties_w(P, m, s, L);
+    launch_edge_from_keys(P, m, s, Lloc, wb, out);
     uint32_t long_runs = 0;
     if (!long_run_count(long_runs)) return EMST_ERR_CUDA;
-    if (long_runs == 0) {
-      launch_edge_from_keys(P, m, s, Lloc, wb, out);
-      return EMST_OK;
-    }
+    if (long_runs == 0) return EMST_OK;
   }
   if (fast) {
     int digits;
@@ -482,15 +539,10 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits) {
     const int s = radix_sort_pairs(P, m, 0, digits, 0);
     cudaMemsetAsync(P.counters + 10, 0, sizeof(uint32_t), P.stream);
     launch_edge_ties(P, m, s);
+    launch_edge_from_keys(P, m, s, Lloc, wb, out);
     uint32_t long_runs = 0;
-    if (cudaMemcpyAsync(&long_runs, P.counters + 10, sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                        P.stream) != cudaSuccess ||
-        cudaStreamSynchronize(P.stream) != cudaSuccess)
-      return EMST_ERR_CUDA;
-    if (long_runs == 0) {
-      launch_edge_from_keys(P, m, s, Lloc, wb, out);
-      return EMST_OK;
-    }
+    if (!long_run_count(long_runs)) return EMST_ERR_CUDA;
+    if (long_runs == 0) return EMST_OK;
   }
   // full path: stable by j, then by (w, i), then (batched) by instance
   launch_edge_keys_j(P, m);
@@ -502,7 +554,7 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits) {
     s = radix_sort_pairs(P, m, 0, (P.inst_bits + 7) / 8, s);
   }
   launch_edge_gather(P, m, P.vals[s], out);
-  return EMST_OK;
+  return read_counters(P, counters) ? EMST_OK : EMST_ERR_CUDA;
 }
 
 namespace {
@@ -670,7 +722,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
   int64_t reruns = 0;
   const size_t need = layout(P, nullptr, !pts_dev, !out_dev && !out_map);
   char *base = nullptr;
-  uint32_t host_counters[48] = {0};
+  uint32_t host_counters[kMailWords] = {0};
   uint64_t prev_visits = 0, prev_queries = 0, prev_distinct = 0;
   Timer tm;
   int rounds = 0;
@@ -683,8 +735,8 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     return EMST_ERR_OOM;
   }
   layout(P, base, !pts_dev, !out_dev && !out_map);
+  if (t_mailbox.open()) P.mail = t_mailbox.words;  // (one address for host and device)
   if (stats) tm.start(stream);
-  CU(cudaMemsetAsync(P.counters, 0, sizeof(uint32_t) * 64, stream));
   if (pts_map) P.points_mapped = pts_map;  // copied by the scene-box pass
   else if (!pts_dev)
     CU(cudaMemcpyAsync((void *)P.points, points, sizeof(float) * (size_t)n * dim,
@@ -697,12 +749,12 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
                        cudaMemcpyDefault, stream));
   if (logging) CU(cudaMemsetAsync(P.log_count, 0, sizeof(unsigned long long), stream));
   if (P.seen) CU(cudaMemsetAsync(P.seen, 0, sizeof(uint32_t) * (size_t)((P.nc - 1 + 31) / 32), stream));
-  run_build(P);
-  tm.mark(1, stream);
-  // Non-finite input is reported before any round runs.
-  CU(cudaMemcpyAsync(host_counters, P.counters, sizeof(host_counters), cudaMemcpyDeviceToHost,
-                     stream));
-  CU(cudaStreamSynchronize(stream));
+  {
+    const bool known = run_build(P, host_counters);
+    tm.mark(1, stream);
+    // Non-finite input is reported before any round runs.
+    if (!known && !read_counters(P, host_counters)) { rc = EMST_ERR_CUDA; goto done; }
+  }
   if (host_counters[1] != 0) { rc = status_from_bits(host_counters[1]); goto done; }
   // a large group of identical points can exist: the search needs its tie rule
   P.ties = host_counters[32] != 0;
@@ -758,11 +810,13 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
         n_tev = rounds + 1;
       }
       if (count) launch_count_seen(P);
+      if (P.mail) P.mail_seq = ++t_mailbox.seq;  // posted by the merge's last kernel
       launch_merge(P);
       CU(cudaPeekAtLastError());  // a launch that failed must not read as a round without edges
-      CU(cudaMemcpyAsync(host_counters, P.counters, sizeof(host_counters), cudaMemcpyDeviceToHost,
-                         stream));
-      CU(cudaStreamSynchronize(stream));
+      if (P.mail ? !wait_mail(P, host_counters) : !read_counters(P, host_counters)) {
+        rc = EMST_ERR_CUDA;
+        goto done;
+      }
       if (host_counters[1] != 0) { rc = status_from_bits(host_counters[1]); goto done; }
       if (learned) reruns += host_counters[13];
       if (count && stats && rounds < 40) {
@@ -778,6 +832,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
       if ((int64_t)host_counters[0] >= expected) { ++rounds; break; }
       if (rounds == 0 && use_graph == 1 && !learned && !logging && !count) {
         // the remaining rounds as one graph ended on the device
+        P.mail = nullptr;
         int kernels = 0;
         const int before = P.launches;
         CU(run_rounds_graph(P, expected, limit, carried != 0, block, 1, &kernels));
@@ -794,7 +849,8 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     tm.mark(2, stream);
     if ((int64_t)host_counters[0] != expected) { rc = EMST_ERR_INTERNAL; goto done; }
     if (!skip_output) {
-      rc = run_output(P, out_dev ? out : (out_map ? out_map : P.out_stage), host_counters[11]);
+      rc = run_output(P, out_dev ? out : (out_map ? out_map : P.out_stage), host_counters[11],
+                      host_counters);
       if (rc != EMST_OK) goto done;
     }
     if (!out_dev && !out_map && !skip_output)
@@ -804,8 +860,6 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     tm.mark(2, stream);
   }
   tm.mark(3, stream);
-  CU(cudaMemcpyAsync(host_counters, P.counters, sizeof(host_counters), cudaMemcpyDeviceToHost,
-                     stream));
   CU(cudaStreamSynchronize(stream));
   CU(cudaGetLastError());
   rc = status_from_bits(host_counters[1]);
@@ -815,6 +869,8 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     *ex->log_count_out = (int64_t)c;
   }
 done:
+  // (a call that fails half way leaves no kernel behind that could still post)
+  if (rc != EMST_OK && P.mail) cudaStreamSynchronize(stream);
   cudaFreeAsync(base, stream);
   if (rc == EMST_ERR_CUDA) cudaGetLastError();
   if (stats) {

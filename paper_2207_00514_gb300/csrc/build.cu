@@ -130,15 +130,15 @@ __global__ void __launch_bounds__(kBlock) k_scene_box_copy4(const float4 *__rest
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, kErrNonFinite);
 }
 
-__global__ void k_box_init(uint32_t *box) {
-  int t = threadIdx.x;
-  if (t < 3) box[t] = 0xFFFFFFFFu;
-  else if (t < 6) box[t] = 0u;
+// All counters to zero, the scene box (4..9) empty: the call's first kernel.
+__global__ void k_counters_init(uint32_t *counters) {
+  const int t = threadIdx.x;
+  counters[t] = t >= 4 && t < 7 ? 0xFFFFFFFFu : 0u;
 }
 
 void launch_scene_box(Problem &P) {
   uint32_t *box = P.counters + 4;
-  k_box_init<<<1, 32, 0, P.stream>>>(box);
+  k_counters_init<<<1, 64, 0, P.stream>>>(P.counters);
   int grid = sm_count() * 4;
   int64_t need = (P.n + kBlock - 1) / kBlock;
   if (need < grid) grid = (int)(need < 1 ? 1 : need);
@@ -354,9 +354,11 @@ __global__ void __launch_bounds__(kBlock) k_gather(const float *__restrict__ pts
                                                    uint32_t *__restrict__ inst_of,
                                                    const uint64_t *__restrict__ sorted_codes,
                                                    const uint64_t *__restrict__ code_hi,
-                                                   unsigned long long *dup) {
+                                                   unsigned long long *dup,
+                                                   uint64_t *__restrict__ arrivals, int64_t splits) {
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
+  if (k < splits) arrivals[k] = 0u;  // for the hierarchy
   uint32_t o = __ldg(perm + k);
   if (inst_of) inst_of[k] = __ldg(inst_in + o);
   const float *p = pts + (int64_t)o * DIM;
@@ -386,13 +388,14 @@ __global__ void __launch_bounds__(kBlock) k_gather(const float *__restrict__ pts
 void launch_gather(Problem &P, const uint32_t *perm) {
   int g = grid_for(P.n, kBlock);
   unsigned long long *dup = reinterpret_cast<unsigned long long *>(P.counters + 28);
-  cudaMemsetAsync(dup, 0, 3 * sizeof(unsigned long long), P.stream);
+  // (zero since the call's first kernel, unless the order is rebuilt)
+  if (P.wide) cudaMemsetAsync(dup, 0, 3 * sizeof(unsigned long long), P.stream);
   if (P.dim == 3)
     k_gather<3><<<g, kBlock, 0, P.stream>>>(P.points, perm, P.n, P.pts, P.labels, P.inst_in,
-                                            P.inst_of, P.keys[0], P.code_hi, dup);
+                                            P.inst_of, P.keys[0], P.code_hi, dup, P.arrivals, P.nc - 1);
   else
     k_gather<2><<<g, kBlock, 0, P.stream>>>(P.points, perm, P.n, P.pts, P.labels, P.inst_in,
-                                            P.inst_of, P.keys[0], P.code_hi, dup);
+                                            P.inst_of, P.keys[0], P.code_hi, dup, P.arrivals, P.nc - 1);
   P.launches += 1;
 }
 
@@ -718,7 +721,6 @@ void launch_build_tree(Problem &P) {
   uint4 *ready = reinterpret_cast<uint4 *>(P.list_buf[1]);
   const uint32_t capacity = (uint32_t)(P.n / 4);
   uint32_t *ready_count = P.counters + kRefitReadyCounter;
-  cudaMemsetAsync(ready_count, 0, sizeof(uint32_t), P.stream);
   const int64_t ctas = grid_for(P.nc, kRefitBlock);
   k_build_local<<<(unsigned)ctas, kRefitBlock, 0, P.stream>>>(
       P.keys[0] /*sorted*/, P.code_hi, P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels, P.range,

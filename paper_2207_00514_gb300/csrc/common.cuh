@@ -299,11 +299,13 @@ struct Problem {
                                      // searched (u64), [36..37] the work queue of the
                                      // persistent traversal (u64), [38..39] distinct internal
                                      // nodes visited (u64), [40] this round's active
-                                     // components and [41] rounds done (graph rounds)
+                                     // components, [41] rounds done (graph rounds)
   uint32_t *count_dev = nullptr;     // graph rounds: counters + 40 (else nullptr)
-  uint32_t *sort_hist = nullptr;     // 8 x 256
-  uint32_t *sort_lookback = nullptr; // tiles x 256
-  int64_t sort_tiles = 0;
+  // The host's mailbox (device address of mapped host memory), or null: a
+  // round's last kernel posts the counters there, then mail_seq.
+  uint32_t *mail = nullptr;
+  uint32_t mail_seq = 0;
+  uint32_t *sort_state = nullptr;    // sort_state_words(n): the radix sort's counters and look-back
   int launches = 0;
 };
 
@@ -321,7 +323,7 @@ void launch_gather(Problem &P, const uint32_t *perm);
 void launch_instance_ids(Problem &P);
 void launch_instance_roots(Problem &P);
 // A4: hierarchy, boxes, records, ranges and round-0 child labels in one
-// bottom-up pass (P.arrivals zeroed first)
+// bottom-up pass (P.arrivals zeroed by launch_gather)
 void launch_build_tree(Problem &P);
 // sort.cu
 // Tile shape of one sort pass (compile-time knobs; the defaults are the measured best).
@@ -338,6 +340,7 @@ constexpr int kSortThreads = EMST_SORT_THREADS;
 constexpr int kSortItems = EMST_SORT_ITEMS;
 constexpr int kSortTile = kSortThreads * kSortItems;
 int64_t sort_tiles_for(int64_t n);
+int64_t sort_state_words(int64_t n);
 // Stable LSD radix sort of (keys, vals) pairs on digits [digit_begin, digit_end)
 // (8-bit digits).  Returns the index (0/1) of the buffers holding the result.
 // Stable sort of (keys[src], vals[src]) by the bits [bit0 + 8 digit_begin,
@@ -367,6 +370,9 @@ void launch_core_to_input(Problem &P, float *out);
 void launch_traverse(Problem &P, bool carried, const float *radius_in, int block, bool count,
                      bool seeded, int learned_pass = 0, bool first = false, int round = -1);
 void launch_merge(Problem &P);
+// posts the counters to the host's mailbox (P.mail, P.mail_seq)
+constexpr int kMailWords = 48;
+void launch_post_mail(Problem &P);
 void launch_fill_u32(Problem &P, uint32_t *p, uint32_t v, int64_t count);
 // count runs: adds the bits of the visited-node bitmap to counters[38..39]
 // and clears it for the next round
@@ -417,12 +423,13 @@ int status_from_bits(uint32_t bits);
 int check_args(const float *points, int64_t n, int dim);
 int bits_for(int64_t v);
 void run_build(Problem &P);
+bool read_counters(Problem &P, uint32_t *out);
 void reset_round_state(Problem &P);
 void run_round(Problem &P, int round, bool carried, int block, bool count);
 // Leaf chunk size actually used for n points and a requested size (0 =
 // default): a power of two, at most the request, leaving at least 2 chunks.
 int effective_leaf(int64_t n, int requested);
-int run_output(Problem &P, emst_edge *out, uint32_t w_bits);
+int run_output(Problem &P, emst_edge *out, uint32_t w_bits, uint32_t *counters);
 
 inline int grid_for(int64_t n, int block) {
   int64_t g = (n + block - 1) / block;

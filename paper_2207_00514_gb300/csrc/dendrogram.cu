@@ -519,7 +519,7 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     off += bytes > 0 ? bytes : 1;
     return at;
   };
-  const int64_t sort_tiles = sort_tiles_for(m), tiles = (m + kScanTile - 1) / kScanTile;
+  const int64_t tiles = (m + kScanTile - 1) / kScanTile;
   // counters, per-level counters and totals first: cleared together
   const size_t o_counters = take(256), o_levels = take(4 * kMaxLevels * sizeof(uint32_t));
   const size_t o_total = take(4 * (size_t)n), clear = off;
@@ -528,7 +528,7 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
   const size_t o_done = take(16 * (size_t)m);
   const size_t o_k0 = take(8 * (size_t)m), o_k1 = take(8 * (size_t)m);
   const size_t o_v0 = take(4 * (size_t)m), o_v1 = take(4 * (size_t)m);
-  const size_t o_hist = take(4 * 8 * 256), o_look = take(4 * 256 * (size_t)sort_tiles);
+  const size_t o_sort = take(4 * (size_t)sort_state_words(m));
   const size_t o_child = take(out_link ? 8 * (size_t)m : 0);
   const size_t o_tiles = take(8 * (size_t)tiles);
   const size_t o_edges = edges_dev ? 0 : take(sizeof(emst_edge) * (size_t)m);
@@ -590,8 +590,7 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     P.keys[1] = reinterpret_cast<uint64_t *>(base + o_k1);
     P.vals[0] = A.vals;
     P.vals[1] = U(o_v1);
-    P.sort_hist = U(o_hist);
-    P.sort_lookback = U(o_look);
+    P.sort_state = U(o_sort);
     // by chain; the edges of one chain stay in rank order (a stable sort)
     const int src = radix_sort_pairs(P, m, 0, (bits_for(n - 1) + 7) / 8, 0, 32);
     uint2 *tile = reinterpret_cast<uint2 *>(base + o_tiles);

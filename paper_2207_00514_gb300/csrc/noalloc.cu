@@ -85,7 +85,7 @@ extern "C" int emst_compute_noalloc(const float *points, int64_t n, int dim, ems
   if (layout(P, nullptr, !pts_dev, !out_dev) > kNoallocScratchBytes) return EMST_ERR_TOO_LARGE;
   layout(P, base, !pts_dev, !out_dev);
 
-  uint32_t host_counters[16] = {0};
+  uint32_t host_counters[kMailWords] = {0};
   // Launch errors first: a failed launch must not read as a round without edges.
   auto sync_counters = [&]() -> bool {
     if (cudaPeekAtLastError() != cudaSuccess) return false;
@@ -115,7 +115,8 @@ extern "C" int emst_compute_noalloc(const float *points, int64_t n, int dim, ems
       if ((int64_t)host_counters[0] >= n - 1) break;
     }
     if ((int64_t)host_counters[0] != n - 1) return EMST_ERR_INTERNAL;
-    const int orc = run_output(P, out_dev ? out_edges : P.out_stage, host_counters[11]);
+    const int orc = run_output(P, out_dev ? out_edges : P.out_stage, host_counters[11],
+                               host_counters);
     if (orc == EMST_ERR_CUDA) return cuda_failure();
     if (orc != EMST_OK) return orc;
     if (!out_dev && cudaMemcpyAsync(out_edges, P.out_stage, sizeof(emst_edge) * (size_t)(n - 1),

@@ -9,10 +9,31 @@
 namespace emst {
 
 constexpr int kBlock = 256;
-// P.counters slots of a round
+// P.counters slots of a round, cleared by its first kernel (k_node_labels) or
+// by the last CTA that counts in them: no memset between the kernels.
 constexpr uint32_t kActiveCounter = 50;  // listed queries
 constexpr uint32_t kActiveQueue = 51;    // list entries handed out
 constexpr uint32_t kActiveDone = 52;     // tiles of k_active_count finished
+
+// The counters to the caller's mailbox (mapped host memory): the words, then
+// the sequence number the host waits for.  Called by a whole CTA.
+__device__ void post_mail(const uint32_t *counters, uint32_t *mail, uint32_t seq) {
+  if (threadIdx.x < kMailWords) mail[threadIdx.x] = __ldcg(counters + threadIdx.x);
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(mail + kMailWords), "r"(seq) : "memory");
+  }
+}
+
+__global__ void k_post_mail(const uint32_t *counters, uint32_t *mail, uint32_t seq) {
+  post_mail(counters, mail, seq);
+}
+
+void launch_post_mail(Problem &P) {
+  k_post_mail<<<1, 64, 0, P.stream>>>(P.counters, P.mail, P.mail_seq);
+  P.launches += 1;
+}
 
 // The weight of curve neighbours k and k + 1 (core2: the mutual reachability
 // weight, §4.5).
@@ -122,7 +143,8 @@ __global__ void __launch_bounds__(kScanThreads, EMST_SCAN_MIN_BLOCKS) k_runs(
     const float4 *__restrict__ pts, const uint32_t *__restrict__ inst_of,
     const float *__restrict__ core2, int64_t n,
     uint32_t *__restrict__ labels_new, uint32_t *__restrict__ bound_next,
-    uint2 *__restrict__ words, uint32_t *tile_total, uint32_t *tile_prefix, uint32_t *done) {
+    uint2 *__restrict__ words, uint32_t *tile_total, uint32_t *tile_prefix, uint32_t *done,
+    const uint32_t *counters, uint32_t *mail, uint32_t mail_seq) {
   __shared__ uint32_t s_warp[kScanThreads / 32];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -198,6 +220,10 @@ __global__ void __launch_bounds__(kScanThreads, EMST_SCAN_MIN_BLOCKS) k_runs(
   __syncthreads();
   if (s_last) {
     __threadfence();
+    if (tid == 0) *done = 0u;  // for the next round
+    // the round's results to the host before the scan, which only the next
+    // round needs: it launches that round meanwhile
+    if (mail) post_mail(counters, mail, mail_seq);
     block_exclusive_scan(tile_total, tile_prefix, gridDim.x);
   }
 }
@@ -207,15 +233,14 @@ static void launch_runs(Problem &P, bool relabel) {
   uint32_t *done = P.counters + 24;
   uint32_t *tile_total = P.scan_tiles, *tile_prefix = P.scan_tiles + tiles;
   uint2 *words = reinterpret_cast<uint2 *>(P.runs);
-  cudaMemsetAsync(done, 0, sizeof(uint32_t), P.stream);
   if (relabel)
     k_runs<true><<<(unsigned)tiles, kScanThreads, 0, P.stream>>>(
         P.labels, P.root, P.pts, P.inst_of, P.core2, P.n, P.labels_buf[P.cur ^ 1],
-        P.bound_buf[P.cur ^ 1], words, tile_total, tile_prefix, done);
+        P.bound_buf[P.cur ^ 1], words, tile_total, tile_prefix, done, P.counters, P.mail, P.mail_seq);
   else
     k_runs<false><<<(unsigned)tiles, kScanThreads, 0, P.stream>>>(
         P.labels, nullptr, P.pts, P.inst_of, nullptr, P.n, nullptr, nullptr, words, tile_total,
-        tile_prefix, done);
+        tile_prefix, done, nullptr, nullptr, 0u);
   P.launches += 1;
 }
 
@@ -226,8 +251,15 @@ __global__ void __launch_bounds__(kBlock) k_node_labels(const uint32_t *__restri
                                                         const uint32_t *__restrict__ tile_prefix,
                                                         const uint2 *__restrict__ range,
                                                         int64_t n, int64_t nc, int leaf,
-                                                        uint2 *__restrict__ nlabels) {
+                                                        uint2 *__restrict__ nlabels,
+                                                        uint32_t *counters) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {  // the round's counters (the first kernel of a round)
+    counters[40] = counters[12];      // components listed by the previous merge
+    counters[12] = 0u;
+    counters[kActiveCounter] = 0u;
+    counters[kActiveQueue] = 0u;
+  }
   if (i >= nc - 1) return;
   // the children split the node's chunk range [first, last] after `split`
   const NodeRange r = unpack_range((uint32_t)i, __ldg(range + i));
@@ -246,7 +278,7 @@ __global__ void __launch_bounds__(kBlock) k_node_labels(const uint32_t *__restri
 void launch_node_labels(Problem &P) {
   k_node_labels<<<grid_for(P.nc - 1, kBlock), kBlock, 0, P.stream>>>(
       P.labels, reinterpret_cast<const uint2 *>(P.runs), P.scan_tiles + scan_tiles_for(P.n), P.range,
-      P.n, P.nc, P.leaf, P.nlabels);
+      P.n, P.nc, P.leaf, P.nlabels, P.counters);
   P.launches += 1;
 }
 
@@ -840,7 +872,10 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_count(
     __threadfence();
     block_exclusive_scan(tile_total, tile_prefix, gridDim.x);
     __syncthreads();
-    if (tid == 0) *count = tile_prefix[gridDim.x - 1] + __ldcg(tile_total + gridDim.x - 1);
+    if (tid == 0) {
+      *count = tile_prefix[gridDim.x - 1] + __ldcg(tile_total + gridDim.x - 1);
+      *done = 0u;  // for the next round
+    }
   }
 }
 
@@ -961,14 +996,12 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
       settled = reinterpret_cast<uint8_t *>(words);
     }
     if (round < kOrderedUntilRound) {
-      cudaMemsetAsync(P.counters + kActiveDone, 0, sizeof(uint32_t), s);
       k_active_count<<<(unsigned)tiles, kActiveThreads, 0, s>>>(P.labels, P.bound, P.comp, P.res, settled,
                                                                P.n, flags, tile_total, tile_prefix,
                                                                P.counters + kActiveDone, active_count);
       k_active_write<<<(unsigned)tiles, kActiveThreads, 0, s>>>(flags, tile_prefix, P.n, active);
       P.launches += 2;
     } else {
-      cudaMemsetAsync(active_count, 0, sizeof(uint32_t), s);
       k_active<<<(unsigned)grid_for((P.n + 3) / 4, 256), 256, 0, s>>>(P.labels, P.bound, P.comp, P.res,
                                                                        P.n, active, active_count);
       P.launches += 1;
@@ -977,7 +1010,6 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     list_count = active_count;
     g = sm_count() * (2048 / block);  // one resident wave
     A.queue = P.counters + kActiveQueue;  // warps take the list in order
-    cudaMemsetAsync(A.queue, 0, sizeof(uint32_t), s);
   }
 #define EMST_LAUNCH(...) launch_trav(k_traverse<__VA_ARGS__>, g, block, s, A, list, list_count)
 // a host flag as a template argument
@@ -1138,12 +1170,9 @@ __global__ void __launch_bounds__(kBlock) k_merge_roots(const uint32_t *__restri
 void launch_merge(Problem &P) {
   const int64_t count = P.active_list ? P.n_active : P.n;
   const int g = grid_for(count, kBlock);
-  // graph rounds: this round's list length exists only on the device
+  // graph rounds: this round's list length exists only on the device (put
+  // there by k_node_labels)
   const uint32_t *count_dev = P.active_list ? P.count_dev : nullptr;
-  if (count_dev)
-    cudaMemcpyAsync(P.count_dev, P.counters + 12, sizeof(uint32_t), cudaMemcpyDeviceToDevice,
-                    P.stream);
-  cudaMemsetAsync(P.counters + 12, 0, sizeof(uint32_t), P.stream);
   k_merge_roots<<<g, kBlock, 0, P.stream>>>(P.active_list, count, count_dev, P.comp, P.comp_buf[P.cur ^ 1],
                                             P.bound_buf[P.cur ^ 1], P.root, P.edges, P.next_list, P.counters, P.n);
   P.launches += 1;

@@ -22,11 +22,22 @@ constexpr int kLookWindow = 8;  // preceding tiles read per look-back round trip
 
 int64_t sort_tiles_for(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 
-// Histograms of all digits in [digit_begin, digit_end) in one pass.
+// The words of P.sort_state: the digits' histograms, the passes' tile counters
+// and the histogram's count of finished CTAs, then two look-back arrays that
+// the passes use in turn (each clears the other for the next one), so one
+// memset serves a whole sort.
+constexpr int64_t kHistWords = 8 * kRadix;
+constexpr int64_t kCounterWords = 64;  // [0..7] tile counters, [8] finished CTAs
+
+int64_t sort_state_words(int64_t n) { return kHistWords + kCounterWords + 2 * kRadix * sort_tiles_for(n); }
+
+// Histograms of all digits in [digit_begin, digit_end) in one pass; the last
+// CTA to finish turns them into exclusive prefix sums.
 __global__ void __launch_bounds__(512) k_sort_hist(const uint64_t *__restrict__ keys, int64_t n,
                                                    int digit_begin, int digit_end, int bit0,
-                                                   uint32_t *__restrict__ hist) {
+                                                   uint32_t *hist, uint32_t *finished) {
   __shared__ uint32_t sh[8][kRadix];
+  __shared__ bool s_last;
   for (int t = threadIdx.x; t < 8 * kRadix; t += blockDim.x) (&sh[0][0])[t] = 0;
   __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -40,24 +51,35 @@ __global__ void __launch_bounds__(512) k_sort_hist(const uint64_t *__restrict__ 
     uint32_t v = (&sh[0][0])[t];
     if (v) atomicAdd(hist + t, v);
   }
-}
-
-// Exclusive scan of each digit's histogram (one CTA of 256 threads per digit).
-__global__ void __launch_bounds__(kRadix) k_sort_scan(uint32_t *hist) {
-  __shared__ uint32_t warp_sum[kRadix / 32];
-  uint32_t *h = hist + blockIdx.x * kRadix;
-  int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  uint32_t v = h[t];
-  uint32_t x = v;
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_sum[w] = x;
+  __threadfence();
   __syncthreads();
-  uint32_t base = 0;
-  for (int q = 0; q < w; ++q) base += warp_sum[q];
-  h[t] = base + x - v;
+  if (threadIdx.x == 0) s_last = atomicAdd(finished, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // a warp per digit, eight bins per lane
+  const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
+  if (d < 8) {
+    uint32_t *h = hist + d * kRadix + lane * 8;
+    uint32_t v[8], sum = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      v[q] = __ldcg(h + q);
+      sum += v[q];
+    }
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    uint32_t run = x - sum;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      h[q] = run;
+      run += v[q];
+    }
+  }
 }
 
 struct SortSmem {
@@ -79,8 +101,8 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
 __global__ void __launch_bounds__(kSortThreads, EMST_SORT_MIN_BLOCKS) k_sort_pass(
     const uint64_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
     uint64_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out, int64_t n, int shift,
-    const uint32_t *__restrict__ digit_offset, uint32_t *lookback, uint32_t *tile_counter,
-    uint32_t *status) {
+    const uint32_t *__restrict__ digit_offset, uint32_t *lookback, uint32_t *next_lookback,
+    uint32_t *tile_counter, uint32_t *status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SortSmem &S = *reinterpret_cast<SortSmem *>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -133,6 +155,7 @@ __global__ void __launch_bounds__(kSortThreads, EMST_SORT_MIN_BLOCKS) k_sort_pas
     S.warp_hist[w][t] = total;
     total += c;
   }
+  next_lookback[(int64_t)tile * kRadix + t] = 0u;
   // Publish this tile's count (tile 0 publishes a finished prefix at once).
   {
     volatile uint32_t *lb = lookback + (int64_t)tile * kRadix + t;
@@ -225,23 +248,23 @@ int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int 
     cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     g_sort_attr_set[dev] = true;
   }
-  uint32_t *hist = P.sort_hist;
-  uint32_t *tile_ctr = P.counters + 16;
-  cudaMemsetAsync(hist, 0, sizeof(uint32_t) * 8 * kRadix, s);
-  cudaMemsetAsync(tile_ctr, 0, sizeof(uint32_t) * 8, s);
+  const int64_t tiles = sort_tiles_for(n);
+  uint32_t *hist = P.sort_state, *counters = hist + kHistWords;
+  uint32_t *look[2] = {counters + kCounterWords, counters + kCounterWords + kRadix * tiles};
+  cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)(kHistWords + kCounterWords + kRadix * tiles), s);
   int hgrid = (int)((n + 511) / 512);
   if (hgrid > sm_count() * 4) hgrid = sm_count() * 4;
-  k_sort_hist<<<hgrid, 512, 0, s>>>(P.keys[src], n, digit_begin, digit_end, bit0, hist);
-  k_sort_scan<<<8, kRadix, 0, s>>>(hist);
-  P.launches += 2;
-  const int64_t tiles = sort_tiles_for(n);
+  k_sort_hist<<<hgrid, 512, 0, s>>>(P.keys[src], n, digit_begin, digit_end, bit0, hist, counters + 8);
+  P.launches += 1;
   for (int d = digit_begin; d < digit_end; ++d) {
-    cudaMemsetAsync(P.sort_lookback, 0, sizeof(uint32_t) * kRadix * tiles, s);
     k_sort_pass<<<(unsigned)tiles, kSortThreads, smem, s>>>(
         P.keys[src], P.vals[src], P.keys[src ^ 1], P.vals[src ^ 1], n, bit0 + 8 * d, hist + d * kRadix,
-        P.sort_lookback, tile_ctr + d, P.counters + 1);
+        look[0], look[1], counters + d, P.counters + 1);
     P.launches += 1;
     src ^= 1;
+    uint32_t *t = look[0];
+    look[0] = look[1];
+    look[1] = t;
   }
   return src;
 }
