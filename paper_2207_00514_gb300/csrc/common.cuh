@@ -326,20 +326,6 @@ void launch_instance_roots(Problem &P);
 // bottom-up pass (P.arrivals zeroed by launch_gather)
 void launch_build_tree(Problem &P);
 // sort.cu
-// Tile shape of one sort pass (compile-time knobs; the defaults are the measured best).
-#ifndef EMST_SORT_THREADS
-#define EMST_SORT_THREADS 256
-#endif
-#ifndef EMST_SORT_ITEMS
-#define EMST_SORT_ITEMS 12
-#endif
-#ifndef EMST_SORT_MIN_BLOCKS
-#define EMST_SORT_MIN_BLOCKS 3
-#endif
-constexpr int kSortThreads = EMST_SORT_THREADS;
-constexpr int kSortItems = EMST_SORT_ITEMS;
-constexpr int kSortTile = kSortThreads * kSortItems;
-int64_t sort_tiles_for(int64_t n);
 int64_t sort_state_words(int64_t n);
 // Stable LSD radix sort of (keys, vals) pairs on digits [digit_begin, digit_end)
 // (8-bit digits).  Returns the index (0/1) of the buffers holding the result.

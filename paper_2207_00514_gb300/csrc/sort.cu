@@ -12,15 +12,36 @@
 namespace emst {
 
 constexpr int kRadix = 256;
-constexpr int kWarps = kSortThreads / 32;
-static_assert(kSortThreads == kRadix, "a sort pass gives each thread one digit");
 constexpr uint32_t kFlagAggregate = 1u << 30;
 constexpr uint32_t kFlagPrefix = 2u << 30;
 constexpr uint32_t kValueMask = (1u << 30) - 1u;
 constexpr int kSpinLimit = 1 << 22;
 constexpr int kLookWindow = 8;  // preceding tiles read per look-back round trip
+// A tile is kSortThreads threads x items.  Each tile costs the others a step
+// of their look-back, so there should be no more than a few hundred until
+// larger ones no longer fit the registers; below that the GPU wants a tile
+// per SM.  A sort of 8 digits (us) with 4 / 8 / 14 items: 600,000 keys 150 /
+// 119 / 150, 1M - / 182 / 152, 2M - / 281 / 254 (core distances of 200,000
+// points, whole call, 4 / 12 items: 519 / 538); 37M keys with 8 / 12 / 14 /
+// 15 items 2,940 / 2,535 / 2,425 / 2,955 (15 spill; 18 at two CTAs per SM
+// 2,820).  Before the ballots and the scatter ahead of the look-back, with
+// 12 items: 200,000 keys 113, 1M 208, 8M 846, 37M 3,061.
+constexpr int kSortThreads = 256;
+constexpr int kSmallItems = 4, kMidItems = 8, kLargeItems = 14;
+constexpr int64_t kMaxEarlyTiles = 300;  // of the two smaller shapes
+constexpr int64_t kSmallMax = kMaxEarlyTiles * kSortThreads * kSmallItems;
+constexpr int64_t kMidMax = kMaxEarlyTiles * kSortThreads * kMidItems;
 
-int64_t sort_tiles_for(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
+// Tiles of a sort of up to n keys, whichever shape serves it.
+static int64_t sort_tiles_for(int64_t n) {
+  auto tiles = [](int64_t c, int items) { return (c + kSortThreads * items - 1) / (kSortThreads * items); };
+  if (n <= kSmallMax) return tiles(n, kSmallItems);
+  const int64_t large = tiles(n, kLargeItems);
+  return large > kMaxEarlyTiles ? large : kMaxEarlyTiles;
+}
+
+constexpr int kWarps = kSortThreads / 32;
+static_assert(kSortThreads == kRadix, "a sort pass gives each thread one digit");
 
 // The words of P.sort_state: the digits' histograms, the passes' tile counters
 // and the histogram's count of finished CTAs, then two look-back arrays that
@@ -82,11 +103,12 @@ __global__ void __launch_bounds__(512) k_sort_hist(const uint64_t *__restrict__ 
   }
 }
 
+template <int ITEMS>
 struct SortSmem {
-  uint64_t keys[kSortTile];
-  uint32_t vals[kSortTile];
+  static constexpr int kTile = kSortThreads * ITEMS;
+  uint64_t keys[kTile];
+  uint32_t vals[kTile];
   uint32_t warp_hist[kWarps][kRadix];
-  uint32_t tile_start[kRadix];   // first local position of each digit in the tile
   uint32_t global_base[kRadix];  // global position of local position 0 of each digit
   uint32_t warp_tot[kWarps];
   uint32_t tile_id;
@@ -98,76 +120,106 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-__global__ void __launch_bounds__(kSortThreads, EMST_SORT_MIN_BLOCKS) k_sort_pass(
+template <int ITEMS, int BLOCKS>
+__global__ void __launch_bounds__(kSortThreads, BLOCKS) k_sort_pass(
     const uint64_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
     uint64_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out, int64_t n, int shift,
     const uint32_t *__restrict__ digit_offset, uint32_t *lookback, uint32_t *next_lookback,
     uint32_t *tile_counter, uint32_t *status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SortSmem &S = *reinterpret_cast<SortSmem *>(smem_raw);
+  SortSmem<ITEMS> &S = *reinterpret_cast<SortSmem<ITEMS> *>(smem_raw);
+  constexpr int kTile = SortSmem<ITEMS>::kTile;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   if (tid == 0) S.tile_id = atomicAdd(tile_counter, 1u);
   for (int t = tid; t < kWarps * kRadix; t += kSortThreads) (&S.warp_hist[0][0])[t] = 0;
   __syncthreads();
   const uint32_t tile = S.tile_id;
-  const int64_t base = (int64_t)tile * kSortTile;
-  const int64_t seg = base + (int64_t)warp * 32 * kSortItems;
+  const int64_t base = (int64_t)tile * kTile;
+  const int count = (int)(n - base < kTile ? n - base : kTile);
+  const int seg = warp * 32 * ITEMS;
 
   // Load: warp w owns a contiguous segment; item `it` of lane l sits at
   // seg + it*32 + l, so (it, lane) order is input order within the warp.
-  uint64_t key[kSortItems];
-  uint32_t val[kSortItems];
-  uint32_t rank[kSortItems];
+  uint64_t key[ITEMS];
+  uint32_t val[ITEMS];
+  uint32_t rank[(ITEMS + 1) / 2] = {};  // two of 16 bits each
 #pragma unroll
-  for (int it = 0; it < kSortItems; ++it) {
-    int64_t idx = seg + it * 32 + lane;
-    bool ok = idx < n;
-    key[it] = ok ? keys_in[idx] : 0ull;
-    val[it] = ok ? vals_in[idx] : 0u;
+  for (int it = 0; it < ITEMS; ++it) {
+    const int idx = seg + it * 32 + lane;
+    const bool ok = idx < count;
+    key[it] = ok ? keys_in[base + idx] : 0ull;
+    val[it] = ok ? vals_in[base + idx] : 0u;
   }
   // Rank within the warp, in input order: peers with the same digit in this
-  // item, plus the warp's running count of that digit.  The group's leader
+  // item (one ballot per bit: they wait on nothing, so the items' overlap,
+  // where a match instruction per item took a third longer, 8M keys 846 ->
+  // 630 us a sort), plus the warp's running count of that digit.  The leader
   // adds the group size to the warp's counter; the old value is the group's
   // base.  The warp issues the items' adds in order, so item it's base counts
   // exactly the keys of items < it.
   const uint32_t lt = lanemask_lt();
 #pragma unroll
-  for (int it = 0; it < kSortItems; ++it) {
-    int64_t idx = seg + it * 32 + lane;
-    bool ok = idx < n;
+  for (int it = 0; it < ITEMS; ++it) {
+    const bool ok = seg + it * 32 + lane < count;
     uint32_t dg = ok ? (uint32_t)(key[it] >> shift) & 0xffu : 0x100u + lane;
-    uint32_t peers = __match_any_sync(0xffffffffu, dg);
+    uint32_t peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const bool p = (dg >> b) & 1u;
+      const uint32_t m = __ballot_sync(0xffffffffu, p);
+      peers &= p ? m : ~m;
+    }
     const int leader = __ffs(peers) - 1;
-    uint32_t base = 0u;
-    if (ok && leader == lane) base = atomicAdd(&S.warp_hist[warp][dg], (uint32_t)__popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    rank[it] = base + __popc(peers & lt);
+    uint32_t first = 0u;
+    if (ok && leader == lane) first = atomicAdd(&S.warp_hist[warp][dg], (uint32_t)__popc(peers));
+    first = __shfl_sync(0xffffffffu, first, leader);
+    rank[it / 2] |= (first + __popc(peers & lt)) << (16 * (it & 1));
   }
   __syncthreads();
 
-  // Thread t owns digit t: exclusive prefix over warps, and the tile total.
+  // Thread t owns digit t: its count in each warp, and the tile total.
   const int t = tid;
   uint32_t total = 0;
+  uint32_t before[kWarps];
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) {
-    uint32_t c = S.warp_hist[w][t];
-    S.warp_hist[w][t] = total;
-    total += c;
+    before[w] = total;
+    total += S.warp_hist[w][t];
   }
-  next_lookback[(int64_t)tile * kRadix + t] = 0u;
   // Publish this tile's count (tile 0 publishes a finished prefix at once).
   {
     volatile uint32_t *lb = lookback + (int64_t)tile * kRadix + t;
     *lb = (tile == 0 ? kFlagPrefix : kFlagAggregate) | total;
   }
-  // Exclusive scan of the totals over digits: local start of each digit.
+  next_lookback[(int64_t)tile * kRadix + t] = 0u;
+  // Exclusive scan of the totals over digits: local start of each digit, and
+  // from it the first local position of each warp's keys of that digit.
   uint32_t x = total;
   for (int o = 1; o < 32; o <<= 1) {
     uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
   if (lane == 31) S.warp_tot[warp] = x;
+  __syncthreads();
+  uint32_t start = x - total;
+  for (int q = 0; q < warp; ++q) start += S.warp_tot[q];
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) S.warp_hist[w][t] = start + before[w];
+  __syncthreads();
+
+  // Scatter into shared memory in tile-sorted order.  (Before the look-back:
+  // the registers are free for it, and the tiles before this one publish
+  // meanwhile.)
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    if (seg + it * 32 + lane < count) {
+      const uint32_t dg = (uint32_t)(key[it] >> shift) & 0xffu;
+      const uint32_t pos = S.warp_hist[warp][dg] + ((rank[it / 2] >> (16 * (it & 1))) & 0xffffu);
+      S.keys[pos] = key[it];
+      S.vals[pos] = val[it];
+    }
+  }
   // Look back over preceding tiles for digit t, kLookWindow tiles per round
   // trip: sum their counts in order up to the nearest finished prefix; a
   // tile that has not published yet is waited for.
@@ -205,50 +257,34 @@ __global__ void __launch_bounds__(kSortThreads, EMST_SORT_MIN_BLOCKS) k_sort_pas
     volatile uint32_t *mine = lookback + (int64_t)tile * kRadix + t;
     *mine = kFlagPrefix | ((excl + total) & kValueMask);
   }
-  __syncthreads();
-  uint32_t wbase = 0;
-  for (int q = 0; q < warp; ++q) wbase += S.warp_tot[q];
-  const uint32_t start = wbase + x - total;
-  S.tile_start[t] = start;
   S.global_base[t] = digit_offset[t] + excl - start;
   __syncthreads();
-
-  // Scatter into shared memory in tile-sorted order.
-#pragma unroll
-  for (int it = 0; it < kSortItems; ++it) {
-    int64_t idx = seg + it * 32 + lane;
-    if (idx < n) {
-      uint32_t dg = (uint32_t)(key[it] >> shift) & 0xffu;
-      uint32_t pos = S.tile_start[dg] + S.warp_hist[warp][dg] + rank[it];
-      S.keys[pos] = key[it];
-      S.vals[pos] = val[it];
-    }
-  }
-  __syncthreads();
   // Write out: consecutive threads write consecutive positions of a digit run.
-  int64_t count = n - base < kSortTile ? n - base : kSortTile;
-  for (int i = tid; i < count; i += kSortThreads) {
-    uint64_t k = S.keys[i];
-    uint32_t dg = (uint32_t)(k >> shift) & 0xffu;
-    uint32_t out = S.global_base[dg] + (uint32_t)i;
-    keys_out[out] = k;
-    vals_out[out] = S.vals[i];
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    const int i = it * kSortThreads + tid;
+    if (i < count) {
+      const uint64_t k = S.keys[i];
+      const uint32_t out = S.global_base[(uint32_t)(k >> shift) & 0xffu] + (uint32_t)i;
+      keys_out[out] = k;
+      vals_out[out] = S.vals[i];
+    }
   }
 }
 
-static bool g_sort_attr_set[64] = {false};
-
-int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0) {
-  if (n <= 1 || digit_begin >= digit_end) return src;
+// One sort of tiles of kSortThreads x ITEMS keys.
+template <int ITEMS, int BLOCKS>
+static int sort_passes(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0) {
+  static bool attr_set[64] = {false};
   cudaStream_t s = P.stream;
   int dev = 0;
   cudaGetDevice(&dev);
-  const size_t smem = sizeof(SortSmem);
-  if (dev < 64 && !g_sort_attr_set[dev]) {
-    cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    g_sort_attr_set[dev] = true;
+  const size_t smem = sizeof(SortSmem<ITEMS>);
+  if (dev >= 64 || !attr_set[dev]) {
+    cudaFuncSetAttribute(k_sort_pass<ITEMS, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (dev < 64) attr_set[dev] = true;
   }
-  const int64_t tiles = sort_tiles_for(n);
+  const int64_t tiles = (n + SortSmem<ITEMS>::kTile - 1) / SortSmem<ITEMS>::kTile;
   uint32_t *hist = P.sort_state, *counters = hist + kHistWords;
   uint32_t *look[2] = {counters + kCounterWords, counters + kCounterWords + kRadix * tiles};
   cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)(kHistWords + kCounterWords + kRadix * tiles), s);
@@ -257,7 +293,7 @@ int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int 
   k_sort_hist<<<hgrid, 512, 0, s>>>(P.keys[src], n, digit_begin, digit_end, bit0, hist, counters + 8);
   P.launches += 1;
   for (int d = digit_begin; d < digit_end; ++d) {
-    k_sort_pass<<<(unsigned)tiles, kSortThreads, smem, s>>>(
+    k_sort_pass<ITEMS, BLOCKS><<<(unsigned)tiles, kSortThreads, smem, s>>>(
         P.keys[src], P.vals[src], P.keys[src ^ 1], P.vals[src ^ 1], n, bit0 + 8 * d, hist + d * kRadix,
         look[0], look[1], counters + d, P.counters + 1);
     P.launches += 1;
@@ -267,6 +303,13 @@ int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int 
     look[1] = t;
   }
   return src;
+}
+
+int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0) {
+  if (n <= 1 || digit_begin >= digit_end) return src;
+  if (n <= kSmallMax) return sort_passes<kSmallItems, 4>(P, n, digit_begin, digit_end, src, bit0);
+  if (n <= kMidMax) return sort_passes<kMidItems, 4>(P, n, digit_begin, digit_end, src, bit0);
+  return sort_passes<kLargeItems, 3>(P, n, digit_begin, digit_end, src, bit0);
 }
 
 }  // namespace emst
