@@ -192,7 +192,6 @@ size_t layout(Problem &P, char *base, bool copy_points, bool copy_edges) {
   P.vals[1] = c.take<uint32_t>(n);
   P.nodes = c.take<NodeRec>(nc - 1);
   P.nlabels = c.take<uint2>(nc - 1);
-  P.arrivals = c.take<uint64_t>(nc - 1);
   P.range = c.take<uint2>(nc - 1);
   P.runs = c.take<uint32_t>(n);
   P.scan_tiles = c.take<uint32_t>(2 * scan_tiles_for(n));

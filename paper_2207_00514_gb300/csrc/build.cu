@@ -354,11 +354,9 @@ __global__ void __launch_bounds__(kBlock) k_gather(const float *__restrict__ pts
                                                    uint32_t *__restrict__ inst_of,
                                                    const uint64_t *__restrict__ sorted_codes,
                                                    const uint64_t *__restrict__ code_hi,
-                                                   unsigned long long *dup,
-                                                   uint64_t *__restrict__ arrivals, int64_t splits) {
+                                                   unsigned long long *dup) {
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  if (k < splits) arrivals[k] = 0u;  // for the hierarchy
   uint32_t o = __ldg(perm + k);
   if (inst_of) inst_of[k] = __ldg(inst_in + o);
   const float *p = pts + (int64_t)o * DIM;
@@ -392,44 +390,46 @@ void launch_gather(Problem &P, const uint32_t *perm) {
   if (P.wide) cudaMemsetAsync(dup, 0, 3 * sizeof(unsigned long long), P.stream);
   if (P.dim == 3)
     k_gather<3><<<g, kBlock, 0, P.stream>>>(P.points, perm, P.n, P.pts, P.labels, P.inst_in,
-                                            P.inst_of, P.keys[0], P.code_hi, dup, P.arrivals, P.nc - 1);
+                                            P.inst_of, P.keys[0], P.code_hi, dup);
   else
     k_gather<2><<<g, kBlock, 0, P.stream>>>(P.points, perm, P.n, P.pts, P.labels, P.inst_in,
-                                            P.inst_of, P.keys[0], P.code_hi, dup, P.arrivals, P.nc - 1);
+                                            P.inst_of, P.keys[0], P.code_hi, dup);
   P.launches += 1;
 }
 
 // ---------------------------------------------------------------------------
-// A4 (b, c). Hierarchy and boxes in one bottom-up pass.
+// A4 (b, c). Hierarchy and boxes without a climb.
 // The hierarchy is Karras's binary radix tree over the leaf chunks (chunks of
 // `leaf` consecutive sorted points; leaf = 1: one point per leaf; chunk c's
 // key is the code of its first point, augmented by c so equal codes still
 // split), numbered as in Fig. 4: internal node i covers a chunk range with
 // one end at i, and its split gamma gives the children gamma (left) and
 // gamma + 1 (right), leaves when the range ends there.
-// Here it is found from the leaves up (the agglomerative form of the same
-// tree): with delta(i) the leading bits shared by the keys of chunks i and
-// i + 1, a node covering chunks [l, r] hangs under the split r (it is the
-// left child) when delta(r) > delta(l - 1), else under the split l - 1 (the
-// right child).  So a left child's index is its right end and a right
-// child's its left end: a node knows its own index once it knows which side
-// it hangs on.  At every split the first child to arrive stops and the
-// second builds the parent: its range from both children's far ends, its
-// box as the union of theirs, its record (both child boxes, the child
-// references, their smallest original ids), range and round-0 child labels,
-// written once at the parent's index; then it carries on upwards.
-// k_build_local: one thread per leaf chunk climbs the splits between two of
-// its CTA's chunks, with the CTA's shared keys' delta values, boxes and
-// arrival counts in shared memory (block-scope acquire-release adds).  A
-// split at the CTA's edge ends the climb in global memory: the thread
-// exchanges its arrival entry (device scope, acquire-release) and the second
-// arriver lists the split.  A split inside the CTA that only one child
-// reached (the other spans CTAs) passes that child's entry to global memory
-// at the end.
-// k_build_up: one thread per listed split builds it and climbs on in global
-// memory; a child's box comes from its record (the union of the record's two
-// child boxes) or from its points (a leaf).
-// Each split gets exactly two arrivals; the entries start at zero.
+// With delta(i) the leading bits shared by the keys of chunks i and i + 1,
+// the node of split s covers the chunks between the nearest splits p < s < q
+// of smaller delta, [p + 1, q] (within any node's range the smallest delta
+// occurs once: there the first differing bit goes from 0 to 1).  It hangs on
+// the side of the larger of delta(p) and delta(q): under q as its left child
+// when delta(q) is larger (its index is then its right end q), else under p
+// as its right child (its index is its left end).  So every node follows
+// from three range queries: the two nearest smaller deltas, and the boxes of
+// its two children -- no arrivals, no walk up the tree.
+// k_build_tile: a CTA takes kBuildTile consecutive chunks, tabulates in
+// shared memory the boxes of every run of 1, 2, 4, ... chunks and the minima
+// of every run of 1, 2, 4, ... deltas, and a thread per split finds p and q
+// by descending the tables and each child's box as the union of two runs.  A
+// split whose p or q lies outside the CTA stays open; the subtrees between
+// the open splits are done and leave as items (box, smallest original id,
+// the open split after them and its delta), some 15 of 128 chunks.
+// k_build_merge: the same over items instead of chunks, a group of CTAs'
+// items per CTA, until one CTA has them all.  A CTA whose group has more
+// items than its tables hold takes them in turn, keeping what stays open.
+// What bounds it: shared-memory wavefronts and the tables' barriers at 28
+// warps per SM.  Measured (us, the climb with one arrival per child that stood
+// here before / this): CTA-local part 2,480 / 1,330 at 37M halo points (its
+// bytes take 570), 23 / 13 at 200,000; the rest 413 / 219 and 79 / 22 -- a
+// climb above the CTAs was a chain of two L2 round trips per level.  256
+// chunks per CTA: whole call 35.43 against 35.19 ms at 37M, the same at 1M.
 // The child labels are the round-0 ones (a one-point chunk k: label k;
 // otherwise several components, kInvalid); a caller with other labels
 // rewrites them (A5).
@@ -451,286 +451,355 @@ __device__ __forceinline__ int prefix_delta(const uint64_t *__restrict__ k,
   return base + 64 + __clz((int)((uint32_t)i ^ (uint32_t)j));
 }
 
-#ifndef EMST_REFIT_BLOCK
-#define EMST_REFIT_BLOCK 128
+#ifndef EMST_BUILD_TILE
+#define EMST_BUILD_TILE 128
 #endif
-constexpr int kRefitBlock = EMST_REFIT_BLOCK;  // leaf chunks per k_build_local CTA
-constexpr int kRefitUpBlock = 128;
-constexpr uint32_t kRefitReadyCounter = 48;  // P.counters slot: splits listed by k_build_local
-
-// The split a node [l, r] hangs under and its side (0: left child, the split
-// is r; 1: right child, the split is l - 1), from delta(l - 1) and delta(r);
-// false for the root.
-__device__ __forceinline__ bool parent_split(int64_t l, int64_t r, int64_t nc, int dl, int dr,
-                                             uint32_t &ps, int &side) {
-  if (l == 0 && r == nc - 1) return false;
-  const bool left = l == 0 || (r != nc - 1 && dr > dl);
-  ps = (uint32_t)(left ? r : l - 1);
-  side = left ? 0 : 1;
-  return true;
-}
-
-// The index of node [l, r] (Fig. 4 numbering): 0 for the root, else the end
-// of its range away from the split it hangs under.
-__device__ __forceinline__ uint32_t node_index(int64_t l, int64_t r, bool root, int side) {
-  return root ? 0u : (uint32_t)(side == 0 ? r : l);
-}
+constexpr int kBuildTile = EMST_BUILD_TILE;  // leaf chunks per k_build_tile CTA
+constexpr int kMergeTile = 256;              // items in a k_build_merge CTA's tables
+// The last CTA's: at most 160 splits stay open on either side of what a CTA
+// holds (their deltas, below 161, fall towards it), so 512 always leave room.
+constexpr int kLastTile = 512;
+constexpr int kMaxGroup = 64;                // CTAs whose items one CTA takes
 
 __device__ __forceinline__ void chunk_box(const float4 *__restrict__ pts, int64_t n, int leaf,
-                                          int64_t c, float *box, uint32_t &idmin) {
+                                          int64_t c, float4 &lo, float4 &hi) {
   const int64_t p0 = c * leaf, p1 = p0 + leaf < n ? p0 + leaf : n;
-  float4 p = __ldg(pts + p0);
-  box[0] = box[3] = p.x;
-  box[1] = box[4] = p.y;
-  box[2] = box[5] = p.z;
-  idmin = __float_as_uint(p.w);
+  lo = hi = __ldg(pts + p0);
   for (int64_t m = p0 + 1; m < p1; ++m) {
-    p = __ldg(pts + m);
-    box[0] = fminf(box[0], p.x); box[1] = fminf(box[1], p.y); box[2] = fminf(box[2], p.z);
-    box[3] = fmaxf(box[3], p.x); box[4] = fmaxf(box[4], p.y); box[5] = fmaxf(box[5], p.z);
-    idmin = min(idmin, __float_as_uint(p.w));
+    const float4 p = __ldg(pts + m);
+    lo.x = fminf(lo.x, p.x); lo.y = fminf(lo.y, p.y); lo.z = fminf(lo.z, p.z);
+    hi.x = fmaxf(hi.x, p.x); hi.y = fmaxf(hi.y, p.y); hi.z = fmaxf(hi.z, p.z);
+    lo.w = __uint_as_float(min(__float_as_uint(lo.w), __float_as_uint(p.w)));
   }
 }
 
-// A finished child's box and smallest original id: a leaf chunk's from its
-// points, an internal node's from its record (written before its arrival was
-// released, so read through L2).
-__device__ __forceinline__ void child_box(const float4 *__restrict__ pts, int64_t n, int leaf,
-                                          const NodeRec *nodes, uint32_t idx, bool is_leaf,
-                                          float *box, uint32_t &idmin) {
-  if (is_leaf) {
-    chunk_box(pts, n, leaf, idx, box, idmin);
+// A subtree's box; lo.w: its smallest original id.
+struct Subtree {
+  float4 lo, hi;
+};
+__device__ __forceinline__ Subtree unite(const Subtree &a, const Subtree &b) {
+  Subtree r;
+  r.lo.x = fminf(a.lo.x, b.lo.x); r.lo.y = fminf(a.lo.y, b.lo.y); r.lo.z = fminf(a.lo.z, b.lo.z);
+  r.hi.x = fmaxf(a.hi.x, b.hi.x); r.hi.y = fmaxf(a.hi.y, b.hi.y); r.hi.z = fmaxf(a.hi.z, b.hi.z);
+  r.lo.w = __uint_as_float(min(__float_as_uint(a.lo.w), __float_as_uint(b.lo.w)));
+  r.hi.w = 0.f;
+  return r;
+}
+
+// Items 0 .. N-1 of a CTA with the splits around them: entry e is the split
+// before item e (entry N the one after the last item).
+template <int TILE>
+struct BuildTables {
+  static constexpr int kLevels = TILE == 128 ? 7 : TILE == 256 ? 8 : 9;
+  static_assert(TILE == 1 << kLevels, "a power of two");
+  float4 lo[kLevels][TILE];                // [k][i]: items i .. i + 2^k - 1
+  float4 hi[kLevels][TILE];
+  int16_t delta[kLevels + 1][TILE + 2];    // [k][e]: entries e .. e + 2^k - 1
+  uint32_t pos[TILE + 1];                  // the splits' chunk positions (k_build_merge)
+  uint32_t open[TILE / 32];
+  uint32_t before[kMaxGroup + 1];          // k_build_merge: items of the group's CTAs before each
+};
+
+struct TreeOut {
+  NodeRec *nodes;
+  uint2 *nlabels, *range;
+  int64_t n, nc;
+  int leaf;
+};
+
+// Node `idx` covering chunks [L, R] with split g and children's boxes a, b:
+// its record, range and round-0 child labels.
+__device__ __forceinline__ void write_node(const TreeOut &T, uint32_t idx, uint32_t L, uint32_t g, uint32_t R,
+                                           const Subtree &a, const Subtree &b) {
+  const bool lleaf = L == g, rleaf = R == g + 1u;
+  NodeRec *rec = T.nodes + idx;
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(rec), "f"(a.lo.x), "f"(a.lo.y),
+               "f"(a.lo.z), "f"(a.hi.x), "f"(a.hi.y), "f"(a.hi.z), "f"(b.lo.x), "f"(b.lo.y)
+               : "memory");
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                   reinterpret_cast<char *>(rec) + 32),
+               "f"(b.lo.z), "f"(b.hi.x), "f"(b.hi.y), "f"(b.hi.z),
+               "f"(__uint_as_float(lleaf ? (kLeafBit | g) : g)),
+               "f"(__uint_as_float(rleaf ? (kLeafBit | (g + 1u)) : g + 1u)), "f"(a.lo.w), "f"(b.lo.w)
+               : "memory");
+  T.range[idx] = pack_range(idx, L, g, R);
+  // a chunk of exactly one point is its own component in round 0
+  auto one_point = [&](int64_t c) { return T.leaf == 1 || T.n - c * T.leaf == 1; };
+  T.nlabels[idx] = make_uint2(lleaf && one_point(g) ? (uint32_t)((int64_t)g * T.leaf) : kInvalid,
+                              rleaf && one_point(g + 1) ? (uint32_t)((int64_t)(g + 1) * T.leaf) : kInvalid);
+}
+
+// One step over the N items in the tables' level 0 (filled by the caller, a
+// barrier not yet passed): builds every node whose range ends inside, and
+// returns for each thread whether the split after its item is open (the last
+// one always counts as open), and then the subtree between the open split
+// before and that one, and its rank among them.  LINEAR: item i is chunk
+// first + i.  Every thread of the CTA (one per item) calls.
+template <int TILE, bool LINEAR>
+__device__ __forceinline__ bool build_step(BuildTables<TILE> &S, int N, uint32_t first, const TreeOut &T,
+                                           Subtree &item, int &rank, int &count) {
+  constexpr int kLevels = BuildTables<TILE>::kLevels;
+  const int i = threadIdx.x;
+  __syncthreads();
+  {
+    Subtree me;
+    int low = 0;
+    if (i < N) { me.lo = S.lo[0][i]; me.hi = S.hi[0][i]; }
+    if (i <= N) low = S.delta[0][i];
+#pragma unroll
+    for (int k = 1; k <= kLevels; ++k) {
+      const int h = 1 << (k - 1);
+      if (2 * h > N + 1) break;
+      if (k < kLevels && i + 2 * h <= N) {
+        Subtree o;
+        o.lo = S.lo[k - 1][i + h];
+        o.hi = S.hi[k - 1][i + h];
+        me = unite(me, o);
+        S.lo[k][i] = me.lo;
+        S.hi[k][i] = me.hi;
+      }
+      if (i + 2 * h <= N + 1) {
+        low = min(low, (int)S.delta[k - 1][i + h]);
+        S.delta[k][i] = (int16_t)low;
+      }
+      __syncthreads();
+    }
+  }
+  auto at = [&](int e) { return LINEAR ? first - 1u + (uint32_t)e : S.pos[e]; };
+  // the union of items [a, a + len): two runs that cover it
+  auto run = [&](int a, int len) {
+    int k = 31 - __clz(len);
+    if (k > kLevels - 1) k = kLevels - 1;
+    Subtree r;
+    r.lo = S.lo[k][a];
+    r.hi = S.hi[k][a];
+    if (len > (1 << k)) {
+      Subtree o;
+      o.lo = S.lo[k][a + len - (1 << k)];
+      o.hi = S.hi[k][a + len - (1 << k)];
+      r = unite(r, o);
+    }
+    return r;
+  };
+  bool open = i < N;
+  if (i < N - 1) {
+    const int e = i + 1;
+    const int d = S.delta[0][e];
+    int p = e, q = e + 1;  // entries [p, e) and (e, q) lie above d
+#pragma unroll
+    for (int k = kLevels; k >= 0; --k) {
+      if (p >= (1 << k) && S.delta[k][p - (1 << k)] > d) p -= 1 << k;
+      if (q + (1 << k) <= N + 1 && S.delta[k][q] > d) q += 1 << k;
+    }
+    if (p > 0 && q <= N) {
+      open = false;
+      --p;
+      const Subtree a = run(p, e - p), b = run(e, q - e);
+      const uint32_t L = at(p) + 1u, R = at(q);
+      const int dl = S.delta[0][p], dr = S.delta[0][q];
+      // (the root: both outer deltas are -1)
+      const uint32_t idx = dr > dl ? R : dl < 0 ? 0u : L;
+      write_node(T, idx, L, at(e), R, a, b);
+    }
+  }
+  const unsigned b = __ballot_sync(0xffffffffu, open);
+  const int warp = i >> 5;
+  if ((i & 31) == 0) S.open[warp] = b;
+  __syncthreads();
+  rank = 0;
+  count = 0;
+#pragma unroll
+  for (int w = 0; w < TILE / 32; ++w) {
+    const int c = __popc(S.open[w]);
+    rank += w < warp ? c : 0;
+    count += c;
+  }
+  unsigned m = b & ((1u << (i & 31)) - 1u);
+  rank += __popc(m);
+  if (open) {
+    int w = warp;
+    while (m == 0u && w > 0) m = S.open[--w];
+    const int prev = m ? w * 32 + 31 - __clz(m) : -1;
+    item = run(prev + 1, i - prev);
+  }
+  return open;
+}
+
+// Where the items of a CTA lie: from its first chunk's place on.
+struct Items {
+  float4 *lo, *hi;  // hi.w: the position of the open split after it
+  int *delta;       // of that split
+};
+
+template <int TILE>
+__global__ void __launch_bounds__(TILE) k_build_tile(const uint64_t *__restrict__ keys,
+                                                     const uint64_t *__restrict__ keys_hi,
+                                                     const float4 *__restrict__ pts, TreeOut T, Items items,
+                                                     uint32_t *__restrict__ counts, uint32_t *status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  BuildTables<TILE> &S = *reinterpret_cast<BuildTables<TILE> *>(smem_raw);
+  const int i = threadIdx.x;
+  const int64_t first = (int64_t)blockIdx.x * TILE;
+  const int N = (int)(T.nc - first < TILE ? T.nc - first : TILE);
+  if (i < N) {
+    float4 lo, hi;
+    chunk_box(pts, T.n, T.leaf, first + i, lo, hi);
+    S.lo[0][i] = lo;
+    S.hi[0][i] = hi;
+  }
+  for (int e = i; e <= N; e += TILE)
+    S.delta[0][e] = (int16_t)prefix_delta(keys, keys_hi, T.nc, T.leaf, first - 1 + e, first + e);
+  Subtree item;
+  int rank, count;
+  const bool open = build_step<TILE, true>(S, N, (uint32_t)first, T, item, rank, count);
+  if (gridDim.x == 1) {
+    if (i == 0 && count != 1) atomicOr(status, kErrChain);  // cannot happen: both ends are here
     return;
   }
-  const float4 *f = reinterpret_cast<const float4 *>(nodes + idx);
-  const float4 a = __ldcg(f), b = __ldcg(f + 1), c = __ldcg(f + 2);
-  const uint4 d = __ldcg(reinterpret_cast<const uint4 *>(f + 3));
-  box[0] = fminf(a.x, b.z); box[1] = fminf(a.y, b.w); box[2] = fminf(a.z, c.x);
-  box[3] = fmaxf(a.w, c.y); box[4] = fmaxf(b.x, c.z); box[5] = fmaxf(b.y, c.w);
-  idmin = min(d.z, d.w);
-}
-
-// Node `idx` covering chunks [L, R] with split g and child boxes Lb, Rb (and
-// their smallest original ids): its whole record, range and round-0 child
-// labels; returns the union in `box` / `idmin` (which may alias Lb or Rb).
-__device__ __forceinline__ void write_node(NodeRec *nodes, uint2 *__restrict__ nlabels,
-                                           uint2 *__restrict__ range, uint32_t idx, uint32_t L,
-                                           uint32_t g, uint32_t R, const float *Lb, const float *Rb,
-                                           uint32_t minL, uint32_t minR, int64_t n, int leaf,
-                                           float *box, uint32_t &idmin) {
-  const bool lleaf = L == g, rleaf = R == g + 1u;
-  // a chunk of exactly one point is its own component in round 0
-  auto one_point = [&](int64_t c) { return n - c * leaf == 1 || leaf == 1; };
-  NodeRec rec;
-  rec.a = make_float4(Lb[0], Lb[1], Lb[2], Lb[3]);
-  rec.b = make_float4(Lb[4], Lb[5], Rb[0], Rb[1]);
-  rec.c = make_float4(Rb[2], Rb[3], Rb[4], Rb[5]);
-  rec.d = make_uint4(lleaf ? (kLeafBit | g) : g, rleaf ? (kLeafBit | (g + 1u)) : g + 1u, minL, minR);
-  nodes[idx] = rec;
-  range[idx] = pack_range(idx, L, g, R);
-  nlabels[idx] = make_uint2(lleaf && one_point(g) ? (uint32_t)((int64_t)g * leaf) : kInvalid,
-                            rleaf && one_point(g + 1) ? (uint32_t)((int64_t)(g + 1) * leaf) : kInvalid);
-#pragma unroll
-  for (int t = 0; t < 3; ++t) {
-    const float lo = fminf(Lb[t], Rb[t]), hi = fmaxf(Lb[3 + t], Rb[3 + t]);
-    box[t] = lo;
-    box[3 + t] = hi;
+  if (open) {
+    items.lo[first + rank] = item.lo;
+    items.hi[first + rank] = make_float4(item.hi.x, item.hi.y, item.hi.z, __uint_as_float((uint32_t)(first + i)));
+    items.delta[first + rank] = S.delta[0][i + 1];
   }
-  idmin = min(minL, minR);
+  if (i == 0) counts[blockIdx.x] = (uint32_t)count;
 }
 
-// A split's arrival entry: 0 until a child arrives, then that child's far end
-// and outer delta (the leading bits its far end's key shares with the key
-// beyond it), so the second arriver learns from its own exchange the parent's
-// whole range and both deltas that say where the parent hangs: no load of
-// either before the sibling's box.  Acquire-release order: the first arriver's
-// stores (its record) are released by its exchange and acquired by the
-// second's.  (With a counter, the far end and the deltas' keys loaded after
-// it, a level above the CTAs took four dependent round trips instead of two:
-// k_build_up 131 -> 78 us at 200,000 halo points, 644 -> 418 us at 37M.)
-__device__ __forceinline__ uint64_t pack_arrival(uint32_t far, int outer_delta) {
-  return (1ull << 63) | ((uint64_t)(uint32_t)(outer_delta + 1) << 32) | (uint64_t)far;
-}
-__device__ __forceinline__ uint32_t arrival_far(uint64_t a) { return (uint32_t)a; }
-__device__ __forceinline__ int arrival_delta(uint64_t a) { return (int)((a >> 32) & 0x7fffffffu) - 1; }
-__device__ __forceinline__ uint64_t exch_acq_rel_gpu(uint64_t *p, uint64_t v) {
-  uint64_t old;
-  asm volatile("atom.acq_rel.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ uint32_t add_acq_rel_cta_shared(uint32_t *p, uint32_t v) {
-  uint32_t old;
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
-  return old;
-}
-
-// A split both of whose children k_build_local finished: the split, the
-// parent's range, and the deltas outside it (+ 1, the left one in the low half).
-__device__ __forceinline__ uint4 ready_entry(uint32_t ps, uint32_t L, uint32_t R, int dl, int dr) {
-  return make_uint4(ps, L, R, (uint32_t)(dl + 1) | ((uint32_t)(dr + 1) << 16));
-}
-
-__global__ void __launch_bounds__(kRefitBlock) k_build_local(
-    const uint64_t *__restrict__ keys, const uint64_t *__restrict__ keys_hi,
-    const float4 *__restrict__ pts, int64_t n, int64_t nc, int leaf, NodeRec *nodes,
-    uint2 *__restrict__ nlabels, uint2 *__restrict__ range, uint64_t *arrivals,
-    uint4 *__restrict__ ready, uint32_t *ready_count, uint32_t capacity, uint32_t *status) {
-  __shared__ int s_delta[kRefitBlock + 1];     // delta(first - 1 + t)
-  __shared__ float s_box[kRefitBlock][2][6];   // both child boxes of each split inside the CTA
-  __shared__ uint32_t s_min[kRefitBlock][2];   // their smallest original ids
-  __shared__ uint32_t s_far[kRefitBlock][2];   // their far ends (kInvalid: not arrived)
-  __shared__ uint32_t s_arrive[kRefitBlock];
-  const int64_t first = (int64_t)blockIdx.x * kRefitBlock;
-  const int64_t last = first + kRefitBlock - 1 < nc - 1 ? first + kRefitBlock - 1 : nc - 1;
-  for (int t = threadIdx.x; t <= kRefitBlock; t += blockDim.x)
-    s_delta[t] = prefix_delta(keys, keys_hi, nc, leaf, first - 1 + t, first + t);
-  s_arrive[threadIdx.x] = 0u;
-  s_far[threadIdx.x][0] = s_far[threadIdx.x][1] = kInvalid;
+// The items of `group` CTAs of the launch before (each CTA's from place
+// span * its index on) reduced to what stays open, in their own first places:
+// no more are written than were read, so nothing unread is overwritten.
+template <int TILE>
+__global__ void __launch_bounds__(TILE) k_build_merge(const uint64_t *__restrict__ keys,
+                                                      const uint64_t *__restrict__ keys_hi, TreeOut T, Items items,
+                                                      int64_t span, int group, int64_t ctas_in,
+                                                      const uint32_t *__restrict__ counts_in,
+                                                      uint32_t *__restrict__ counts, uint32_t *status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  BuildTables<TILE> &S = *reinterpret_cast<BuildTables<TILE> *>(smem_raw);
+  const int i = threadIdx.x;
+  const int64_t c0 = (int64_t)blockIdx.x * group;
+  const int ctas = (int)(ctas_in - c0 < group ? ctas_in - c0 : group);
+  const int64_t first = c0 * span;
+  const bool last_cta = gridDim.x == 1;
+  if (i < kMaxGroup + 1) S.before[i] = i > 0 && i <= ctas ? counts_in[c0 + i - 1] : 0u;
+  if (i == TILE - 1) {
+    S.pos[0] = (uint32_t)first - 1u;
+    S.delta[0][0] = (int16_t)prefix_delta(keys, keys_hi, T.nc, T.leaf, first - 1, first);
+  }
   __syncthreads();
-  const int64_t k = first + threadIdx.x;  // this thread's chunk
-  if (k <= last) {
-    float box[6];
-    uint32_t idmin;
-    chunk_box(pts, n, leaf, k, box, idmin);
-    int64_t l = k, r = k;
-    uint32_t ps;
-    int side;
-    bool up = parent_split(l, r, nc, s_delta[l - first], s_delta[r - first + 1], ps, side);
-    while (up) {
-      const uint32_t far = side == 0 ? (uint32_t)l : (uint32_t)r;
-      if ((int64_t)ps < first || (int64_t)ps >= last) {
-        // a split at the CTA's edge: its other child lies (partly) in another CTA
-        const int dl = s_delta[l - first], dr = s_delta[r - first + 1];
-        const uint64_t sib = exch_acq_rel_gpu(arrivals + ps, pack_arrival(far, side == 0 ? dl : dr));
-        if (sib != 0u) {  // second: list it
-          const uint32_t at = atomicAdd(ready_count, 1u);
-          if (at < capacity)
-            ready[at] = side == 0
-                            ? ready_entry(ps, (uint32_t)l, arrival_far(sib), dl, arrival_delta(sib))
-                            : ready_entry(ps, arrival_far(sib), (uint32_t)r, arrival_delta(sib), dr);
-          else atomicOr(status, kErrChain);  // cannot happen (see launch_build_tree)
-        }
-        break;
-      }
-      const int j = (int)(ps - first);
+  if (i < 32) {  // running totals of two counts per lane
+    static_assert(kMaxGroup == 64, "two counts per lane");
+    const uint32_t a = S.before[2 * i + 1], b = S.before[2 * i + 2];
+    uint32_t x = a + b;
 #pragma unroll
-      for (int t = 0; t < 6; ++t) s_box[j][side][t] = box[t];
-      s_min[j][side] = idmin;
-      s_far[j][side] = far;
-      if (add_acq_rel_cta_shared(&s_arrive[j], 1u) == 0u) break;  // first: the sibling carries on
-      float sib[6];
-#pragma unroll
-      for (int t = 0; t < 6; ++t) sib[t] = s_box[j][side ^ 1][t];
-      const uint32_t sibmin = s_min[j][side ^ 1], sibfar = s_far[j][side ^ 1];
-      if (side == 0 ? (sibfar <= ps || (int64_t)sibfar > last) : ((int64_t)sibfar < first || sibfar > ps)) {
-        atomicOr(status, kErrChain);  // cannot happen: the sibling lies in this CTA
-        break;
-      }
-      // the parent covers [L, R] with split ps; which side it hangs on gives its index
-      const int64_t L = side == 0 ? l : (int64_t)sibfar, R = side == 0 ? (int64_t)sibfar : r;
-      uint32_t ps2;
-      int side2;
-      up = parent_split(L, R, nc, s_delta[L - first], s_delta[R - first + 1], ps2, side2);
-      const uint32_t idx = node_index(L, R, !up, side2);
-      if (side == 0)
-        write_node(nodes, nlabels, range, idx, (uint32_t)L, ps, (uint32_t)R, box, sib, idmin, sibmin, n,
-                   leaf, box, idmin);
-      else
-        write_node(nodes, nlabels, range, idx, (uint32_t)L, ps, (uint32_t)R, sib, box, sibmin, idmin, n,
-                   leaf, box, idmin);
-      l = L;
-      r = R;
-      ps = ps2;
-      side = side2;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (i >= o) x += y;
     }
+    S.before[2 * i + 1] = x - b;
+    S.before[2 * i + 2] = x;
   }
   __syncthreads();
-  // a split inside the CTA that one child reached: the other spans CTAs and
-  // arrives in k_build_up
-  const int64_t s = first + threadIdx.x;
-  if (s < last && s_arrive[threadIdx.x] == 1u) {
-    const int side = s_far[threadIdx.x][0] != kInvalid ? 0 : 1;
-    const uint32_t far = s_far[threadIdx.x][side];
-    arrivals[s] = pack_arrival(far, s_delta[(int64_t)far - first + side]);
-  }
-}
-
-__global__ void __launch_bounds__(kRefitUpBlock) k_build_up(
-    const float4 *__restrict__ pts, int64_t n, int64_t nc, int leaf, NodeRec *nodes,
-    uint2 *__restrict__ nlabels, uint2 *__restrict__ range, uint64_t *arrivals,
-    const uint4 *__restrict__ ready, const uint32_t *ready_count, uint32_t capacity,
-    uint32_t *status) {
-  const uint32_t count = min(*ready_count, capacity);
-  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < count; t += gridDim.x * blockDim.x) {
-    const uint4 e = __ldg(ready + t);
-    uint32_t ps = e.x;
-    if (e.y > ps || e.z <= ps || (int64_t)e.z >= nc) {  // cannot happen: both children arrived
-      atomicOr(status, kErrChain);
+  const int total = (int)S.before[ctas];
+  int have = 0, read = 0;
+  int64_t out = first;
+  for (;;) {
+    const int take = min(total - read, TILE - have);
+    if (i < take) {
+      const uint32_t f = (uint32_t)(read + i);
+      int lo = 0, hi = ctas - 1;  // the last CTA whose items start at or before f
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (S.before[mid] <= f) lo = mid;
+        else hi = mid - 1;
+      }
+      const int64_t at = first + lo * span + (int64_t)(f - S.before[lo]);
+      const float4 hi4 = items.hi[at];
+      S.lo[0][have + i] = items.lo[at];
+      S.hi[0][have + i] = hi4;
+      S.pos[have + i + 1] = __float_as_uint(hi4.w);
+      S.delta[0][have + i + 1] = (int16_t)items.delta[at];
+    }
+    read += take;
+    have += take;
+    Subtree item;
+    int rank, count;
+    const bool open = build_step<TILE, false>(S, have, 0u, T, item, rank, count);
+    const bool more = read < total;
+    const uint32_t pos = open ? S.pos[i + 1] : 0u;
+    const int16_t delta = open ? S.delta[0][i + 1] : (int16_t)0;
+    __syncthreads();
+    if (more && (last_cta || count <= TILE / 2)) {  // on with these and the next ones
+      if (open) {
+        S.lo[0][rank] = item.lo;
+        S.hi[0][rank] = item.hi;
+        S.pos[rank + 1] = pos;
+        S.delta[0][rank + 1] = delta;
+      }
+      have = count;
+      if (have >= TILE) {  // cannot happen (kLastTile)
+        if (i == 0) atomicOr(status, kErrChain);
+        return;
+      }
       continue;
     }
-    float box[6], sib[6];
-    uint32_t idmin, sibmin;
-    child_box(pts, n, leaf, nodes, ps, e.y == ps, box, idmin);
-    child_box(pts, n, leaf, nodes, ps + 1u, e.z == ps + 1u, sib, sibmin);
-    int64_t L = e.y, R = e.z;
-    int dl = (int)(e.w & 0xffffu) - 1, dr = (int)(e.w >> 16) - 1;
-    int side = 0;  // the child whose box is in `box`
-    while (true) {
-      uint32_t ps2;
-      int side2;
-      const bool up = parent_split(L, R, nc, dl, dr, ps2, side2);
-      const uint32_t idx = node_index(L, R, !up, side2);
-      if (side == 0)
-        write_node(nodes, nlabels, range, idx, (uint32_t)L, ps, (uint32_t)R, box, sib, idmin, sibmin, n,
-                   leaf, box, idmin);
-      else
-        write_node(nodes, nlabels, range, idx, (uint32_t)L, ps, (uint32_t)R, sib, box, sibmin, idmin, n,
-                   leaf, box, idmin);
-      if (!up) break;
-      // arrive at the parent's split; the record just written is released with the exchange
-      ps = ps2;
-      side = side2;
-      const uint64_t other = exch_acq_rel_gpu(
-          arrivals + ps, pack_arrival(side == 0 ? (uint32_t)L : (uint32_t)R, side == 0 ? dl : dr));
-      if (other == 0u) break;  // first: the sibling carries on
-      const uint32_t sibfar = arrival_far(other);
-      if (side == 0 ? (sibfar <= ps || (int64_t)sibfar >= nc) : sibfar > ps) {  // cannot happen
-        atomicOr(status, kErrChain);
-        break;
-      }
-      const uint32_t sidx = side == 0 ? ps + 1u : ps;  // the sibling's index or leaf chunk
-      const bool sleaf = side == 0 ? sibfar == ps + 1u : sibfar == ps;
-      child_box(pts, n, leaf, nodes, sidx, sleaf, sib, sibmin);
-      if (side == 0) {
-        R = sibfar;
-        dr = arrival_delta(other);
-      } else {
-        L = sibfar;
-        dl = arrival_delta(other);
-      }
+    if (open) {
+      items.lo[out + rank] = item.lo;
+      items.hi[out + rank] = make_float4(item.hi.x, item.hi.y, item.hi.z, __uint_as_float(pos));
+      items.delta[out + rank] = delta;
     }
+    out += count;
+    if (!more) break;
+    if (open && rank == count - 1) {  // a fresh start after the last one
+      S.pos[0] = pos;
+      S.delta[0][0] = delta;
+    }
+    have = 0;
+  }
+  if (i == 0) {
+    counts[blockIdx.x] = (uint32_t)(out - first);
+    if (last_cta && out - first != 1) atomicOr(status, kErrChain);  // cannot happen: the root is built
   }
 }
 
 void launch_build_tree(Problem &P) {
-  // A listed split has both children inside CTAs of k_build_local but lies at
-  // the edge of one, so it is the boundary between two: fewer listed splits
-  // than k_build_local has CTAs, so n / 4 entries are room enough.  list_buf[1]
-  // (n words) is free until the rounds.
-  uint4 *ready = reinterpret_cast<uint4 *>(P.list_buf[1]);
-  const uint32_t capacity = (uint32_t)(P.n / 4);
-  uint32_t *ready_count = P.counters + kRefitReadyCounter;
-  const int64_t ctas = grid_for(P.nc, kRefitBlock);
-  k_build_local<<<(unsigned)ctas, kRefitBlock, 0, P.stream>>>(
-      P.keys[0] /*sorted*/, P.code_hi, P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels, P.range,
-      P.arrivals, ready, ready_count, capacity, P.counters + 1);
-  int64_t g = ctas / kRefitUpBlock + 1;
-  if (g > (int64_t)sm_count() * 16) g = (int64_t)sm_count() * 16;
-  k_build_up<<<(unsigned)g, kRefitUpBlock, 0, P.stream>>>(P.pts, P.n, P.nc, P.leaf, P.nodes, P.nlabels,
-                                                          P.range, P.arrivals, ready, ready_count,
-                                                          capacity, P.counters + 1);
-  P.launches += 2;
+  // The items lie in arrays that the rounds set up later (16, 16 and 4 bytes
+  // per point), their counts in list_buf[1] (n words; a count per CTA of each launch).
+  const TreeOut T = {P.nodes, P.nlabels, P.range, P.n, P.nc, P.leaf};
+  const Items items = {reinterpret_cast<float4 *>(P.comp_buf[0]), reinterpret_cast<float4 *>(P.comp_buf[1]),
+                       reinterpret_cast<int *>(P.root)};
+  static bool attr_set[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 64 || !attr_set[dev]) {
+    cudaFuncSetAttribute(k_build_tile<kBuildTile>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(BuildTables<kBuildTile>));
+    cudaFuncSetAttribute(k_build_merge<kMergeTile>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(BuildTables<kMergeTile>));
+    cudaFuncSetAttribute(k_build_merge<kLastTile>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(BuildTables<kLastTile>));
+    if (dev < 64) attr_set[dev] = true;
+  }
+  int64_t ctas = (P.nc + kBuildTile - 1) / kBuildTile, span = kBuildTile;
+  uint32_t *counts = P.list_buf[1];
+  k_build_tile<kBuildTile><<<(unsigned)ctas, kBuildTile, sizeof(BuildTables<kBuildTile>), P.stream>>>(
+      P.keys[0] /*sorted*/, P.code_hi, P.pts, T, items, counts, P.counters + 1);
+  P.launches += 1;
+  while (ctas > 1) {
+    // groups of 16 while that leaves CTAs for the whole GPU, larger ones
+    // (tables filled more than once per CTA) beyond that
+    const int group = ctas <= kMaxGroup ? (int)ctas : ctas > 16384 ? kMaxGroup : 16;
+    const int64_t next = (ctas + group - 1) / group;
+    if (next == 1)
+      k_build_merge<kLastTile><<<1, kLastTile, sizeof(BuildTables<kLastTile>), P.stream>>>(
+          P.keys[0], P.code_hi, T, items, span, group, ctas, counts, counts + ctas, P.counters + 1);
+    else
+      k_build_merge<kMergeTile><<<(unsigned)next, kMergeTile, sizeof(BuildTables<kMergeTile>), P.stream>>>(
+          P.keys[0], P.code_hi, T, items, span, group, ctas, counts, counts + ctas, P.counters + 1);
+    P.launches += 1;
+    counts += ctas;
+    ctas = next;
+    span *= group;
+  }
 }
 
 }  // namespace emst

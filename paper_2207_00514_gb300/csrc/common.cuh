@@ -260,7 +260,6 @@ struct Problem {
                                       // else nullptr; the sorted low words are keys[0]
   NodeRec *nodes = nullptr;       // nc-1 internal nodes
   uint2 *nlabels = nullptr;       // nc-1: child labels of each internal node (A5)
-  uint64_t *arrivals = nullptr;      // nc-1: per split of the build, the child that arrived first (0: none)
   uint2 *range = nullptr;            // nc-1: each internal node's leaf-chunk range [first, last]
                                      //      and split (the last chunk of its left child), packed
                                      //      by pack_range (one end of the range is the node itself)
@@ -323,7 +322,7 @@ void launch_gather(Problem &P, const uint32_t *perm);
 void launch_instance_ids(Problem &P);
 void launch_instance_roots(Problem &P);
 // A4: hierarchy, boxes, records, ranges and round-0 child labels in one
-// bottom-up pass (P.arrivals zeroed by launch_gather)
+// pass and its merges (uses comp_buf, root and list_buf[1])
 void launch_build_tree(Problem &P);
 // sort.cu
 int64_t sort_state_words(int64_t n);
