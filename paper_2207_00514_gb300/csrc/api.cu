@@ -193,6 +193,7 @@ size_t layout(Problem &P, char *base, bool copy_points, bool copy_edges) {
   P.nodes = c.take<NodeRec>(nc - 1);
   P.nlabels = c.take<uint2>(nc - 1);
   P.range = c.take<uint2>(nc - 1);
+  P.mixed = c.take<uint32_t>((nc - 1 + 31) / 32);
   P.runs = c.take<uint32_t>(n);
   P.scan_tiles = c.take<uint32_t>(2 * scan_tiles_for(n));
   P.labels_buf[0] = c.take<uint32_t>(n);

@@ -503,6 +503,7 @@ struct BuildTables {
 struct TreeOut {
   NodeRec *nodes;
   uint2 *nlabels, *range;
+  uint32_t *mixed;
   int64_t n, nc;
   int leaf;
 };
@@ -652,6 +653,8 @@ __global__ void __launch_bounds__(TILE) k_build_tile(const uint64_t *__restrict_
   Subtree item;
   int rank, count;
   const bool open = build_step<TILE, true>(S, N, (uint32_t)first, T, item, rank, count);
+  // every node still has its child labels to be rewritten (k_node_labels)
+  if (i < TILE / 32 && first + i * 32 < T.nc - 1) T.mixed[first / 32 + i] = 0xffffffffu;
   if (gridDim.x == 1) {
     if (i == 0 && count != 1) atomicOr(status, kErrChain);  // cannot happen: both ends are here
     return;
@@ -764,7 +767,7 @@ __global__ void __launch_bounds__(TILE) k_build_merge(const uint64_t *__restrict
 void launch_build_tree(Problem &P) {
   // The items lie in arrays that the rounds set up later (16, 16 and 4 bytes
   // per point), their counts in list_buf[1] (n words; a count per CTA of each launch).
-  const TreeOut T = {P.nodes, P.nlabels, P.range, P.n, P.nc, P.leaf};
+  const TreeOut T = {P.nodes, P.nlabels, P.range, P.mixed, P.n, P.nc, P.leaf};
   const Items items = {reinterpret_cast<float4 *>(P.comp_buf[0]), reinterpret_cast<float4 *>(P.comp_buf[1]),
                        reinterpret_cast<int *>(P.root)};
   static bool attr_set[64] = {false};

@@ -263,6 +263,7 @@ struct Problem {
   uint2 *range = nullptr;            // nc-1: each internal node's leaf-chunk range [first, last]
                                      //      and split (the last chunk of its left child), packed
                                      //      by pack_range (one end of the range is the node itself)
+  uint32_t *mixed = nullptr;         // bit per node: its child labels may still change (k_node_labels)
   uint32_t *runs = nullptr;          // n: per 32 curve positions, the bitmap of their label
                                      //    boundaries and the count of boundaries before them
                                      //    within their scan tile (plus the tile's entry of

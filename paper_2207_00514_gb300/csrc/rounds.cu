@@ -9,6 +9,12 @@
 namespace emst {
 
 constexpr int kBlock = 256;
+// From here on a round's passes over all points are bound by bandwidth and by
+// atomics on a few addresses, below by the latency of one wave: k_node_labels
+// with four words per warp and k_runs looking before its atomics take 1.01 ms
+// off a 37M call (35.17 -> 34.17) and add 30 us at 1M (1,592 -> 1,622); at 3M
+// they take 10 us off (4,101 -> 4,091).
+constexpr int64_t kManyPoints = 2500000;
 // P.counters slots of a round, cleared by its first kernel (k_node_labels) or
 // by the last CTA that counts in them: no memset between the kernels.
 constexpr uint32_t kActiveCounter = 50;  // listed queries
@@ -142,9 +148,9 @@ __global__ void __launch_bounds__(kScanThreads, EMST_SCAN_MIN_BLOCKS) k_runs(
     const uint32_t *__restrict__ labels_old, const uint32_t *__restrict__ root,
     const float4 *__restrict__ pts, const uint32_t *__restrict__ inst_of,
     const float *__restrict__ core2, int64_t n,
-    uint32_t *__restrict__ labels_new, uint32_t *__restrict__ bound_next,
+    uint32_t *__restrict__ labels_new, uint32_t *bound_next,
     uint2 *__restrict__ words, uint32_t *tile_total, uint32_t *tile_prefix, uint32_t *done,
-    const uint32_t *counters, uint32_t *mail, uint32_t mail_seq) {
+    const uint32_t *counters, uint32_t *mail, uint32_t mail_seq, bool look) {
   __shared__ uint32_t s_warp[kScanThreads / 32];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -186,8 +192,10 @@ __global__ void __launch_bounds__(kScanThreads, EMST_SCAN_MIN_BLOCKS) k_runs(
         // (no bound across instances)
         const float4 p = __ldg(pts + seg + k), r = __ldg(pts + seg + k + 1);
         const uint32_t w = __float_as_uint(pair_weight(p, r, core2, seg + k));
-        atomicMin(&bound_next[lab[q]], w);
-        atomicMin(&bound_next[nxt], w);
+        // look: a bound only falls, so one read at or below w, however old,
+        // stands (in the late rounds every boundary lowers one of a few)
+        if (!look || w < bound_next[lab[q]]) atomicMin(&bound_next[lab[q]], w);
+        if (!look || w < bound_next[nxt]) atomicMin(&bound_next[nxt], w);
       }
     }
     if (RELABEL && k < rem) labels_new[seg + k] = lab[q];
@@ -236,49 +244,84 @@ static void launch_runs(Problem &P, bool relabel) {
   if (relabel)
     k_runs<true><<<(unsigned)tiles, kScanThreads, 0, P.stream>>>(
         P.labels, P.root, P.pts, P.inst_of, P.core2, P.n, P.labels_buf[P.cur ^ 1],
-        P.bound_buf[P.cur ^ 1], words, tile_total, tile_prefix, done, P.counters, P.mail, P.mail_seq);
+        P.bound_buf[P.cur ^ 1], words, tile_total, tile_prefix, done, P.counters, P.mail, P.mail_seq,
+        P.n >= kManyPoints);
   else
     k_runs<false><<<(unsigned)tiles, kScanThreads, 0, P.stream>>>(
         P.labels, nullptr, P.pts, P.inst_of, nullptr, P.n, nullptr, nullptr, words, tile_total,
-        tile_prefix, done, nullptr, nullptr, 0u);
+        tile_prefix, done, nullptr, nullptr, 0u, false);
   P.launches += 1;
 }
 
 void launch_label_runs(Problem &P) { launch_runs(P, false); }
 
+// A node whose leaves share one component keeps sharing it, so its own entry
+// (its children's labels) is final: from then on searches either stop above it
+// (its label, in its parent's entry, is the query's) or may enter it as a
+// whole, and the old label X in its entry is not the query's either (labels
+// are names of components that merged; X's went into the component the node
+// now belongs to, and no other component can carry that name again).  So a
+// round only writes the nodes that held several components before it: a bit
+// per node says which (all set by the build), cleared when the last two
+// merge.  (37M halos: 2.13 -> 1.35 ms over the ten rounds.)
+// WORDS: words of them a warp takes (kManyPoints).
+template <int WORDS>
 __global__ void __launch_bounds__(kBlock) k_node_labels(const uint32_t *__restrict__ labels,
                                                         const uint2 *__restrict__ words,
                                                         const uint32_t *__restrict__ tile_prefix,
                                                         const uint2 *__restrict__ range,
                                                         int64_t n, int64_t nc, int leaf,
+                                                        uint32_t *__restrict__ mixed,
                                                         uint2 *__restrict__ nlabels,
                                                         uint32_t *counters) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) {  // the round's counters (the first kernel of a round)
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  if (t == 0) {  // the round's counters (the first kernel of a round)
     counters[40] = counters[12];      // components listed by the previous merge
     counters[12] = 0u;
     counters[kActiveCounter] = 0u;
     counters[kActiveQueue] = 0u;
   }
-  if (i >= nc - 1) return;
-  // the children split the node's chunk range [first, last] after `split`
-  const NodeRange r = unpack_range((uint32_t)i, __ldg(range + i));
-  const int64_t a0 = (int64_t)r.first * leaf;
-  const int64_t b0 = ((int64_t)r.split + 1) * leaf - 1;
-  const int64_t a1 = b0 + 1;
-  const int64_t b1 = ((int64_t)r.last + 1) * leaf < n ? ((int64_t)r.last + 1) * leaf - 1 : n - 1;
-  const uint32_t l0 = __ldg(labels + a0), l1 = __ldg(labels + a1);
-  const uint32_t lab0 =
-      runs_at(words, tile_prefix, b0) == runs_at(words, tile_prefix, a0) ? l0 : kInvalid;
-  const uint32_t lab1 =
-      runs_at(words, tile_prefix, b1) == runs_at(words, tile_prefix, a1) ? l1 : kInvalid;
-  nlabels[i] = make_uint2(lab0, lab1);
+  const int64_t w0 = (t >> 5) * WORDS;
+  const int64_t word_count = (nc - 1 + 31) >> 5;
+  uint32_t mine = 0u;
+  if (lane < WORDS && w0 + lane < word_count) mine = mixed[w0 + lane];
+#pragma unroll
+  for (int q = 0; q < WORDS; ++q) {
+    const uint32_t word = __shfl_sync(0xffffffffu, mine, q);
+    if (word == 0u) continue;
+    const int64_t i = (w0 + q) * 32 + lane;
+    bool several = false;
+    if (i < nc - 1 && ((word >> lane) & 1u)) {
+      // the children split the node's chunk range [first, last] after `split`
+      const NodeRange r = unpack_range((uint32_t)i, __ldg(range + i));
+      const int64_t a0 = (int64_t)r.first * leaf;
+      const int64_t b0 = ((int64_t)r.split + 1) * leaf - 1;
+      const int64_t a1 = b0 + 1;
+      const int64_t b1 = ((int64_t)r.last + 1) * leaf < n ? ((int64_t)r.last + 1) * leaf - 1 : n - 1;
+      const uint32_t l0 = __ldg(labels + a0), l1 = __ldg(labels + a1);
+      const uint32_t lab0 =
+          runs_at(words, tile_prefix, b0) == runs_at(words, tile_prefix, a0) ? l0 : kInvalid;
+      const uint32_t lab1 =
+          runs_at(words, tile_prefix, b1) == runs_at(words, tile_prefix, a1) ? l1 : kInvalid;
+      nlabels[i] = make_uint2(lab0, lab1);
+      several = lab0 != lab1 || lab0 == kInvalid;
+    }
+    const uint32_t left = __ballot_sync(0xffffffffu, several);
+    if (lane == 0 && left != word) mixed[w0 + q] = left;
+  }
 }
 
 void launch_node_labels(Problem &P) {
-  k_node_labels<<<grid_for(P.nc - 1, kBlock), kBlock, 0, P.stream>>>(
-      P.labels, reinterpret_cast<const uint2 *>(P.runs), P.scan_tiles + scan_tiles_for(P.n), P.range,
-      P.n, P.nc, P.leaf, P.nlabels, P.counters);
+  const int64_t nodes = P.nc - 1;
+  const uint2 *words = reinterpret_cast<const uint2 *>(P.runs);
+  const uint32_t *prefix = P.scan_tiles + scan_tiles_for(P.n);
+  if (nodes >= kManyPoints)
+    k_node_labels<4><<<grid_for((nodes + 3) / 4, kBlock), kBlock, 0, P.stream>>>(
+        P.labels, words, prefix, P.range, P.n, P.nc, P.leaf, P.mixed, P.nlabels, P.counters);
+  else
+    k_node_labels<1><<<grid_for(nodes, kBlock), kBlock, 0, P.stream>>>(
+        P.labels, words, prefix, P.range, P.n, P.nc, P.leaf, P.mixed, P.nlabels, P.counters);
   P.launches += 1;
 }
 
