@@ -273,7 +273,7 @@ int bits_for(int64_t v) {  // bits needed to represent values in [0, v]
 // A2-A4 (a): codes, their stable order, the points gathered into it.
 static void build_order64(Problem &P) {
   launch_morton(P);
-  const int src = radix_sort_pairs(P, P.n, 0, 8, 0);
+  const int src = radix_sort_pairs(P, P.n, 0, 8, 0, 0, true);
   if (src != 0) {  // keep the sorted codes in keys[0] and the order in vals[0]
     std::swap(P.keys[0], P.keys[1]);
     std::swap(P.vals[0], P.vals[1]);
@@ -287,7 +287,7 @@ static void build_order64(Problem &P) {
 // the high words carrying that order; the low words follow the final order.
 static void build_order128(Problem &P) {
   launch_morton128(P);
-  const int s = radix_sort_pairs(P, P.n, 0, 8, 0);
+  const int s = radix_sort_pairs(P, P.n, 0, 8, 0, 0, true);
   launch_gather_u64(P, P.wide_hi, P.vals[s], P.keys[s ^ 1]);
   cudaMemcpyAsync(P.vals[s ^ 1], P.vals[s], sizeof(uint32_t) * (size_t)P.n,
                   cudaMemcpyDeviceToDevice, P.stream);
@@ -316,7 +316,15 @@ bool run_build(Problem &P, uint32_t *counters) {
     build_order128(P);
   } else {
     build_order64(P);
-    if (P.auto_wide && read_counters(P, counters)) {
+    // the tree follows at once, and the counters travel meanwhile
+    const bool ahead = P.auto_wide && P.mail && P.n >= 2;
+    if (ahead) {
+      P.mail_seq = ++t_mailbox.seq;
+      launch_post_mail(P);
+      launch_build_tree(P, true);
+    }
+    if (ahead ? cudaPeekAtLastError() == cudaSuccess && wait_mail(P, counters)
+              : P.auto_wide && read_counters(P, counters)) {
       P.code_collisions = (int64_t)counters[30] | ((int64_t)counters[31] << 32);
       known = true;
       if (counters[1] != 0) return known;
@@ -324,6 +332,8 @@ bool run_build(Problem &P, uint32_t *counters) {
         P.wide = true;
         build_order128(P);
         known = false;
+      } else if (ahead) {
+        return known;
       }
     }
   }
@@ -518,7 +528,7 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits, uint32_t *counters) 
   // a run is long (a lattice, many equal distances), then the next path
   if (P.num_inst == 1 && !P.ties && wb > 0) {
     launch_edge_keys_wi(P, m, L);
-    const int s = radix_sort_pairs(P, m, 0, (wb + 7) / 8, 0, L);
+    const int s = radix_sort_pairs(P, m, 0, (wb + 7) / 8, 0, L, true);
     // (the count of long runs is zero since the call's first kernel; the
     // edges are written without waiting for it, and again below if need be)
     launch_edge_ties_w(P, m, s, L);
@@ -536,8 +546,7 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits, uint32_t *counters) 
       launch_edge_keys_inst_wi(P, m, wb + Lloc, Lloc);
       digits = (P.inst_bits + wb + Lloc + 7) / 8;
     }
-    const int s = radix_sort_pairs(P, m, 0, digits, 0);
-    cudaMemsetAsync(P.counters + 10, 0, sizeof(uint32_t), P.stream);
+    const int s = radix_sort_pairs(P, m, 0, digits, 0, 0, true);
     launch_edge_ties(P, m, s);
     launch_edge_from_keys(P, m, s, Lloc, wb, out);
     uint32_t long_runs = 0;
@@ -546,7 +555,7 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits, uint32_t *counters) 
   }
   // full path: stable by j, then by (w, i), then (batched) by instance
   launch_edge_keys_j(P, m);
-  int s = radix_sort_pairs(P, m, 0, (L + 7) / 8, 0);
+  int s = radix_sort_pairs(P, m, 0, (L + 7) / 8, 0, 0, true);
   launch_edge_keys_wi_of(P, m, s, L);
   s = radix_sort_pairs(P, m, 0, (L + wb + 7) / 8, s);
   if (P.num_inst > 1) {
@@ -774,12 +783,14 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     // components of every unfinished instance, so more than ceil(log2 n)
     // rounds (n: the largest instance) means something is wrong.
     const int limit = bits_for(largest - 1) + 1;
+    const bool ahead = P.mail && use_graph != 1;  // (the counters are posted before the next round starts)
+    P.stop_at = (uint32_t)expected;
     for (rounds = 0;; ++rounds) {
       if (rounds >= limit) { rc = EMST_ERR_ROUND_LIMIT; goto done; }
       if (stats && rounds < 40)
         stats->components_per_round[rounds] = n - (int64_t)host_counters[0];
-      if (rounds > 0) launch_node_labels(P);
-      else if (!P.near_j) launch_upper_bounds(P);
+      if (rounds > 0 && !ahead) launch_node_labels(P);
+      else if (rounds == 0 && !P.near_j) launch_upper_bounds(P);
       if (learned || logging) launch_comp_sizes(P);
       if (logging) launch_log_samples(P, rounds, rounds > 0 && carried);
       if (stats && rounds < 40) {
@@ -812,6 +823,11 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
       if (count) launch_count_seen(P);
       if (P.mail) P.mail_seq = ++t_mailbox.seq;  // posted by the merge's last kernel
       launch_merge(P);
+      advance_round(P, 0);
+      // the next round's first kernel, before this one's outcome is known: the
+      // GPU has work while the counters travel (it ends at once, or does no
+      // harm, when this was the last round)
+      if (ahead) launch_node_labels(P);
       CU(cudaPeekAtLastError());  // a launch that failed must not read as a round without edges
       if (P.mail ? !wait_mail(P, host_counters) : !read_counters(P, host_counters)) {
         rc = EMST_ERR_CUDA;
@@ -828,7 +844,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
         prev_queries = u64(34);
         prev_distinct = u64(38);
       }
-      advance_round(P, (int64_t)host_counters[12]);
+      P.n_active = (int64_t)host_counters[12];
       if ((int64_t)host_counters[0] >= expected) { ++rounds; break; }
       if (rounds == 0 && use_graph == 1 && !learned && !logging && !count) {
         // the remaining rounds as one graph ended on the device
@@ -860,7 +876,8 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     tm.mark(2, stream);
   }
   tm.mark(3, stream);
-  CU(cudaStreamSynchronize(stream));
+  // (the output's last kernel has posted: everything before it is complete)
+  if (!P.mail || expected == 0 || skip_output || !(out_dev || out_map)) CU(cudaStreamSynchronize(stream));
   CU(cudaGetLastError());
   rc = status_from_bits(host_counters[1]);
   if (logging && ex->log_count_out) {

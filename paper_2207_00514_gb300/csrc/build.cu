@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(kBlock) k_scene_box(const float *__restrict__ 
                                                       uint32_t *__restrict__ box,
                                                       uint32_t *__restrict__ status,
                                                       float *__restrict__ copy) {
+  wait_for_previous();
   float lo[3] = {INFINITY, INFINITY, INFINITY};
   float hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool bad = false;
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(kBlock) k_scene_box_copy4(const float4 *__rest
                                                             uint32_t *__restrict__ box,
                                                             uint32_t *__restrict__ status,
                                                             float4 *__restrict__ copy) {
+  wait_for_previous();
   float lo[3] = {INFINITY, INFINITY, INFINITY};
   float hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool bad = false;
@@ -153,18 +155,18 @@ void launch_scene_box(Problem &P) {
     const float4 *src = reinterpret_cast<const float4 *>(P.points_mapped);
     float4 *dst = reinterpret_cast<float4 *>(copy);
     if (P.dim == 3)
-      k_scene_box_copy4<3><<<g4, kBlock, 0, P.stream>>>(src, nv, tail, box, P.counters + 1, dst);
+      launch_next(P, k_scene_box_copy4<3>, g4, kBlock, 0, src, nv, tail, box, P.counters + 1, dst);
     else
-      k_scene_box_copy4<2><<<g4, kBlock, 0, P.stream>>>(src, nv, tail, box, P.counters + 1, dst);
+      launch_next(P, k_scene_box_copy4<2>, g4, kBlock, 0, src, nv, tail, box, P.counters + 1, dst);
   } else if (P.points_mapped) {  // read the host input through its mapping, keep a device copy
     if (P.dim == 3)
-      k_scene_box<3, true><<<grid, kBlock, 0, P.stream>>>(P.points_mapped, P.n, box, P.counters + 1, copy);
+      launch_next(P, k_scene_box<3, true>, grid, kBlock, 0, P.points_mapped, P.n, box, P.counters + 1, copy);
     else
-      k_scene_box<2, true><<<grid, kBlock, 0, P.stream>>>(P.points_mapped, P.n, box, P.counters + 1, copy);
+      launch_next(P, k_scene_box<2, true>, grid, kBlock, 0, P.points_mapped, P.n, box, P.counters + 1, copy);
   } else if (P.dim == 3) {
-    k_scene_box<3, false><<<grid, kBlock, 0, P.stream>>>(P.points, P.n, box, P.counters + 1, nullptr);
+    launch_next(P, k_scene_box<3, false>, grid, kBlock, 0, P.points, P.n, box, P.counters + 1, nullptr);
   } else {
-    k_scene_box<2, false><<<grid, kBlock, 0, P.stream>>>(P.points, P.n, box, P.counters + 1, nullptr);
+    launch_next(P, k_scene_box<2, false>, grid, kBlock, 0, P.points, P.n, box, P.counters + 1, nullptr);
   }
   P.launches += 2;
 }
@@ -183,7 +185,9 @@ __global__ void __launch_bounds__(kBlock) k_morton(const float *__restrict__ pts
                                                    const uint32_t *__restrict__ box,
                                                    const uint32_t *__restrict__ inst_in, int bits,
                                                    uint64_t *__restrict__ keys,
-                                                   uint32_t *__restrict__ vals) {
+                                                   uint32_t *__restrict__ vals, ClearWords clear) {
+  wait_for_previous();
+  clear_words(clear);
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const Quantizer Q = make_quantizer(box, DIM, bits);
@@ -197,14 +201,15 @@ __global__ void __launch_bounds__(kBlock) k_morton(const float *__restrict__ pts
 }
 
 void launch_morton(Problem &P) {
+  const ClearWords clear = {P.sort_state, sort_clear_words(P.n)};
   int g = grid_for(P.n, kBlock);
   const int bits = code_bits(P.dim, P.inst_bits);
   if (P.dim == 3)
-    k_morton<3><<<g, kBlock, 0, P.stream>>>(P.points, P.n, P.counters + 4, P.inst_in, bits,
-                                            P.keys[0], P.vals[0]);
+    launch_next(P, k_morton<3>, g, kBlock, 0, P.points, P.n, P.counters + 4, P.inst_in, bits,
+                                            P.keys[0], P.vals[0], clear);
   else
-    k_morton<2><<<g, kBlock, 0, P.stream>>>(P.points, P.n, P.counters + 4, P.inst_in, bits,
-                                            P.keys[0], P.vals[0]);
+    launch_next(P, k_morton<2>, g, kBlock, 0, P.points, P.n, P.counters + 4, P.inst_in, bits,
+                                            P.keys[0], P.vals[0], clear);
   P.launches += 1;
 }
 
@@ -222,7 +227,9 @@ __global__ void __launch_bounds__(kBlock) k_morton128(const float *__restrict__ 
                                                       uint64_t *__restrict__ code_hi,
                                                       uint64_t *__restrict__ code_lo,
                                                       uint64_t *__restrict__ keys,
-                                                      uint32_t *__restrict__ vals) {
+                                                      uint32_t *__restrict__ vals, ClearWords clear) {
+  wait_for_previous();
+  clear_words(clear);
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   constexpr int B = DIM == 3 ? 42 : 64;
@@ -256,25 +263,27 @@ __global__ void __launch_bounds__(kBlock) k_morton128(const float *__restrict__ 
 }
 
 void launch_morton128(Problem &P) {
+  const ClearWords clear = {P.sort_state, sort_clear_words(P.n)};
   int g = grid_for(P.n, kBlock);
   if (P.dim == 3)
-    k_morton128<3><<<g, kBlock, 0, P.stream>>>(P.points, P.n, P.counters + 4, P.wide_hi, P.wide_lo,
-                                               P.keys[0], P.vals[0]);
+    launch_next(P, k_morton128<3>, g, kBlock, 0, P.points, P.n, P.counters + 4, P.wide_hi, P.wide_lo,
+                                               P.keys[0], P.vals[0], clear);
   else
-    k_morton128<2><<<g, kBlock, 0, P.stream>>>(P.points, P.n, P.counters + 4, P.wide_hi, P.wide_lo,
-                                               P.keys[0], P.vals[0]);
+    launch_next(P, k_morton128<2>, g, kBlock, 0, P.points, P.n, P.counters + 4, P.wide_hi, P.wide_lo,
+                                               P.keys[0], P.vals[0], clear);
   P.launches += 1;
 }
 
 // out[k] = src[idx[k]] (a 64-bit word carried through a permutation)
 __global__ void k_gather_u64(const uint64_t *__restrict__ src, const uint32_t *__restrict__ idx,
                              int64_t n, uint64_t *__restrict__ out) {
+  wait_for_previous();
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) out[k] = __ldg(src + __ldg(idx + k));
 }
 
 void launch_gather_u64(Problem &P, const uint64_t *src, const uint32_t *idx, uint64_t *out) {
-  k_gather_u64<<<grid_for(P.n, kBlock), kBlock, 0, P.stream>>>(src, idx, P.n, out);
+  launch_next(P, k_gather_u64, grid_for(P.n, kBlock), kBlock, 0, src, idx, P.n, out);
   P.launches += 1;
 }
 
@@ -282,6 +291,7 @@ void launch_gather_u64(Problem &P, const uint64_t *src, const uint32_t *idx, uin
 __global__ void __launch_bounds__(kBlock) k_instance_ids(const int64_t *__restrict__ offsets,
                                                          int64_t num_inst, int64_t n,
                                                          uint32_t *__restrict__ inst_in) {
+  wait_for_previous();
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   int64_t lo = 0, hi = num_inst - 1;  // last instance whose start is <= k
@@ -293,7 +303,7 @@ __global__ void __launch_bounds__(kBlock) k_instance_ids(const int64_t *__restri
 }
 
 void launch_instance_ids(Problem &P) {
-  k_instance_ids<<<grid_for(P.n, kBlock), kBlock, 0, P.stream>>>(P.offsets, P.num_inst, P.n,
+  launch_next(P, k_instance_ids, grid_for(P.n, kBlock), kBlock, 0, P.offsets, P.num_inst, P.n,
                                                                  P.inst_in);
   P.launches += 1;
 }
@@ -306,6 +316,7 @@ __global__ void __launch_bounds__(kBlock) k_instance_roots(const int64_t *__rest
                                                            const uint2 *__restrict__ range,
                                                            uint32_t *__restrict__ inst_root,
                                                            uint32_t *status) {
+  wait_for_previous();
   int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (I >= num_inst) return;
   const int64_t a = __ldg(offsets + I), b = __ldg(offsets + I + 1) - 1;
@@ -329,8 +340,7 @@ __global__ void __launch_bounds__(kBlock) k_instance_roots(const int64_t *__rest
 }
 
 void launch_instance_roots(Problem &P) {
-  k_instance_roots<<<grid_for(P.num_inst, kBlock), kBlock, 0, P.stream>>>(
-      P.offsets, P.num_inst, P.nc, P.leaf, P.range, P.inst_root, P.counters + 1);
+  launch_next(P, k_instance_roots, grid_for(P.num_inst, kBlock), kBlock, 0, P.offsets, P.num_inst, P.nc, P.leaf, P.range, P.inst_root, P.counters + 1);
   P.launches += 1;
 }
 
@@ -355,6 +365,7 @@ __global__ void __launch_bounds__(kBlock) k_gather(const float *__restrict__ pts
                                                    const uint64_t *__restrict__ sorted_codes,
                                                    const uint64_t *__restrict__ code_hi,
                                                    unsigned long long *dup) {
+  wait_for_previous();
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   uint32_t o = __ldg(perm + k);
@@ -389,10 +400,10 @@ void launch_gather(Problem &P, const uint32_t *perm) {
   // (zero since the call's first kernel, unless the order is rebuilt)
   if (P.wide) cudaMemsetAsync(dup, 0, 3 * sizeof(unsigned long long), P.stream);
   if (P.dim == 3)
-    k_gather<3><<<g, kBlock, 0, P.stream>>>(P.points, perm, P.n, P.pts, P.labels, P.inst_in,
+    launch_next(P, k_gather<3>, g, kBlock, 0, P.points, perm, P.n, P.pts, P.labels, P.inst_in,
                                             P.inst_of, P.keys[0], P.code_hi, dup);
   else
-    k_gather<2><<<g, kBlock, 0, P.stream>>>(P.points, perm, P.n, P.pts, P.labels, P.inst_in,
+    launch_next(P, k_gather<2>, g, kBlock, 0, P.points, perm, P.n, P.pts, P.labels, P.inst_in,
                                             P.inst_of, P.keys[0], P.code_hi, dup);
   P.launches += 1;
 }
@@ -501,12 +512,19 @@ struct BuildTables {
 };
 
 struct TreeOut {
+  // not null: nothing to build when more than n / 64 codes collide (the host
+  // is about to find the same count and starts over with 128-bit codes)
+  const unsigned long long *collisions;
   NodeRec *nodes;
   uint2 *nlabels, *range;
   uint32_t *mixed;
   int64_t n, nc;
   int leaf;
 };
+
+__device__ __forceinline__ bool abandoned(const TreeOut &T) {
+  return T.collisions && __ldcg(T.collisions) * 64ull > (unsigned long long)T.n;
+}
 
 // Node `idx` covering chunks [L, R] with split g and children's boxes a, b:
 // its record, range and round-0 child labels.
@@ -637,6 +655,8 @@ __global__ void __launch_bounds__(TILE) k_build_tile(const uint64_t *__restrict_
                                                      const uint64_t *__restrict__ keys_hi,
                                                      const float4 *__restrict__ pts, TreeOut T, Items items,
                                                      uint32_t *__restrict__ counts, uint32_t *status) {
+  wait_for_previous();
+  if (abandoned(T)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BuildTables<TILE> &S = *reinterpret_cast<BuildTables<TILE> *>(smem_raw);
   const int i = threadIdx.x;
@@ -676,6 +696,8 @@ __global__ void __launch_bounds__(TILE) k_build_merge(const uint64_t *__restrict
                                                       int64_t span, int group, int64_t ctas_in,
                                                       const uint32_t *__restrict__ counts_in,
                                                       uint32_t *__restrict__ counts, uint32_t *status) {
+  wait_for_previous();
+  if (abandoned(T)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BuildTables<TILE> &S = *reinterpret_cast<BuildTables<TILE> *>(smem_raw);
   const int i = threadIdx.x;
@@ -764,10 +786,12 @@ __global__ void __launch_bounds__(TILE) k_build_merge(const uint64_t *__restrict
   }
 }
 
-void launch_build_tree(Problem &P) {
+void launch_build_tree(Problem &P, bool unless_colliding) {
   // The items lie in arrays that the rounds set up later (16, 16 and 4 bytes
   // per point), their counts in list_buf[1] (n words; a count per CTA of each launch).
-  const TreeOut T = {P.nodes, P.nlabels, P.range, P.mixed, P.n, P.nc, P.leaf};
+  const unsigned long long *collisions =
+      unless_colliding ? reinterpret_cast<const unsigned long long *>(P.counters + 30) : nullptr;
+  const TreeOut T = {collisions, P.nodes, P.nlabels, P.range, P.mixed, P.n, P.nc, P.leaf};
   const Items items = {reinterpret_cast<float4 *>(P.comp_buf[0]), reinterpret_cast<float4 *>(P.comp_buf[1]),
                        reinterpret_cast<int *>(P.root)};
   static bool attr_set[64] = {false};
@@ -784,8 +808,7 @@ void launch_build_tree(Problem &P) {
   }
   int64_t ctas = (P.nc + kBuildTile - 1) / kBuildTile, span = kBuildTile;
   uint32_t *counts = P.list_buf[1];
-  k_build_tile<kBuildTile><<<(unsigned)ctas, kBuildTile, sizeof(BuildTables<kBuildTile>), P.stream>>>(
-      P.keys[0] /*sorted*/, P.code_hi, P.pts, T, items, counts, P.counters + 1);
+  launch_next(P, k_build_tile<kBuildTile>, (unsigned)ctas, kBuildTile, sizeof(BuildTables<kBuildTile>), P.keys[0] /*sorted*/, P.code_hi, P.pts, T, items, counts, P.counters + 1);
   P.launches += 1;
   while (ctas > 1) {
     // groups of 16 while that leaves CTAs for the whole GPU, larger ones
@@ -793,11 +816,9 @@ void launch_build_tree(Problem &P) {
     const int group = ctas <= kMaxGroup ? (int)ctas : ctas > 16384 ? kMaxGroup : 16;
     const int64_t next = (ctas + group - 1) / group;
     if (next == 1)
-      k_build_merge<kLastTile><<<1, kLastTile, sizeof(BuildTables<kLastTile>), P.stream>>>(
-          P.keys[0], P.code_hi, T, items, span, group, ctas, counts, counts + ctas, P.counters + 1);
+      launch_next(P, k_build_merge<kLastTile>, 1, kLastTile, sizeof(BuildTables<kLastTile>), P.keys[0], P.code_hi, T, items, span, group, ctas, counts, counts + ctas, P.counters + 1);
     else
-      k_build_merge<kMergeTile><<<(unsigned)next, kMergeTile, sizeof(BuildTables<kMergeTile>), P.stream>>>(
-          P.keys[0], P.code_hi, T, items, span, group, ctas, counts, counts + ctas, P.counters + 1);
+      launch_next(P, k_build_merge<kMergeTile>, (unsigned)next, kMergeTile, sizeof(BuildTables<kMergeTile>), P.keys[0], P.code_hi, T, items, span, group, ctas, counts, counts + ctas, P.counters + 1);
     P.launches += 1;
     counts += ctas;
     ctas = next;

@@ -279,6 +279,7 @@ struct Problem {
   uint32_t *active_list = nullptr;   // this round's active labels (nullptr: all n)
   uint32_t *next_list = nullptr;     // roots appended by the merge
   int64_t n_active = 0;
+  uint32_t stop_at = 0xFFFFFFFFu;    // edges at which no further round is needed
   uint2 *res = nullptr;              // n: (w bits, neighbour curve index)
   float *core2 = nullptr;            // n: mutual reachability -- squared core distances in
                                      //    curve order (nullptr: the Euclidean weight)
@@ -310,6 +311,45 @@ struct Problem {
 };
 
 // ---------------------------------------------------------------------------
+// Chained launches.  A call is a chain of many short kernels; started in plain
+// stream order each waits for the one before it to drain, and then for its own
+// launch: 2.5 us a kernel on this GPU.  launch_next lets the kernel start as
+// soon as the CTAs of the one before have ended, and the kernel itself waits,
+// as its first step and before it touches global memory, until that kernel's
+// writes are complete (which includes all earlier kernels, since each waits).
+// (With an early trigger in the kernel before, its successors' CTAs take SM
+// slots while they wait: a sort of 200,000 keys took 85 us instead of 77;
+// without chaining 97.)  Every kernel launched so calls wait_for_previous.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... KArgs, class... Args>
+inline void launch_next(const Problem &P, void (*kernel)(KArgs...), int64_t grid, int block, size_t smem,
+                        Args... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = smem;
+  c.stream = P.stream;
+  cudaLaunchAttribute chained;
+  chained.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  chained.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &chained;
+  c.numAttrs = P.graph_round ? 0 : 1;  // (a captured loop body takes plain edges)
+  cudaLaunchKernelEx(&c, kernel, static_cast<KArgs>(args)...);
+}
+
+// `words` words at p cleared by the whole grid.
+struct ClearWords {
+  uint32_t *p;
+  int64_t words;
+};
+__device__ __forceinline__ void clear_words(const ClearWords &c) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < c.words; t += (int64_t)gridDim.x * blockDim.x)
+    c.p[t] = 0u;
+}
+
+// ---------------------------------------------------------------------------
 // Launchers (host side), one per kernel family.
 // ---------------------------------------------------------------------------
 // build.cu
@@ -324,7 +364,8 @@ void launch_instance_ids(Problem &P);
 void launch_instance_roots(Problem &P);
 // A4: hierarchy, boxes, records, ranges and round-0 child labels in one
 // pass and its merges (uses comp_buf, root and list_buf[1])
-void launch_build_tree(Problem &P);
+// unless_colliding: not if more than n / 64 codes collide (counters[30..31])
+void launch_build_tree(Problem &P, bool unless_colliding = false);
 // sort.cu
 int64_t sort_state_words(int64_t n);
 // Stable LSD radix sort of (keys, vals) pairs on digits [digit_begin, digit_end)
@@ -332,7 +373,11 @@ int64_t sort_state_words(int64_t n);
 // Stable sort of (keys[src], vals[src]) by the bits [bit0 + 8 digit_begin,
 // bit0 + 8 digit_end) of the keys (digit d of the key >> bit0 per pass);
 // returns the buffer index holding the result.
-int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0 = 0);
+// cleared: the first sort_clear_words(n) words of P.sort_state are zero (the
+// kernel that made the keys cleared them, see clear_words), else a memset.
+int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0 = 0,
+                     bool cleared = false);
+int64_t sort_clear_words(int64_t n);
 // rounds.cu
 #ifndef EMST_TRAVERSE_MIN_BLOCKS
 #define EMST_TRAVERSE_MIN_BLOCKS 8      // resident 256-thread CTAs the traversal's registers must allow (32 registers: measured best)

@@ -174,6 +174,7 @@ struct Contract {
 // decreasing) and, in the same pass, every point's lowest slot.
 __global__ void k_dg_check(const emst_edge *__restrict__ e, int64_t m, int64_t n, uint2 *node,
                            uint32_t *__restrict__ uf, uint32_t *counters) {
+  wait_for_previous();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) uf[k] = (uint32_t)k;
   if (k >= m) return;
@@ -427,6 +428,7 @@ __device__ __forceinline__ Segment scan_segments(Segment s, Segment &before) {
 __global__ void __launch_bounds__(kDgBlock) k_dg_tiles(const uint64_t *__restrict__ keys,
                                                        const uint32_t *__restrict__ vals, int64_t m,
                                                        uint2 *__restrict__ tiles, const uint32_t *status) {
+  wait_for_previous();
   if (*status != 0u) return;
   uint64_t k[kScanItems + 1];
   uint32_t v[kScanItems], heads;
@@ -445,6 +447,7 @@ __global__ void __launch_bounds__(kDgBlock) k_dg_finish(const uint64_t *__restri
                                                         uint32_t *__restrict__ child,
                                                         uint32_t *__restrict__ out_parent,
                                                         const uint32_t *status) {
+  wait_for_previous();
   __shared__ uint32_t s_carry;
   if (*status != 0u) return;
   uint64_t k[kScanItems + 1];
@@ -486,6 +489,7 @@ __global__ void __launch_bounds__(kDgBlock) k_dg_finish(const uint64_t *__restri
 __global__ void k_dg_rows(const emst_edge *__restrict__ e, int64_t m,
                           const uint32_t *__restrict__ size_out, const uint2 *__restrict__ child,
                           uint4 *__restrict__ link, const uint32_t *status) {
+  wait_for_previous();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= m || *status != 0u) return;
   const uint2 c = child[k];
@@ -595,12 +599,11 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     const int src = radix_sort_pairs(P, m, 0, (bits_for(n - 1) + 7) / 8, 0, 32);
     uint2 *tile = reinterpret_cast<uint2 *>(base + o_tiles);
     uint32_t *size = link ? P.vals[src ^ 1] : nullptr;  // the sort's other buffer is free again
-    k_dg_tiles<<<(unsigned)tiles, kDgBlock, 0, s>>>(P.keys[src], P.vals[src], m, tile, status);
-    k_dg_finish<<<(unsigned)tiles, kDgBlock, 0, s>>>(P.keys[src], P.vals[src], m, n, tile, A.node, size,
+    launch_next(P, k_dg_tiles, (unsigned)tiles, kDgBlock, 0, P.keys[src], P.vals[src], m, tile, status);
+    launch_next(P, k_dg_finish, (unsigned)tiles, kDgBlock, 0, P.keys[src], P.vals[src], m, n, tile, A.node, size,
                                                      A.child, pout, status);
     if (link)
-      k_dg_rows<<<grid_for(m, kDgBlock), kDgBlock, 0, s>>>(
-          e, m, size, reinterpret_cast<const uint2 *>(A.child), link, status);
+      launch_next(P, k_dg_rows, grid_for(m, kDgBlock), kDgBlock, 0, e, m, size, reinterpret_cast<const uint2 *>(A.child), link, status);
     ok = cudaPeekAtLastError() == cudaSuccess;
     if (out_link && !link_dev)
       cudaMemcpyAsync(out_link, link, 16 * (size_t)m, cudaMemcpyDeviceToHost, s);

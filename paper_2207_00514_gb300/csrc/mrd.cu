@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(kCoreBlock) k_core_knn(const float4 *__restric
                                                          int64_t n, int leaf, int m,
                                                          float *__restrict__ core2,
                                                          uint32_t *status) {
+  wait_for_previous();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (m == 0) {
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(kCoreBlock) k_core_knn(const float4 *__restric
 // Curve order -> the caller's order (the original index rides in pts.w).
 __global__ void k_core_to_input(const float4 *__restrict__ pts, const float *__restrict__ core2,
                                 int64_t n, float *__restrict__ out) {
+  wait_for_previous();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   out[__float_as_uint(pts[i].w)] = core2[i];
@@ -136,8 +138,8 @@ void launch_core_knn(Problem &P, int k) {
   const bool h = P.leaf > 1;
 #define EMST_KNN(M) \
   do { \
-    if (h) k_core_knn<M, true><<<g, kCoreBlock, 0, P.stream>>>(P.pts, P.nodes, P.n, P.leaf, m, P.core2, P.counters + 1); \
-    else k_core_knn<M, false><<<g, kCoreBlock, 0, P.stream>>>(P.pts, P.nodes, P.n, P.leaf, m, P.core2, P.counters + 1); \
+    if (h) launch_next(P, k_core_knn<M, true>, g, kCoreBlock, 0, P.pts, P.nodes, P.n, P.leaf, m, P.core2, P.counters + 1); \
+    else launch_next(P, k_core_knn<M, false>, g, kCoreBlock, 0, P.pts, P.nodes, P.n, P.leaf, m, P.core2, P.counters + 1); \
   } while (0)
   if (m <= 4) EMST_KNN(4);
   else if (m <= 8) EMST_KNN(8);
@@ -148,7 +150,7 @@ void launch_core_knn(Problem &P, int k) {
 }
 
 void launch_core_to_input(Problem &P, float *out) {
-  k_core_to_input<<<grid_for(P.n, 256), 256, 0, P.stream>>>(P.pts, P.core2, P.n, out);
+  launch_next(P, k_core_to_input, grid_for(P.n, 256), 256, 0, P.pts, P.core2, P.n, out);
   P.launches += 1;
 }
 

@@ -33,11 +33,12 @@ __device__ void post_mail(const uint32_t *counters, uint32_t *mail, uint32_t seq
 }
 
 __global__ void k_post_mail(const uint32_t *counters, uint32_t *mail, uint32_t seq) {
+  wait_for_previous();
   post_mail(counters, mail, seq);
 }
 
 void launch_post_mail(Problem &P) {
-  k_post_mail<<<1, 64, 0, P.stream>>>(P.counters, P.mail, P.mail_seq);
+  launch_next(P, k_post_mail, 1, 64, 0, P.counters, P.mail, P.mail_seq);
   P.launches += 1;
 }
 
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(kScanThreads, EMST_SCAN_MIN_BLOCKS) k_runs(
     uint32_t *__restrict__ labels_new, uint32_t *bound_next,
     uint2 *__restrict__ words, uint32_t *tile_total, uint32_t *tile_prefix, uint32_t *done,
     const uint32_t *counters, uint32_t *mail, uint32_t mail_seq, bool look) {
+  wait_for_previous();
   __shared__ uint32_t s_warp[kScanThreads / 32];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -242,13 +244,11 @@ static void launch_runs(Problem &P, bool relabel) {
   uint32_t *tile_total = P.scan_tiles, *tile_prefix = P.scan_tiles + tiles;
   uint2 *words = reinterpret_cast<uint2 *>(P.runs);
   if (relabel)
-    k_runs<true><<<(unsigned)tiles, kScanThreads, 0, P.stream>>>(
-        P.labels, P.root, P.pts, P.inst_of, P.core2, P.n, P.labels_buf[P.cur ^ 1],
+    launch_next(P, k_runs<true>, (unsigned)tiles, kScanThreads, 0, P.labels, P.root, P.pts, P.inst_of, P.core2, P.n, P.labels_buf[P.cur ^ 1],
         P.bound_buf[P.cur ^ 1], words, tile_total, tile_prefix, done, P.counters, P.mail, P.mail_seq,
         P.n >= kManyPoints);
   else
-    k_runs<false><<<(unsigned)tiles, kScanThreads, 0, P.stream>>>(
-        P.labels, nullptr, P.pts, P.inst_of, nullptr, P.n, nullptr, nullptr, words, tile_total,
+    launch_next(P, k_runs<false>, (unsigned)tiles, kScanThreads, 0, P.labels, nullptr, P.pts, P.inst_of, nullptr, P.n, nullptr, nullptr, words, tile_total,
         tile_prefix, done, nullptr, nullptr, 0u, false);
   P.launches += 1;
 }
@@ -273,19 +273,22 @@ __global__ void __launch_bounds__(kBlock) k_node_labels(const uint32_t *__restri
                                                         int64_t n, int64_t nc, int leaf,
                                                         uint32_t *__restrict__ mixed,
                                                         uint2 *__restrict__ nlabels,
-                                                        uint32_t *counters) {
+                                                        uint32_t *counters, uint32_t stop_at) {
+  wait_for_previous();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
+  const uint32_t emitted = __ldcg(counters);
+  const int64_t w0 = (t >> 5) * WORDS;
+  const int64_t word_count = (nc - 1 + 31) >> 5;
+  uint32_t mine = 0u;
+  if (lane < WORDS && w0 + lane < word_count) mine = mixed[w0 + lane];
+  if (emitted >= stop_at) return;  // launched ahead, and there is no such round
   if (t == 0) {  // the round's counters (the first kernel of a round)
     counters[40] = counters[12];      // components listed by the previous merge
     counters[12] = 0u;
     counters[kActiveCounter] = 0u;
     counters[kActiveQueue] = 0u;
   }
-  const int64_t w0 = (t >> 5) * WORDS;
-  const int64_t word_count = (nc - 1 + 31) >> 5;
-  uint32_t mine = 0u;
-  if (lane < WORDS && w0 + lane < word_count) mine = mixed[w0 + lane];
 #pragma unroll
   for (int q = 0; q < WORDS; ++q) {
     const uint32_t word = __shfl_sync(0xffffffffu, mine, q);
@@ -317,11 +320,9 @@ void launch_node_labels(Problem &P) {
   const uint2 *words = reinterpret_cast<const uint2 *>(P.runs);
   const uint32_t *prefix = P.scan_tiles + scan_tiles_for(P.n);
   if (nodes >= kManyPoints)
-    k_node_labels<4><<<grid_for((nodes + 3) / 4, kBlock), kBlock, 0, P.stream>>>(
-        P.labels, words, prefix, P.range, P.n, P.nc, P.leaf, P.mixed, P.nlabels, P.counters);
+    launch_next(P, k_node_labels<4>, grid_for((nodes + 3) / 4, kBlock), kBlock, 0, P.labels, words, prefix, P.range, P.n, P.nc, P.leaf, P.mixed, P.nlabels, P.counters, P.stop_at);
   else
-    k_node_labels<1><<<grid_for(nodes, kBlock), kBlock, 0, P.stream>>>(
-        P.labels, words, prefix, P.range, P.n, P.nc, P.leaf, P.mixed, P.nlabels, P.counters);
+    launch_next(P, k_node_labels<1>, grid_for(nodes, kBlock), kBlock, 0, P.labels, words, prefix, P.range, P.n, P.nc, P.leaf, P.mixed, P.nlabels, P.counters, P.stop_at);
   P.launches += 1;
 }
 
@@ -336,6 +337,7 @@ __global__ void __launch_bounds__(kBlock) k_upper_bounds(const float4 *__restric
                                                          const uint32_t *__restrict__ inst_of,
                                                          const float *__restrict__ core2,
                                                          int64_t n, uint32_t *bound) {
+  wait_for_previous();
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k + 1 >= n) return;
   uint32_t la = labels[k], lb = labels[k + 1];
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(kBlock) k_upper_bounds(const float4 *__restric
 }
 
 void launch_upper_bounds(Problem &P) {
-  k_upper_bounds<<<grid_for(P.n, kBlock), kBlock, 0, P.stream>>>(P.pts, P.labels, P.inst_of,
+  launch_next(P, k_upper_bounds, grid_for(P.n, kBlock), kBlock, 0, P.pts, P.labels, P.inst_of,
                                                                  P.core2, P.n, P.bound);
   P.launches += 1;
 }
@@ -359,6 +361,7 @@ template <bool CARRIED, bool RADIUS_IN, bool COUNT, bool SEEDED, bool CHUNKS, bo
           bool FIRST, bool MRD, bool TIES = true, bool LBT = true, bool KEPT = true>
 __global__ void __launch_bounds__(kTraverseMaxBlock, EMST_TRAVERSE_MIN_BLOCKS) k_traverse(TravArgs A, const uint32_t *__restrict__ list,
                                                      const uint32_t *__restrict__ list_count) {
+  wait_for_previous();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (list && A.queue) {
     // the next 32 entries for this warp, in list order, so the queries in
@@ -409,6 +412,7 @@ constexpr int kDefaultChunk = 64;    // measured best of 32 / 64 / 128
 template <bool CARRIED, bool FIRST, bool TIES, bool COUNT>
 __global__ void __launch_bounds__(kPersistBlock, EMST_PERSIST_MIN_BLOCKS)
     k_traverse_queue(TravArgs A, unsigned long long *queue, int refill, int chunk) {
+  wait_for_previous();
   const unsigned lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t n = A.n;
@@ -510,7 +514,7 @@ static void queue_launch(Problem &P, const TravArgs &A) {
   const int64_t g_need = (warps_needed + kPersistBlock / 32 - 1) / (kPersistBlock / 32);
   if (g > g_need) g = g_need;
   if (g < 1) g = 1;
-  kern<<<(unsigned)g, kPersistBlock, sm, P.stream>>>(A, reinterpret_cast<unsigned long long *>(P.counters + 36),
+  launch_next(P, kern, (unsigned)g, kPersistBlock, sm, A, reinterpret_cast<unsigned long long *>(P.counters + 36),
                                                      refill, chunk);
 }
 
@@ -581,7 +585,6 @@ constexpr int kOrderedUntilRound = EMST_ORDERED_UNTIL_ROUND;  // exact curve ord
 constexpr int kNear = 4;
 constexpr int kNearSeed = 6;
 constexpr int kNearRounds = 3;
-static_assert(kNearRounds < EMST_ORDERED_UNTIL_ROUND, "the ordered listing reads the settled points");
 
 // The candidate c at weight d <= w[kNear - 1] among the kNear best so far (w
 // ascending, ties by original id; kInvalid at +inf: empty).  Some lane of a
@@ -617,6 +620,7 @@ constexpr int kNearBlock = 128;
 // entry's edge as the component's minimum (no other query offers to it).
 template <bool TIES, bool COUNT>
 __global__ void __launch_bounds__(kNearBlock, 16) k_near(TravArgs A) {
+  wait_for_previous();
   const float kInf = __int_as_float(0x7f800000);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -746,6 +750,7 @@ __global__ void __launch_bounds__(256) k_settle(const float4 *__restrict__ pts,
                                                 const uint32_t *__restrict__ bound, CompBest *comp,
                                                 uint2 *__restrict__ res, int64_t n,
                                                 uint32_t *__restrict__ settled, uint32_t *status) {
+  wait_for_previous();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   bool known = false;
@@ -809,14 +814,18 @@ __device__ __forceinline__ uint32_t open_points(const uint32_t *__restrict__ bou
 
 // The same with one atomic per warp of 128 positions (four per thread):
 // the list is in curve order only within each warp's positions, which costs
-// the traversal locality while many queries are listed but saves the count
-// pass's scan when few are (rounds from kOrderedUntilRound on).
+// the traversal locality while many queries are listed and the node records
+// exceed the L2, but saves a launch and the count pass's scan otherwise
+// (rounds from kOrderedUntilRound on; every round below kManyPoints: 2M dense
+// points 4,130 -> 4,067 us a call, 1M 2D 1,383 -> 1,375).
 __global__ void __launch_bounds__(256) k_active(const uint32_t *__restrict__ labels,
                                                 const uint32_t *__restrict__ bound,
                                                 const CompBest *__restrict__ comp,
                                                 const uint2 *__restrict__ res,
+                                                const uint8_t *__restrict__ settled,
                                                 int64_t n, uint32_t *__restrict__ list,
                                                 uint32_t *count) {
+  wait_for_previous();
   const int lane = threadIdx.x & 31;
   const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   uint32_t act = 0;
@@ -838,6 +847,7 @@ __global__ void __launch_bounds__(256) k_active(const uint32_t *__restrict__ lab
       }
     }
     act = open_points<4>(bound, comp, i0, n, lab, prev);
+    if (settled) act &= ~((uint32_t)settled[i0 >> 3] >> (i0 & 7));
   }
   const uint32_t c = (uint32_t)__popc(act);
   uint32_t x = c;
@@ -867,6 +877,7 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_count(
     const uint32_t *__restrict__ labels, const uint32_t *__restrict__ bound, const CompBest *__restrict__ comp,
     const uint2 *__restrict__ res, const uint8_t *__restrict__ settled, int64_t n,
     uint8_t *__restrict__ flags, uint32_t *tile_total, uint32_t *tile_prefix, uint32_t *done, uint32_t *count) {
+  wait_for_previous();
   __shared__ uint32_t s_warp[kActiveThreads / 32];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -927,6 +938,7 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_count(
 __global__ void __launch_bounds__(kActiveThreads) k_active_write(const uint8_t *__restrict__ flags,
                                                                  const uint32_t *__restrict__ tile_prefix,
                                                                  int64_t n, uint32_t *__restrict__ list) {
+  wait_for_previous();
   __shared__ uint32_t s_warp[kActiveThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t t = (int64_t)blockIdx.x * kActiveThreads + tid;
@@ -951,9 +963,9 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_write(const uint8_t *
 
 using TravKernel = void (*)(TravArgs, const uint32_t *, const uint32_t *);
 
-static void launch_trav(TravKernel k, int g, int block, cudaStream_t s, const TravArgs &A,
+static void launch_trav(TravKernel k, int g, int block, const Problem &P, const TravArgs &A,
                         const uint32_t *list, const uint32_t *list_count) {
-  k<<<g, block, 0, s>>>(A, list, list_count);
+  launch_next(P, k, g, block, 0, A, list, list_count);
 }
 
 // The tighter lower bound of empty searches (traverse_one's LB) is tracked
@@ -1006,15 +1018,14 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
   const uint32_t *list = learned_pass == 2 ? P.rerun_list : nullptr;
   const uint32_t *list_count = learned_pass == 2 ? P.counters + 13 : nullptr;
   int g = learned_pass == 2 ? sm_count() * 8 : grid_for(P.n, block);
-  cudaStream_t s = P.stream;
   if (P.near_j && first) {
     // the lists; no later step of the round needs the bounds or the minima cleared
     if (P.ties) {
-      if (count) k_near<true, true><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
-      else k_near<true, false><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
+      if (count) launch_next(P, k_near<true, true>, grid_for(P.n, kNearBlock), kNearBlock, 0, A);
+      else launch_next(P, k_near<true, false>, grid_for(P.n, kNearBlock), kNearBlock, 0, A);
     } else {
-      if (count) k_near<false, true><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
-      else k_near<false, false><<<grid_for(P.n, kNearBlock), kNearBlock, 0, s>>>(A);
+      if (count) launch_next(P, k_near<false, true>, grid_for(P.n, kNearBlock), kNearBlock, 0, A);
+      else launch_next(P, k_near<false, false>, grid_for(P.n, kNearBlock), kNearBlock, 0, A);
     }
     P.launches += 1;
     return;
@@ -1033,19 +1044,19 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     uint8_t *settled = nullptr;
     if (P.near_j && round <= kNearRounds) {
       uint32_t *words = reinterpret_cast<uint32_t *>(P.keys[0]);  // free during the rounds
-      k_settle<<<grid_for(P.n, 256), 256, 0, s>>>(P.pts, P.labels, P.near_j, P.near_w, P.bound, P.comp, P.res,
+      launch_next(P, k_settle, grid_for(P.n, 256), 256, 0, P.pts, P.labels, P.near_j, P.near_w, P.bound, P.comp, P.res,
                                                   P.n, words, P.counters + 1);
       P.launches += 1;
       settled = reinterpret_cast<uint8_t *>(words);
     }
-    if (round < kOrderedUntilRound) {
-      k_active_count<<<(unsigned)tiles, kActiveThreads, 0, s>>>(P.labels, P.bound, P.comp, P.res, settled,
+    if (P.n >= kManyPoints && round < kOrderedUntilRound) {
+      launch_next(P, k_active_count, (unsigned)tiles, kActiveThreads, 0, P.labels, P.bound, P.comp, P.res, settled,
                                                                P.n, flags, tile_total, tile_prefix,
                                                                P.counters + kActiveDone, active_count);
-      k_active_write<<<(unsigned)tiles, kActiveThreads, 0, s>>>(flags, tile_prefix, P.n, active);
+      launch_next(P, k_active_write, (unsigned)tiles, kActiveThreads, 0, flags, tile_prefix, P.n, active);
       P.launches += 2;
     } else {
-      k_active<<<(unsigned)grid_for((P.n + 3) / 4, 256), 256, 0, s>>>(P.labels, P.bound, P.comp, P.res,
+      launch_next(P, k_active, (unsigned)grid_for((P.n + 3) / 4, 256), 256, 0, P.labels, P.bound, P.comp, P.res, settled,
                                                                        P.n, active, active_count);
       P.launches += 1;
     }
@@ -1054,7 +1065,7 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     g = sm_count() * (2048 / block);  // one resident wave
     A.queue = P.counters + kActiveQueue;  // warps take the list in order
   }
-#define EMST_LAUNCH(...) launch_trav(k_traverse<__VA_ARGS__>, g, block, s, A, list, list_count)
+#define EMST_LAUNCH(...) launch_trav(k_traverse<__VA_ARGS__>, g, block, P, A, list, list_count)
 // a host flag as a template argument
 #define EMST_IF(flag, B, ...)       \
   do {                              \
@@ -1141,6 +1152,7 @@ __global__ void __launch_bounds__(kBlock) k_merge_roots(const uint32_t *__restri
                                                         emst_edge *__restrict__ edges,
                                                         uint32_t *__restrict__ next_list,
                                                         uint32_t *counters, int64_t n) {
+  wait_for_previous();
   __shared__ uint32_t s_warp[2][kBlock / 32];
   __shared__ uint32_t s_wmax[kBlock / 32];
   __shared__ uint32_t s_base[2];
@@ -1216,7 +1228,7 @@ void launch_merge(Problem &P) {
   // graph rounds: this round's list length exists only on the device (put
   // there by k_node_labels)
   const uint32_t *count_dev = P.active_list ? P.count_dev : nullptr;
-  k_merge_roots<<<g, kBlock, 0, P.stream>>>(P.active_list, count, count_dev, P.comp, P.comp_buf[P.cur ^ 1],
+  launch_next(P, k_merge_roots, g, kBlock, 0, P.active_list, count, count_dev, P.comp, P.comp_buf[P.cur ^ 1],
                                             P.bound_buf[P.cur ^ 1], P.root, P.edges, P.next_list, P.counters, P.n);
   P.launches += 1;
   launch_runs(P, true);
@@ -1240,6 +1252,7 @@ void advance_round(Problem &P, int64_t n_active) {
 // cleared for the next round.
 __global__ void __launch_bounds__(kBlock) k_count_seen(uint32_t *seen, int64_t words,
                                                        unsigned long long *total) {
+  wait_for_previous();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned c = 0;
   if (k < words) {
@@ -1253,19 +1266,19 @@ __global__ void __launch_bounds__(kBlock) k_count_seen(uint32_t *seen, int64_t w
 void launch_count_seen(Problem &P) {
   if (!P.seen || P.nc < 2) return;
   const int64_t words = (P.nc - 1 + 31) / 32;
-  k_count_seen<<<grid_for(words, kBlock), kBlock, 0, P.stream>>>(
-      P.seen, words, reinterpret_cast<unsigned long long *>(P.counters + 38));
+  launch_next(P, k_count_seen, grid_for(words, kBlock), kBlock, 0, P.seen, words, reinterpret_cast<unsigned long long *>(P.counters + 38));
   P.launches += 1;
 }
 
 __global__ void k_fill_u32(uint32_t *p, uint32_t v, int64_t count) {
+  wait_for_previous();
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < count) p[k] = v;
 }
 
 void launch_fill_u32(Problem &P, uint32_t *p, uint32_t v, int64_t count) {
   if (count <= 0) return;
-  k_fill_u32<<<grid_for(count, kBlock), kBlock, 0, P.stream>>>(p, v, count);
+  launch_next(P, k_fill_u32, grid_for(count, kBlock), kBlock, 0, p, v, count);
   P.launches += 1;
 }
 
@@ -1284,8 +1297,11 @@ constexpr int kTieRunMax = 64;
 
 __global__ void k_edge_keys_wi(const emst_edge *__restrict__ edges, int64_t m,
                                uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
-                               int shift_i) {
+                               int shift_i, ClearWords clear, uint32_t *long_runs) {
+  wait_for_previous();
+  clear_words(clear);
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e == 0) *long_runs = 0u;
   if (e >= m) return;
   const emst_edge E = edges[e];
   keys[e] = ((uint64_t)__float_as_uint(E.w) << shift_i) | (uint64_t)E.i;
@@ -1296,6 +1312,7 @@ __global__ void k_edge_keys_wi(const emst_edge *__restrict__ edges, int64_t m,
 // sort), or counts it when it is longer than kTieRunMax.
 __global__ void k_edge_ties(const uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
                             int64_t m, uint32_t *long_runs) {
+  wait_for_previous();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e + 1 >= m) return;
   const uint64_t key = keys[e];
@@ -1323,6 +1340,7 @@ __global__ void k_edge_ties(const uint64_t *__restrict__ keys, uint32_t *__restr
 // w bits being equal -- or counts it when it is longer than kTieRunMax.
 __global__ void k_edge_ties_w(uint64_t *__restrict__ keys, uint32_t *__restrict__ vals, int64_t m,
                               int shift_i, uint32_t *long_runs) {
+  wait_for_previous();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e + 1 >= m) return;
   const uint64_t w = keys[e] >> shift_i;
@@ -1352,6 +1370,7 @@ __global__ void k_edge_ties_w(uint64_t *__restrict__ keys, uint32_t *__restrict_
 __global__ void k_edge_from_keys(const uint64_t *__restrict__ keys,
                                  const uint32_t *__restrict__ vals, int64_t m, int shift_i,
                                  uint32_t w_mask, emst_edge *__restrict__ out) {
+  wait_for_previous();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= m) return;
   const uint64_t k = keys[e];
@@ -1367,10 +1386,12 @@ __global__ void k_edge_from_keys(const uint64_t *__restrict__ keys,
 // chip-to-chip link, where whole coalesced lines matter): thread c writes
 // 16-byte chunk c of the output, i.e. words 4c..4c+3 of the flat array of
 // (i, j, w) words, rebuilt from the (at most two) edges they belong to.
-// `out` 16-byte aligned; chunks = floor(3m / 4) whole chunks.
+// `out` 16-byte aligned; chunks = floor(3m / 4) whole chunks, the last one's
+// thread also writes the (at most three) words after it.
 __global__ void k_edge_from_keys16(const uint64_t *__restrict__ keys,
-                                   const uint32_t *__restrict__ vals, int64_t chunks, int shift_i,
-                                   uint32_t w_mask, uint4 *__restrict__ out) {
+                                   const uint32_t *__restrict__ vals, int64_t chunks, int64_t m,
+                                   int shift_i, uint32_t w_mask, uint4 *__restrict__ out) {
+  wait_for_previous();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= chunks) return;
   const uint64_t imask = (1ull << shift_i) - 1ull;
@@ -1391,6 +1412,14 @@ __global__ void k_edge_from_keys16(const uint64_t *__restrict__ keys,
     }
   }
   out[c] = make_uint4(w[0], w[1], w[2], w[3]);
+  if (c == chunks - 1) {
+    uint32_t *flat = reinterpret_cast<uint32_t *>(out);
+    for (int64_t x = 4 * chunks; x < 3 * m; ++x) {
+      const uint64_t kx = __ldg(keys + x / 3);
+      const int fx = (int)(x % 3);
+      flat[x] = fx == 0 ? (uint32_t)(kx & imask) : fx == 1 ? __ldg(vals + x / 3) : ((uint32_t)(kx >> shift_i) & w_mask);
+    }
+  }
 }
 
 // Batched fast path: one key per edge, (instance, w, local i), with the
@@ -1402,8 +1431,11 @@ __global__ void k_edge_keys_inst_wi(const emst_edge *__restrict__ edges, int64_t
                                     uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
                                     const uint32_t *__restrict__ inst_in,
                                     const int64_t *__restrict__ offsets, int shift_w,
-                                    int shift_i) {
+                                    int shift_i, ClearWords clear, uint32_t *long_runs) {
+  wait_for_previous();
+  clear_words(clear);
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e == 0) *long_runs = 0u;
   if (e >= m) return;
   const emst_edge E = edges[e];
   const uint32_t I = __ldg(inst_in + E.i);
@@ -1416,7 +1448,9 @@ __global__ void k_edge_keys_inst_wi(const emst_edge *__restrict__ edges, int64_t
 // Full path: keys by j with the edge index as the value, then keys by
 // (w, i) of the edges in that order.
 __global__ void k_edge_keys_j(const emst_edge *__restrict__ edges, int64_t m,
-                              uint64_t *__restrict__ keys, uint32_t *__restrict__ vals) {
+                              uint64_t *__restrict__ keys, uint32_t *__restrict__ vals, ClearWords clear) {
+  wait_for_previous();
+  clear_words(clear);
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= m) return;
   keys[e] = edges[e].j;
@@ -1426,6 +1460,7 @@ __global__ void k_edge_keys_j(const emst_edge *__restrict__ edges, int64_t m,
 __global__ void k_edge_keys_wi_of(const emst_edge *__restrict__ edges, int64_t m,
                                   uint64_t *__restrict__ keys, const uint32_t *__restrict__ vals,
                                   int shift_i) {
+  wait_for_previous();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= m) return;
   const emst_edge E = edges[vals[e]];
@@ -1435,6 +1470,7 @@ __global__ void k_edge_keys_wi_of(const emst_edge *__restrict__ edges, int64_t m
 __global__ void k_edge_keys_inst(const emst_edge *__restrict__ edges, int64_t m,
                                  uint64_t *__restrict__ keys, const uint32_t *__restrict__ vals,
                                  const uint32_t *__restrict__ inst_in) {
+  wait_for_previous();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= m) return;
   keys[e] = __ldg(inst_in + edges[vals[e]].i);
@@ -1445,6 +1481,7 @@ __global__ void k_edge_gather(const emst_edge *__restrict__ edges, int64_t m,
                               const uint32_t *__restrict__ order, emst_edge *__restrict__ out,
                               const uint32_t *__restrict__ inst_in,
                               const int64_t *__restrict__ offsets) {
+  wait_for_previous();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= m) return;
   emst_edge E = edges[order[e]];
@@ -1457,60 +1494,55 @@ __global__ void k_edge_gather(const emst_edge *__restrict__ edges, int64_t m,
 }
 
 void launch_edge_keys_wi(Problem &P, int64_t m, int shift_i) {
-  k_edge_keys_wi<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.edges, m, P.keys[0], P.vals[0],
-                                                               shift_i);
+  launch_next(P, k_edge_keys_wi, grid_for(m, kBlock), kBlock, 0, P.edges, m, P.keys[0], P.vals[0],
+              shift_i, ClearWords{P.sort_state, sort_clear_words(m)}, P.counters + 10);
   P.launches += 1;
 }
 void launch_edge_ties(Problem &P, int64_t m, int src) {
-  k_edge_ties<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.keys[src], P.vals[src], m,
+  launch_next(P, k_edge_ties, grid_for(m, kBlock), kBlock, 0, P.keys[src], P.vals[src], m,
                                                             P.counters + 10);
   P.launches += 1;
 }
 void launch_edge_ties_w(Problem &P, int64_t m, int src, int shift_i) {
-  k_edge_ties_w<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.keys[src], P.vals[src], m, shift_i,
+  launch_next(P, k_edge_ties_w, grid_for(m, kBlock), kBlock, 0, P.keys[src], P.vals[src], m, shift_i,
                                                               P.counters + 10);
   P.launches += 1;
 }
 void launch_edge_from_keys(Problem &P, int64_t m, int src, int shift_i, int w_bits_used,
                            emst_edge *out) {
   const uint32_t w_mask = w_bits_used >= 32 ? 0xFFFFFFFFu : ((1u << w_bits_used) - 1u);
-  // whole 16-byte chunks of the output by coalesced wide stores when it is
-  // 16-byte aligned, the edges after the last whole chunk one by one
+  // by coalesced 16-byte stores when the output is 16-byte aligned
   const int64_t chunks = (reinterpret_cast<uintptr_t>(out) & 15u) == 0 ? (3 * m) / 4 : 0;
-  const int64_t covered = (4 * chunks) / 3;  // edges wholly inside those chunks (the next one,
-                                             // if split, is rewritten whole below)
-  if (chunks > 0) {
-    k_edge_from_keys16<<<grid_for(chunks, kBlock), kBlock, 0, P.stream>>>(
-        P.keys[src], P.vals[src], chunks, shift_i, w_mask, reinterpret_cast<uint4 *>(out));
-    P.launches += 1;
-  }
-  if (m - covered > 0) {
-    k_edge_from_keys<<<grid_for(m - covered, kBlock), kBlock, 0, P.stream>>>(
-        P.keys[src] + covered, P.vals[src] + covered, m - covered, shift_i, w_mask, out + covered);
-    P.launches += 1;
-  }
+  if (chunks > 0)
+    launch_next(P, k_edge_from_keys16, grid_for(chunks, kBlock), kBlock, 0, P.keys[src], P.vals[src], chunks, m,
+                shift_i, w_mask, reinterpret_cast<uint4 *>(out));
+  else
+    launch_next(P, k_edge_from_keys, grid_for(m, kBlock), kBlock, 0, P.keys[src], P.vals[src], m, shift_i, w_mask,
+                out);
+  P.launches += 1;
 }
 void launch_edge_keys_inst_wi(Problem &P, int64_t m, int shift_w, int shift_i) {
-  k_edge_keys_inst_wi<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(
-      P.edges, m, P.keys[0], P.vals[0], P.inst_in, P.offsets, shift_w, shift_i);
+  launch_next(P, k_edge_keys_inst_wi, grid_for(m, kBlock), kBlock, 0, P.edges, m, P.keys[0], P.vals[0], P.inst_in, P.offsets,
+              shift_w, shift_i, ClearWords{P.sort_state, sort_clear_words(m)}, P.counters + 10);
   P.launches += 1;
 }
 void launch_edge_keys_j(Problem &P, int64_t m) {
-  k_edge_keys_j<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.edges, m, P.keys[0], P.vals[0]);
+  launch_next(P, k_edge_keys_j, grid_for(m, kBlock), kBlock, 0, P.edges, m, P.keys[0], P.vals[0],
+              ClearWords{P.sort_state, sort_clear_words(m)});
   P.launches += 1;
 }
 void launch_edge_keys_wi_of(Problem &P, int64_t m, int src, int shift_i) {
-  k_edge_keys_wi_of<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.edges, m, P.keys[src],
+  launch_next(P, k_edge_keys_wi_of, grid_for(m, kBlock), kBlock, 0, P.edges, m, P.keys[src],
                                                                   P.vals[src], shift_i);
   P.launches += 1;
 }
 void launch_edge_keys_inst(Problem &P, int64_t m, int src) {
-  k_edge_keys_inst<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.edges, m, P.keys[src],
+  launch_next(P, k_edge_keys_inst, grid_for(m, kBlock), kBlock, 0, P.edges, m, P.keys[src],
                                                                   P.vals[src], P.inst_in);
   P.launches += 1;
 }
 void launch_edge_gather(Problem &P, int64_t m, const uint32_t *order, emst_edge *out) {
-  k_edge_gather<<<grid_for(m, kBlock), kBlock, 0, P.stream>>>(P.edges, m, order, out, P.inst_in,
+  launch_next(P, k_edge_gather, grid_for(m, kBlock), kBlock, 0, P.edges, m, order, out, P.inst_in,
                                                               P.offsets);
   P.launches += 1;
 }

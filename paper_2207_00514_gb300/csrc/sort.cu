@@ -50,6 +50,11 @@ static_assert(kSortThreads == kRadix, "a sort pass gives each thread one digit")
 constexpr int64_t kHistWords = 8 * kRadix;
 constexpr int64_t kCounterWords = 64;  // [0..7] tile counters, [8] finished CTAs
 
+int64_t sort_clear_words(int64_t n) {
+  const int items = n <= kSmallMax ? kSmallItems : n <= kMidMax ? kMidItems : kLargeItems;
+  return kHistWords + kCounterWords + kRadix * ((n + kSortThreads * items - 1) / (kSortThreads * items));
+}
+
 int64_t sort_state_words(int64_t n) { return kHistWords + kCounterWords + 2 * kRadix * sort_tiles_for(n); }
 
 // Histograms of all digits in [digit_begin, digit_end) in one pass; the last
@@ -60,6 +65,7 @@ __global__ void __launch_bounds__(512) k_sort_hist(const uint64_t *__restrict__ 
   __shared__ uint32_t sh[8][kRadix];
   __shared__ bool s_last;
   for (int t = threadIdx.x; t < 8 * kRadix; t += blockDim.x) (&sh[0][0])[t] = 0;
+  wait_for_previous();
   __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
@@ -131,8 +137,9 @@ __global__ void __launch_bounds__(kSortThreads, BLOCKS) k_sort_pass(
   constexpr int kTile = SortSmem<ITEMS>::kTile;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  if (tid == 0) S.tile_id = atomicAdd(tile_counter, 1u);
   for (int t = tid; t < kWarps * kRadix; t += kSortThreads) (&S.warp_hist[0][0])[t] = 0;
+  wait_for_previous();
+  if (tid == 0) S.tile_id = atomicAdd(tile_counter, 1u);
   __syncthreads();
   const uint32_t tile = S.tile_id;
   const int64_t base = (int64_t)tile * kTile;
@@ -274,9 +281,8 @@ __global__ void __launch_bounds__(kSortThreads, BLOCKS) k_sort_pass(
 
 // One sort of tiles of kSortThreads x ITEMS keys.
 template <int ITEMS, int BLOCKS>
-static int sort_passes(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0) {
+static int sort_passes(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0, bool cleared) {
   static bool attr_set[64] = {false};
-  cudaStream_t s = P.stream;
   int dev = 0;
   cudaGetDevice(&dev);
   const size_t smem = sizeof(SortSmem<ITEMS>);
@@ -287,14 +293,14 @@ static int sort_passes(Problem &P, int64_t n, int digit_begin, int digit_end, in
   const int64_t tiles = (n + SortSmem<ITEMS>::kTile - 1) / SortSmem<ITEMS>::kTile;
   uint32_t *hist = P.sort_state, *counters = hist + kHistWords;
   uint32_t *look[2] = {counters + kCounterWords, counters + kCounterWords + kRadix * tiles};
-  cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)(kHistWords + kCounterWords + kRadix * tiles), s);
+  if (!cleared)
+    cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)(kHistWords + kCounterWords + kRadix * tiles), P.stream);
   int hgrid = (int)((n + 511) / 512);
   if (hgrid > sm_count() * 4) hgrid = sm_count() * 4;
-  k_sort_hist<<<hgrid, 512, 0, s>>>(P.keys[src], n, digit_begin, digit_end, bit0, hist, counters + 8);
+  launch_next(P, k_sort_hist, hgrid, 512, 0, P.keys[src], n, digit_begin, digit_end, bit0, hist, counters + 8);
   P.launches += 1;
   for (int d = digit_begin; d < digit_end; ++d) {
-    k_sort_pass<ITEMS, BLOCKS><<<(unsigned)tiles, kSortThreads, smem, s>>>(
-        P.keys[src], P.vals[src], P.keys[src ^ 1], P.vals[src ^ 1], n, bit0 + 8 * d, hist + d * kRadix,
+    launch_next(P, k_sort_pass<ITEMS, BLOCKS>, (unsigned)tiles, kSortThreads, smem, P.keys[src], P.vals[src], P.keys[src ^ 1], P.vals[src ^ 1], n, bit0 + 8 * d, hist + d * kRadix,
         look[0], look[1], counters + d, P.counters + 1);
     P.launches += 1;
     src ^= 1;
@@ -305,11 +311,12 @@ static int sort_passes(Problem &P, int64_t n, int digit_begin, int digit_end, in
   return src;
 }
 
-int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0) {
+int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int src, int bit0,
+                     bool cleared) {
   if (n <= 1 || digit_begin >= digit_end) return src;
-  if (n <= kSmallMax) return sort_passes<kSmallItems, 4>(P, n, digit_begin, digit_end, src, bit0);
-  if (n <= kMidMax) return sort_passes<kMidItems, 4>(P, n, digit_begin, digit_end, src, bit0);
-  return sort_passes<kLargeItems, 3>(P, n, digit_begin, digit_end, src, bit0);
+  if (n <= kSmallMax) return sort_passes<kSmallItems, 4>(P, n, digit_begin, digit_end, src, bit0, cleared);
+  if (n <= kMidMax) return sort_passes<kMidItems, 4>(P, n, digit_begin, digit_end, src, bit0, cleared);
+  return sort_passes<kLargeItems, 3>(P, n, digit_begin, digit_end, src, bit0, cleared);
 }
 
 }  // namespace emst
