@@ -365,19 +365,21 @@ __global__ void __launch_bounds__(kTraverseMaxBlock, EMST_TRAVERSE_MIN_BLOCKS) k
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (list && A.queue) {
     // the next 32 entries for this warp, in list order, so the queries in
-    // flight stay a window of the list (and of the curve) that L2 holds
-    for (;;) {
-      const uint32_t lane = threadIdx.x & 31;
-      uint32_t at = 0;
-      if (lane == 0) at = atomicAdd(A.queue, 32u);
-      at = __shfl_sync(0xffffffffu, at, 0);
-      const uint32_t count = *list_count;
-      if (at >= count) break;
-      at += lane;
-      if (at < count)
+    // flight stay a window of the list (and of the curve) that L2 holds: the
+    // first ones by the warp's place in the grid, the others from the queue
+    // (every warp's first from the queue would be twenty thousand atomics on
+    // one word before any search starts)
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t count = *list_count;
+    const uint32_t grid = gridDim.x * blockDim.x;
+    for (uint32_t at = (uint32_t)gid - lane; at < count;) {
+      if (at + lane < count)
         traverse_one<CARRIED, RADIUS_IN, COUNT, SEEDED, CHUNKS, LEARNED, FIRST, MRD, TIES, LBT, KEPT>(
-            A, __ldg(list + at));
+            A, __ldg(list + at + lane));
       __syncwarp();
+      if (count <= grid) break;
+      if (lane == 0) at = grid + atomicAdd(A.queue, 32u);
+      at = __shfl_sync(0xffffffffu, at, 0);
     }
   } else if (list) {
     const int64_t count = *list_count;
