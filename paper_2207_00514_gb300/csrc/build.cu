@@ -384,13 +384,18 @@ __global__ void __launch_bounds__(kBlock) k_gather(const float *__restrict__ pts
   // sorted codes: equal 32 positions back means all between are equal too
   const bool run = k >= 32 && __ldg(sorted_codes + k) == __ldg(sorted_codes + k - 32) &&
                    (!code_hi || __ldg(code_hi + k) == __ldg(code_hi + k - 32));
+  // and, two longer than a run of equal keys that the output orders in place
+  // (kTieRunMax), for it to choose its sort
+  const bool longer = run && k >= kGroupLong && __ldg(sorted_codes + k) == __ldg(sorted_codes + k - kGroupLong) &&
+                      (!code_hi || __ldg(code_hi + k) == __ldg(code_hi + k - kGroupLong));
   const unsigned mask = __activemask();
+  const unsigned cl = __ballot_sync(mask, longer);
   const unsigned cs = __popc(__ballot_sync(mask, same)), cd = __popc(__ballot_sync(mask, differ));
   const unsigned cr = __ballot_sync(mask, run);
   if ((threadIdx.x & 31) == (unsigned)(__ffs(mask) - 1)) {
     if (cs) atomicAdd(dup, (unsigned long long)cs);
     if (cd) atomicAdd(dup + 1, (unsigned long long)cd);
-    if (cr) atomicOr(reinterpret_cast<unsigned int *>(dup + 2), 1u);
+    if (cr) atomicOr(reinterpret_cast<unsigned int *>(dup + 2), cl ? 3u : 1u);
   }
 }
 

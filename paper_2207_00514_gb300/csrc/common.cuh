@@ -13,6 +13,8 @@ constexpr uint32_t kInvalid = 0xFFFFFFFFu;   // no label / no neighbour
 constexpr uint32_t kLeafBit = 0x80000000u;   // child reference of a leaf
 constexpr uint32_t kNoBound = 0xFFFFFFFFu;   // "+inf" in the u32 radius arrays
 constexpr uint64_t kEmptyKey = ~0ull;        // empty per-component minimum
+constexpr int kTieRunMax = 64;               // edges of equal key that the output orders in place
+constexpr int kGroupLong = kTieRunMax + 1;   // equal codes that far apart: a longer run is likely
 
 // The minimum outgoing edge of a component (A8) as one 128-bit key, ordered
 // as the pair (key, mx): key = (w bits << 32) | min original id (w >= 0, so
@@ -231,6 +233,7 @@ struct Problem {
   uint32_t *seen = nullptr;          // count runs: bitmap of the internal nodes visited this round
   bool ties = true;                  // the search needs its tie rule (a run of > 32 equal
                                      // codes exists; set after the build, true when unknown)
+  bool long_group = false;           // more than kTieRunMax + 1 points share a code
   bool want_near = false;            // set before layout(): carve the near lists
   uint4 *near_j = nullptr;           // n: each point's nearest points, by curve index
   float4 *near_w = nullptr;          // n: their weights

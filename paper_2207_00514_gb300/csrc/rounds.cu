@@ -1295,8 +1295,6 @@ void launch_fill_u32(Problem &P, uint32_t *p, uint32_t v, int64_t count) {
 // the full path: a stable sort by j, then a stable sort by (w, i) (and by
 // instance in the batched form, which always takes it), then a gather.
 // ---------------------------------------------------------------------------
-constexpr int kTieRunMax = 64;
-
 __global__ void k_edge_keys_wi(const emst_edge *__restrict__ edges, int64_t m,
                                uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
                                int shift_i, ClearWords clear, uint32_t *long_runs) {
