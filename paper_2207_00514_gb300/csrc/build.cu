@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kBlock) k_morton128(const float *__restrict__ 
   wait_for_previous();
   clear_words(clear);
   // the FP64 divisions once per CTA (this GPU has few FP64 units: a division
-  // per point and axis took 190 us for 2M points, this 40)
+  // per point and axis took 190 us for 2M points, this 65)
   __shared__ double s_lo[3], s_scale[3];
   constexpr int B = DIM == 3 ? 42 : 64;
   const double twoB = DIM == 3 ? 4398046511104.0 : 18446744073709551616.0;  // 2^B
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kBlock) k_gather(const float *__restrict__ pts
     longer = run && k >= kGroupLong && equal_codes(k - kGroupLong);
   }
   // one atomic per CTA and counter (one per warp, all on the same words, made
-  // this pass ten times as long on dense clusters: 95 -> 14 us for 2M points)
+  // this pass three times as long on dense clusters: 95 -> 32 us for 2M points)
   const int cs = __syncthreads_count(same), cd = __syncthreads_count(differ);
   const int cr = __syncthreads_or(run) ? (__syncthreads_or(longer) ? 3 : 1) : 0;
   if (threadIdx.x == 0) {
