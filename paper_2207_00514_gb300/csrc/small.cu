@@ -65,7 +65,8 @@ struct SmallArgs {
 // The curve key of a point: the 128-bit Z-curve code of build.cu (42 bits per
 // axis in 3D, 64 in 2D, quantised in FP64) with its lowest 16 bits replaced
 // by the point's index, which makes the keys distinct.
-__device__ __forceinline__ Key curve_key(const float (&x)[3], const float *lo, const float *hi, int dim,
+// lo, scale: the box's lower corner and 2^bits / extent (0 for a flat axis).
+__device__ __forceinline__ Key curve_key(const float (&x)[3], const double *lo, const double *scale, int dim,
                                          uint32_t idx) {
   const double twoB = dim == 3 ? 4398046511104.0 : 18446744073709551616.0;
   const uint64_t qmax = dim == 3 ? ((1ull << 42) - 1ull) : ~0ull;
@@ -73,9 +74,7 @@ __device__ __forceinline__ Key curve_key(const float (&x)[3], const float *lo, c
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (d >= dim) continue;
-    const double l = (double)lo[d], ext = __dsub_rn((double)hi[d], l);
-    const double sc = ext > 0.0 ? __ddiv_rn(twoB, ext) : 0.0;
-    const double t = __dmul_rn(__dsub_rn((double)x[d], l), sc);
+    const double t = __dmul_rn(__dsub_rn((double)x[d], lo[d]), scale[d]);
     q[d] = t >= twoB ? qmax : (uint64_t)t;
   }
   Key k;
@@ -93,10 +92,37 @@ __device__ __forceinline__ Key curve_key(const float (&x)[3], const float *lo, c
   return k;
 }
 
-// Bitonic sort of the first `size` (a power of two) keys of s, by the CTA.
+__device__ __forceinline__ Key shfl_xor_key(const Key &k, int j) {
+  Key r;
+  r.hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)k.hi, j);
+  r.lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)k.lo, j);
+  return r;
+}
+
+// Bitonic sort of the first `size` (a power of two, at least 32) keys of s, by
+// the CTA.  The steps over distances below 32 stay in a warp's registers: 21
+// barriers instead of 55 for 1,024 keys.
 __device__ __forceinline__ void tile_sort(Key *s, int size) {
-  for (int k = 2; k <= size; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
+  const int lane = threadIdx.x & 31;
+  // the steps k = k0 .. k1 over distances 16 .. 1, on rows of 32 keys
+  auto rows = [&](int k0, int k1) {
+    __syncthreads();
+    for (int r = (int)threadIdx.x >> 5; r < size / 32; r += kWarpsPerCta) {
+      const int e = r * 32 + lane;
+      Key x = s[e];
+      for (int k = k0; k <= k1; k <<= 1) {
+        for (int j = k / 2 < 16 ? k / 2 : 16; j > 0; j >>= 1) {
+          const Key y = shfl_xor_key(x, j);
+          const bool keep_small = ((e & k) == 0) == ((lane & j) == 0);
+          if (key_less(y, x) == keep_small) x = y;
+        }
+      }
+      s[e] = x;
+    }
+  };
+  rows(2, 32);
+  for (int k = 64; k <= size; k <<= 1) {
+    for (int j = k >> 1; j >= 32; j >>= 1) {
       __syncthreads();
       for (int t = threadIdx.x; t < size / 2; t += kThreads) {
         const int a = ((t & ~(j - 1)) << 1) | (t & (j - 1)), b = a | j;
@@ -107,6 +133,7 @@ __device__ __forceinline__ void tile_sort(Key *s, int size) {
         }
       }
     }
+    rows(k, k);
   }
   __syncthreads();
 }
@@ -297,9 +324,11 @@ __device__ __forceinline__ void write_box(const SmallArgs &A, int first, int row
 __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Key *s_keys = reinterpret_cast<Key *>(smem_raw);
-  __shared__ float s_box[6];
+  uint4 *todo = reinterpret_cast<uint4 *>(smem_raw);  // (between the sorts: at most 32 entries per warp)
+  __shared__ double s_lo[3], s_scale[3];
   __shared__ uint32_t s_cnt[kWarpsPerCta];
   __shared__ uint32_t s_base;
+  __shared__ int s_todo, s_taken;
   const float kInf = __int_as_float(0x7f800000);
   const int tid = threadIdx.x, lane = tid & 31;
   const int gtid = blockIdx.x * kThreads + tid, gthreads = gridDim.x * kThreads;
@@ -339,9 +368,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
   if (!grid_barrier(bar, status, phase)) return;
   if (__ldcg(status) != 0u) return;  // non-finite input: the same value for every CTA
   const float *src = A.copy ? A.copy : A.src;
-  if (tid < 3) {
-    s_box[tid] = tid < dim ? ordered_to_float(~__ldcg(counters + 2 + tid)) : 0.f;
-    s_box[3 + tid] = tid < dim ? ordered_to_float(__ldcg(counters + 5 + tid)) : 0.f;
+  if (tid < dim) {  // (the FP64 divisions here, not per point: few FP64 units)
+    const double twoB = dim == 3 ? 4398046511104.0 : 18446744073709551616.0;
+    const double lo = (double)ordered_to_float(~__ldcg(counters + 2 + tid));
+    const double ext = __dsub_rn((double)ordered_to_float(__ldcg(counters + 5 + tid)), lo);
+    s_lo[tid] = lo;
+    s_scale[tid] = ext > 0.0 ? __ddiv_rn(twoB, ext) : 0.0;
   }
   __syncthreads();
 
@@ -349,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
   const int tile = A.tile, ntiles = (n + tile - 1) / tile;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int begin = t * tile, cnt = n - begin < tile ? n - begin : tile;
-    int size = 2;
+    int size = 32;
     while (size < cnt) size <<= 1;
     for (int i = tid; i < size; i += kThreads) {
       Key k = {~0ull, ~0ull};
@@ -359,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
 #pragma unroll
         for (int q = 0; q < 3; ++q)
           if (q < dim) x[q] = src[idx * dim + q];
-        k = curve_key(x, s_box, s_box + 3, dim, (uint32_t)idx);
+        k = curve_key(x, s_lo, s_scale, dim, (uint32_t)idx);
       }
       s_keys[i] = k;
     }
@@ -419,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
   int limit = 1;
   while ((1 << (limit - 1)) < n) ++limit;  // ceil(log2 n) + 1
   ++limit;
-  // curve positions a warp settles together (their searches run one by one)
+  // curve positions a warp looks at together
   int chunk = (n + gwarps - 1) / gwarps;
   if (chunk > 32) chunk = 32;
   for (int round = 0;; ++round) {
@@ -431,12 +463,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
     const uint32_t *labels = A.labels[cur];
     const uint32_t *bound = A.bound[cur];
     CompBest *comp = A.comp[cur];
-    // queries
-    for (int i0 = gwarp * chunk; i0 < n; i0 += gwarps * chunk) {
-      const int i = i0 + lane;
+    // queries: every warp looks at its positions, the CTA's warps share those
+    // that need a search (neighbours on the curve often all do, or none)
+    for (int base = 0; base < n; base += gwarps * chunk) {
+      const int i = base + gwarp * chunk + lane;
+      bool act = false;
       uint32_t me = 0;
       uint2 prev = make_uint2(0u, kInvalid);
-      bool act = false;
       if (lane < chunk && i < n) {
         me = labels[i];
         if (round > 0) prev = A.res[i];
@@ -453,26 +486,36 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
           }
         }
       }
-      unsigned todo = __ballot_sync(0xffffffffu, act);
-      while (todo) {
-        const int l = __ffs(todo) - 1;
-        todo &= todo - 1u;
-        const int q = i0 + l;
-        const uint32_t qme = __shfl_sync(0xffffffffu, me, l);
-        const uint32_t qlb = __shfl_sync(0xffffffffu, prev.x, l);
-        const uint32_t r0 = __shfl_sync(0xffffffffu, min(bound[qme], best_weight(comp + qme)), 0);
-        if (qlb > r0) continue;
+      if (tid == 0) s_todo = s_taken = 0;
+      __syncthreads();
+      const unsigned b = __ballot_sync(0xffffffffu, act);
+      int at = 0;
+      if (lane == 0 && b) at = atomicAdd(&s_todo, __popc(b));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
+      if (act) todo[at] = make_uint4((uint32_t)i, me, prev.x, 0u);
+      __syncthreads();
+      const int count = s_todo;
+      for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(&s_taken, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= count) break;
+        const uint4 e = todo[t];
+        const int q = (int)e.x;
+        const uint32_t r0 = __shfl_sync(0xffffffffu, min(bound[e.y], best_weight(comp + e.y)), 0);
+        if (e.z > r0) continue;
         const float4 p = A.pts[q];
-        const Found f = warp_search(A, labels, p, qme, r0);
+        const Found f = warp_search(A, labels, p, e.y, r0);
         if (lane == 0) {
           // nothing within r0: the smallest rejected bound is a lower bound of
           // the nearest other component from here on
           const uint32_t lb = f.lb != kNoBound ? f.lb : (r0 != kNoBound ? r0 : 0u);
           A.res[q] = make_uint2(f.j != kInvalid ? f.w : lb, f.j);
-          if (f.j != kInvalid) offer(comp + qme, f.w, __float_as_uint(p.w), f.id, labels[f.j], status);
+          if (f.j != kInvalid) offer(comp + e.y, f.w, __float_as_uint(p.w), f.id, labels[f.j], status);
         }
         __syncwarp();
       }
+      __syncthreads();
     }
     if (!grid_barrier(bar, status, phase)) return;
     // merge: one thread per component (a label is the position of one of its points)
@@ -567,7 +610,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_small(SmallArgs A) {
   const int m = n - 1;
   for (int t = blockIdx.x; t < (m + tile - 1) / tile; t += gridDim.x) {
     const int begin = t * tile, cnt = m - begin < tile ? m - begin : tile;
-    int size = 2;
+    int size = 32;
     while (size < cnt) size <<= 1;
     for (int i = tid; i < size; i += kThreads) {
       Key k = {~0ull, ~0ull};
