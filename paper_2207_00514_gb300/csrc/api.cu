@@ -110,9 +110,15 @@ struct Mailbox {
   uint32_t *words = nullptr;  // kMailWords, then the sequence number of the last post
   uint32_t seq = 0;
   bool open() {
-    if (!words && cudaHostAlloc((void **)&words, 4096, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-      cudaGetLastError();
-      words = nullptr;
+    if (!words) {
+      // (another thread's stream may be under capture: the allocation is no part of it)
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (cudaHostAlloc((void **)&words, 4096, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        words = nullptr;
+      }
+      cudaThreadExchangeStreamCaptureMode(&mode);
     }
     if (words && seq == 0) std::memset(words, 0, 4096);
     return words != nullptr;
