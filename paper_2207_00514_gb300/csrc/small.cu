@@ -13,11 +13,13 @@
 // traverse.cuh).  The tree is unique under the total order (w, i, j), so it
 // does not depend on the hierarchy.
 //
-// What bounds it: the latency of dependent L2 accesses and of the barriers.
-// Measured (us per call, general path / this one): 333 points 540 / 116,
-// 10,000 uniform 920 / 368, 16,384 970-1100 / 340-490, 30,000 1080-1250 /
-// 620-980 by shape and dimension; at 65,536 they meet (1120-1430 / 920-1530),
-// so the limit lies at half that.
+// What bounds it: the latency of dependent L2 accesses, of the barriers (four
+// and three a round, 1-2 us each) and, from some thousand points on, of the
+// tile sorts (7 us each for 1,024 keys).  Measured (us per call, general path
+// / this one): 333 points 345 / 113, 10,000 496-532 / 251-262, 16,384 512-611 /
+// 290-338, 30,000 576-611 / 443-478, 32,768 552-657 / 445-517 by shape and
+// dimension: they meet not far above, and a point's index has 16 bits in the
+// sort keys.
 #include <cstring>
 
 #include "grid.cuh"
