@@ -33,16 +33,14 @@ METRIC = "EMST Mpoints/s at 37M 3D clustered, plain vs learned-radius; % HBM roo
 WORKLOAD = ("37,000,000 FP32 3D points: 80% in NFW halos (power-law member counts m^-1.9 on "
             "[10, 1e5], c = 5, r_vir = 0.01 (m/1e5)^(1/3)), 20% uniform, unit box, seed 2")
 # DRAM bytes (read + write) of each round's traversal on this workload (37M
-# halo points, seed 2): its k_traverse launch, plus from round 2 on the
-# k_active launches that list the queries to search (inside the round's CUDA
-# events), from one ncu capture of one whole call of the kernels as they are
-# now:
+# halo points, seed 2): the launches inside the round's CUDA events (k_near;
+# k_settle, k_active* and k_traverse), from one ncu capture of one whole call
+# of the kernels as they are now:
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
-#       --clock-control none -k regex:"k_traverse|k_active" -c 24 --csv
+#       --clock-control none -k regex:"k_near|k_settle|k_traverse|k_active" --csv
 #       python bench.py --workload once
-# (one pass per launch).  Set back to None whenever those kernels change.
-TRAVERSE_DRAM_BYTES_PER_ROUND = [5220.5e6, 6216.1e6, 6480.0e6, 3833.9e6, 1894.4e6, 1398.3e6,
-                                 818.0e6, 537.6e6, 472.7e6, 455.1e6, 444.7e6]
+# (one pass per launch).  None: not captured since those kernels changed.
+TRAVERSE_DRAM_BYTES_PER_ROUND = None
 PAPER_CONTEXT = ("paper: Hacc37M (real 37M 3D cosmology points) on one A100 in < 0.5 s, best-case "
                  "270 MFeatures/s ~ 90 Mpoints/s; other data, other GPU: context only")
 
@@ -157,32 +155,33 @@ def measured_peaks():
 
 # Algorithmic bytes of one traversal launch (Algorithm 2 over every point), by
 # what the method must read or write at least once:
-#  round 0 (every label is the point's own index, every query searches):
-#    per query 56 B -- its point (16), label (4), component bound (4), the
-#    component's best so far (8), its result (8), the update of the
-#    component's 16-byte (w, min id, max id, outside label) minimum (16) --
-#    and per distinct internal node visited its 64-B record;
-#  later rounds: per point 24 B to decide whether to search at all -- label
-#    (4), component bound (4) and best so far (8), its previous result (8)
-#    (a skipped query rewrites its result only when it held a neighbour,
-#    not counted) -- plus per query that searches 44 B -- its point (16),
-#    its previous neighbour's label (4), its new result (8), the minimum's
-#    update (16) -- and per distinct internal node visited 72 B: the record
-#    (64) and its child labels (8).
-BYTES_FIRST_QUERY = 56
-BYTES_POINT = 24
+#  round 0 (every label is the point's own index, every query searches and
+#    leaves its four nearest points): per query 72 B -- its point (16), its
+#    list (32), its result (8), its component's 16-byte (w, min id, max id,
+#    outside label) minimum (16) -- and per distinct internal node visited its
+#    64-B record;
+#  later rounds: per point 12 B to decide whether to search at all -- its label
+#    (4) and previous result (8) (a skipped query rewrites its result only when
+#    it held a neighbour, not counted) -- per component its bound (4) and best
+#    so far (8), plus per query that searches 44 B -- its point (16), its
+#    previous neighbour's label (4), its new result (8), the minimum's update
+#    (16) -- and per distinct internal node visited 72 B: the record (64) and
+#    its child labels (8).
+BYTES_FIRST_QUERY = 72
+BYTES_POINT = 12
+BYTES_COMPONENT = 12
 BYTES_SEARCH = 44
 BYTES_RECORD_FIRST = 64
 BYTES_RECORD = 72
 
 
-def traversal_round_bytes(n: int, queries, distinct):
+def traversal_round_bytes(n: int, queries, distinct, components):
     out = []
-    for r, (q, d) in enumerate(zip(queries, distinct)):
+    for r, (q, d, c) in enumerate(zip(queries, distinct, components)):
         if r == 0:
             out.append(float(q * BYTES_FIRST_QUERY + d * BYTES_RECORD_FIRST))
         else:
-            out.append(float(n * BYTES_POINT + q * BYTES_SEARCH + d * BYTES_RECORD))
+            out.append(float(n * BYTES_POINT + c * BYTES_COMPONENT + q * BYTES_SEARCH + d * BYTES_RECORD))
     return out
 
 
@@ -651,7 +650,7 @@ def main():
     torch.cuda.synchronize(dev)
     same_counted = bool(torch.equal(out, ref_edges))
     peak, peak_kind = measured_peaks()
-    rb = traversal_round_bytes(n, vis["round_queries"], vis["round_distinct_nodes"])
+    rb = traversal_round_bytes(n, vis["round_queries"], vis["round_distinct_nodes"], vis["components_per_round"])
     rr = min(len(rb), len(round_ms))
     tot_bytes, tot_ms = sum(rb[:rr]), sum(round_ms[:rr])
     achieved = tot_bytes / (tot_ms / 1e3) / 1e9 if tot_ms > 0 else 0.0
@@ -670,7 +669,7 @@ def main():
     if measured:
         per_round["dram_bytes"] = measured
         per_round["dram_over_algorithmic"] = [round(d / b, 3) for d, b in zip(measured, rb)]
-    roofline = {"bound": "hbm", "kernel": "k_traverse (Algorithm 2 queries, one thread per point)",
+    roofline = {"bound": "hbm", "kernel": "k_near and k_traverse (Algorithm 2 queries, one thread per point)",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic,
                 "peak_kind": (f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs copy)" if peak_kind == "measured"
@@ -678,7 +677,7 @@ def main():
                 "avg_launch_ms": tot_ms / max(rr, 1), "launches": rr,
                 "algorithmic_bytes_per_launch": tot_bytes / max(rr, 1),
                 "bytes_model": (f"round 0: {BYTES_FIRST_QUERY} B per query + {BYTES_RECORD_FIRST} B per distinct "
-                                f"internal node visited; later rounds: {BYTES_POINT} B per point + "
+                                f"internal node visited; later rounds: {BYTES_POINT} B per point + {BYTES_COMPONENT} B per component + "
                                 f"{BYTES_SEARCH} B per query that searches + {BYTES_RECORD} B per distinct "
                                 "internal node visited (counted by an instrumented call); time = the "
                                 "round's traversal CUDA events in the timed calls"),
