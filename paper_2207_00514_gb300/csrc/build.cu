@@ -11,6 +11,41 @@ constexpr int kBlock = 256;
 // A1. Scene box: per-dimension min / max of all coordinates, plus a flag for
 // any non-finite coordinate.  box[0..2] = ordered min, box[3..5] = ordered max.
 // ---------------------------------------------------------------------------
+// A CTA's box into the scene box: one atomic per bound (one per warp, all on
+// the same few words, made up most of the pass: 200,000 points 20 -> 3.5 us).
+template <int DIM>
+__device__ __forceinline__ void box_result(const float (&lo)[3], const float (&hi)[3], bool bad,
+                                           uint32_t *box, uint32_t *status) {
+  __shared__ uint32_t s_part[kBlock / 32][6];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < DIM; ++q) {  // (an empty range, +inf > -inf, is the neutral one)
+    const uint32_t l = __reduce_min_sync(0xffffffffu, float_to_ordered(lo[q]));
+    const uint32_t h = __reduce_max_sync(0xffffffffu, float_to_ordered(hi[q]));
+    if (lane == 0) {
+      s_part[warp][q] = l;
+      s_part[warp][3 + q] = h;
+    }
+  }
+  const bool any_bad = __syncthreads_or(bad);
+  if (threadIdx.x < 2 * DIM) {
+    const int q = threadIdx.x % DIM;
+    const bool upper = threadIdx.x >= DIM;
+    uint32_t v = s_part[0][upper ? 3 + q : q];
+    for (int w = 1; w < kBlock / 32; ++w) {
+      const uint32_t x = s_part[w][upper ? 3 + q : q];
+      v = upper ? max(v, x) : min(v, x);
+    }
+    // (a CTA without a finite coordinate on this axis leaves the box alone)
+    if (upper) {
+      if (v != float_to_ordered(-INFINITY)) atomicMax(&box[3 + q], v);
+    } else if (v != float_to_ordered(INFINITY)) {
+      atomicMin(&box[q], v);
+    }
+  }
+  if (any_bad && threadIdx.x == 0) atomicOr(status, kErrNonFinite);
+}
+
 // COPY: the points are read from pinned host memory through its device
 // mapping and written to `copy` (device) on the way, so the host-to-device
 // transfer of a host input is this pass itself.
@@ -43,23 +78,7 @@ __global__ void __launch_bounds__(kBlock) k_scene_box(const float *__restrict__ 
     take(k + 3 * stride);
   }
   for (; k < n; k += stride) take(k);
-#pragma unroll
-  for (int q = 0; q < DIM; ++q) {
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[q] = fminf(lo[q], __shfl_xor_sync(0xffffffffu, lo[q], o));
-      hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
-    }
-  }
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int q = 0; q < DIM; ++q) {
-      if (lo[q] <= hi[q]) {
-        atomicMin(&box[q], float_to_ordered(lo[q]));
-        atomicMax(&box[3 + q], float_to_ordered(hi[q]));
-      }
-    }
-  }
-  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, kErrNonFinite);
+  box_result<DIM>(lo, hi, bad, box, status);
 }
 
 // The COPY form reading 16 bytes per load (the host input through its
@@ -113,23 +132,7 @@ __global__ void __launch_bounds__(kBlock) k_scene_box_copy4(const float4 *__rest
       take(s1[t], (int)((4 * nv + t) % DIM));
     }
   }
-#pragma unroll
-  for (int q = 0; q < DIM; ++q) {
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[q] = fminf(lo[q], __shfl_xor_sync(0xffffffffu, lo[q], o));
-      hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
-    }
-  }
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int q = 0; q < DIM; ++q) {
-      if (lo[q] <= hi[q]) {
-        atomicMin(&box[q], float_to_ordered(lo[q]));
-        atomicMax(&box[3 + q], float_to_ordered(hi[q]));
-      }
-    }
-  }
-  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, kErrNonFinite);
+  box_result<DIM>(lo, hi, bad, box, status);
 }
 
 // All counters to zero, the scene box (4..9) empty: the call's first kernel.
