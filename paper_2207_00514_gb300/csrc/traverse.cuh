@@ -165,7 +165,7 @@ __device__ __forceinline__ uint32_t visit(Query &q, uint32_t node,
   // and so does a group at one equal distance from the query.  (Checked
   // only when a tie occurs; a leaf resolves its own ties.)
   // (the ids are read again in the rare tie case: kept live through the
-  // leaf scans above they cost the hot loop a register it does not have)
+  // leaf scans above they cost the hot loop a register)
   // Only when the input has a run of more than 32 equal codes (`ties`):
   // otherwise no group of identical points is larger than that, a tie
   // involves a few points at most and the check would only cost time.
@@ -268,7 +268,7 @@ __device__ __forceinline__ bool explore(Query &q, uint32_t node, const NodeRec *
     // and so does a group at one equal distance from the query.  (Checked
     // only when a tie occurs; a leaf resolves its own ties.)
     // (the ids are read again in the rare tie case: kept live through the
-    // leaf scans above they cost the hot loop a register it does not have)
+    // leaf scans above they cost the hot loop a register)
     // Only when the input has a run of more than 32 equal codes (`ties`):
     // otherwise no group of identical points is larger than that, a tie
     // involves a few points at most and the check would only cost time.
@@ -498,9 +498,9 @@ __device__ __forceinline__ void finish_query(const TravArgs &A, int64_t i, Query
 }
 
 // One query, start to finish (the one-thread-per-point form): the same
-// steps as start_query + explore + finish_query in one piece.  The kernel is
-// held to 32 registers, so nothing stays live through the search that can be
-// read again after it.
+// steps as start_query + explore + finish_query in one piece.  Registers are
+// few (EMST_TRAVERSE_MIN_BLOCKS), so nothing stays live through the search that
+// can be read again after it.
 // KEPT: a neighbour of an earlier round may still stand (keep_neighbour) and
 // settles the query; otherwise the caller has ruled that out (the listing
 // kernels settle those, and after the first round every neighbour has merged)
