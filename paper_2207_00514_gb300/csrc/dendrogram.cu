@@ -496,6 +496,297 @@ __global__ void k_dg_rows(const emst_edge *__restrict__ e, int64_t m,
   link[k] = make_uint4(min(c.x, c.y), max(c.x, c.y), __float_as_uint(e[k].w), size_out[k]);
 }
 
+// ---------------------------------------------------------------------------
+// A tree of at most kOneCtaEdges edges: the same contraction, chains, order and
+// totals by one CTA, everything but the edges and the result in shared memory,
+// in one launch.  What bounds a small tree is latency: over global memory,
+// with a grid barrier per step and a launch per sort pass, the contraction is
+// slower here than halving the ranks in shared memory was.  Random trees of
+// 300 / 1,000 / 2,000 / 4,096 edges, us a call: halving 114 / 129 / 153 / 182,
+// contraction in global memory 112 / 150 / 163 / 180, this 70 / 77 / 89 / 112
+// (paths 107 / 120 / 143 / 172, 122 / 168 / 183 / 193, 73 / 76 / 87 / 111).
+// It serves every size that fits: at the largest it still takes two thirds of
+// the other.
+// ---------------------------------------------------------------------------
+constexpr int kOneCtaEdges = 4096;  // the largest whose arrays fit (197 KB)
+constexpr int kOneCtaThreads = 1024;
+constexpr int kOneCtaLevels = 16;   // vertices halve: 13 reach 4,097
+constexpr uint32_t kSlotBits = 13;  // slots below 2 * kOneCtaEdges, chains below kOneCtaEdges + 1
+constexpr uint32_t kTook16 = 0x8000u;
+static_assert(2 * kOneCtaEdges <= 1 << kSlotBits && 2 * (kOneCtaEdges + 1) < (int)kTook16, "ids in 16 bits");
+
+// Where the one-CTA form's arrays lie in shared memory (byte offsets).
+struct OneCtaLayout {
+  int low, uf, total, done, rest[2], keys, vals, comp, bytes;
+  int padded;  // keys are sorted as a power of two
+  __host__ __device__ explicit OneCtaLayout(int n) {
+    const int m = n - 1;
+    padded = 32;
+    while (padded < m) padded <<= 1;
+    int off = 0;
+    auto take = [&](int b) {
+      const int at = off;
+      off = (off + b + 7) & ~7;
+      return at;
+    };
+    done = take(8 * m);
+    rest[0] = take(8 * (m / 2 + 1));  // (with rest[1]: the 2m child entries, 8m bytes, later on)
+    rest[1] = take(8 * (m / 2 + 1));
+    low = take(4 * 2 * n);
+    uf = take(4 * 2 * n);  // (the running totals later on)
+    total = take(4 * n);   // (the totals before each chain later on)
+    keys = take(4 * padded);
+    vals = take(4 * m);
+    comp = take(2 * 2 * n);
+    bytes = off;
+  }
+};
+
+// Ascending sort of s[0 .. size), a power of two of at least 32, by the CTA;
+// the steps over distances below 32 stay in a warp's registers.
+__device__ __forceinline__ void sort_words(uint32_t *s, int size) {
+  const int lane = threadIdx.x & 31;
+  auto rows = [&](int k0, int k1) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < size; e += blockDim.x) {
+      uint32_t x = s[e];
+      for (int k = k0; k <= k1; k <<= 1)
+        for (int j = k / 2 < 16 ? k / 2 : 16; j > 0; j >>= 1) {
+          const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+          x = ((e & k) == 0) == ((lane & j) == 0) ? min(x, y) : max(x, y);
+        }
+      s[e] = x;
+    }
+  };
+  rows(2, 32);
+  for (int k = 64; k <= size; k <<= 1) {
+    for (int j = k >> 1; j >= 32; j >>= 1) {
+      __syncthreads();
+      for (int t = threadIdx.x; t < size / 2; t += blockDim.x) {
+        const int a = ((t & ~(j - 1)) << 1) | (t & (j - 1)), b = a | j;
+        const uint32_t x = s[a], y = s[b];
+        if ((y < x) == ((a & k) == 0)) {
+          s[a] = y;
+          s[b] = x;
+        }
+      }
+    }
+    rows(k, k);
+  }
+  __syncthreads();
+}
+
+// blockDim: whole warps, at most kOneCtaThreads.  *status: the call's result,
+// written in any case.
+__global__ void __launch_bounds__(kOneCtaThreads, 1) k_dg_one_cta(const emst_edge *__restrict__ e, int n,
+                                                               uint4 *__restrict__ link,
+                                                               uint32_t *__restrict__ out_parent,
+                                                               uint32_t *status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint32_t c_done[kOneCtaLevels], c_rest[kOneCtaLevels], c_comp[kOneCtaLevels];
+  __shared__ uint32_t s_warp[kOneCtaThreads / 32];
+  const OneCtaLayout L(n);
+  // a row: x = rank, y = the vertices of its sides, 16 bits each, flagged kTook16
+  uint2 *done = reinterpret_cast<uint2 *>(smem_raw + L.done);
+  uint2 *rest[2] = {reinterpret_cast<uint2 *>(smem_raw + L.rest[0]), reinterpret_cast<uint2 *>(smem_raw + L.rest[1])};
+  uint32_t *low = reinterpret_cast<uint32_t *>(smem_raw + L.low);  // a vertex's lowest slot
+  uint32_t *uf = reinterpret_cast<uint32_t *>(smem_raw + L.uf);
+  uint32_t *total = reinterpret_cast<uint32_t *>(smem_raw + L.total);
+  uint32_t *keys = reinterpret_cast<uint32_t *>(smem_raw + L.keys);
+  uint32_t *vals = reinterpret_cast<uint32_t *>(smem_raw + L.vals);
+  uint16_t *comp = reinterpret_cast<uint16_t *>(smem_raw + L.comp);  // the component that holds a vertex
+  const int tid = threadIdx.x, lane = tid & 31, threads = blockDim.x;
+  const int m = n - 1;
+  const uint32_t lt = (1u << lane) - 1u;
+  auto place = [&](bool want, uint32_t *counter) {  // (whole warps call)
+    const unsigned b = __ballot_sync(0xffffffffu, want);
+    uint32_t at = 0;
+    if (lane == 0 && b) at = atomicAdd(counter, (uint32_t)__popc(b));
+    return __shfl_sync(0xffffffffu, at, 0) + __popc(b & lt);
+  };
+  for (int v = tid; v < 2 * n; v += threads) {
+    low[v] = kInvalid;
+    uf[v] = (uint32_t)v;
+  }
+  for (int v = tid; v < n; v += threads) total[v] = 0u;
+  if (tid < kOneCtaLevels) c_done[tid] = c_rest[tid] = c_comp[tid] = 0u;
+  __syncthreads();
+  uint32_t err = 0;
+  for (int k = tid; k < m; k += threads) {  // (k_dg_check)
+    const emst_edge x = e[k];
+    if (x.i >= (uint32_t)n || x.j >= (uint32_t)n || x.i == x.j || !(x.w == x.w) || (k + 1 < m && e[k + 1].w < x.w)) {
+      err = kErrBadInput;
+    } else {
+      atomicMin(low + x.i, 2u * (uint32_t)k);
+      atomicMin(low + x.j, 2u * (uint32_t)k + 1u);
+    }
+  }
+  int base = 0, nv = n, ne = m, dstart = 0, levels = 0;
+  while (!__syncthreads_or(err) && ne > 0 && levels < kOneCtaLevels) {
+    const int lv = levels++;
+    uint2 *from = rest[lv & 1], *next = rest[(lv + 1) & 1];
+    for (int b = 0; b < ne; b += threads) {
+      const int t = b + tid;
+      bool take = false, keep = false;
+      uint32_t rank = 0, u = 0, v = 0;
+      if (t < ne) {
+        if (lv == 0) {
+          rank = (uint32_t)t;
+          u = e[t].i;
+          v = e[t].j;
+        } else {
+          const uint2 row = from[t];
+          rank = row.x;
+          u = row.y & 0xffffu;
+          v = row.y >> 16;
+        }
+        const bool tu = low[u] >> 1 == rank, tv = low[v] >> 1 == rank;
+        take = tu || tv;
+        keep = !take;
+        if (take && !uf_unite(uf, u, v)) err = kErrSpin;
+        u |= tu ? kTook16 : 0u;
+        v |= tv ? kTook16 : 0u;
+      }
+      const uint32_t d = place(take, c_done + lv);
+      if (take) done[dstart + d] = make_uint2(rank, u | v << 16);
+      const uint32_t r = place(keep, c_rest + lv);
+      if (keep) {
+        if (r <= (uint32_t)m / 2) next[r] = make_uint2(rank, u | v << 16);
+        else err = kErrBadInput;  // more edges than half the vertices: not a tree
+      }
+    }
+    __syncthreads();
+    for (int b = 0; b < nv; b += threads) {
+      const int v = base + b + tid;
+      const bool in = b + tid < nv, root = in && uf[v] == (uint32_t)v;
+      const int g = base + nv + (int)place(root, c_comp + lv);
+      if (in && low[v] == kInvalid) err = kErrBadInput;  // a vertex without an edge: not a tree
+      if (root) {
+        if (g < 2 * n) comp[v] = (uint16_t)g;
+        else err = kErrBadInput;
+      }
+    }
+    if (__syncthreads_or(err)) break;
+    const int left = (int)c_rest[lv];
+    for (int t = tid; t < nv; t += threads) {
+      const uint32_t v = (uint32_t)(base + t), r = uf_find<true>(uf, v);
+      if (r != v) comp[v] = comp[r];
+    }
+    for (int t = tid; t < left; t += threads) {
+      const uint2 row = next[t];
+      uint32_t u = row.y & 0xffffu, v = row.y >> 16;
+      uf_find2<true>(uf, u, v);
+      if (u == v) {  // an edge inside a component: it closes a cycle
+        err = kErrBadInput;
+        continue;
+      }
+      u = comp[u];
+      v = comp[v];
+      next[t] = make_uint2(row.x, u | v << 16);
+      atomicMin(low + u, 2u * row.x);
+      atomicMin(low + v, 2u * row.x + 1u);
+    }
+    dstart += ne - left;
+    base += nv;
+    nv = (int)c_comp[lv];
+    ne = left;
+  }
+  if (ne > 0) err |= kErrBadInput;
+  if (__syncthreads_or(err)) {
+    // (every error is of the input but a spin that ran out)
+    const int spin = __syncthreads_or(err & kErrSpin);
+    if (tid == 0) *status = spin ? kErrSpin : kErrBadInput;
+    return;
+  }
+  // chains, level by level (totals of lower chains are complete)
+  int d0 = 0;
+  for (int lv = 0; lv < levels; ++lv) {
+    const int d1 = d0 + (int)c_done[lv];
+    for (int b = d0; b < d1; b += threads) {
+      const int t = b + tid;
+      uint32_t c = 0, w = 0;
+      if (t < d1) {
+        const uint2 row = done[t];
+        const bool tu = (row.y & kTook16) != 0u, tv = (row.y >> 16 & kTook16) != 0u;
+        const uint32_t u = row.y & (kTook16 - 1u), v = row.y >> 16 & (kTook16 - 1u);
+        auto points = [&](uint32_t g) { return g < (uint32_t)n ? 1u : total[g - n]; };
+        w = (tu ? points(u) : 0u) + (tv ? points(v) : 0u);
+        c = comp[u];
+        while (low[c] != kInvalid && low[c] >> 1 < row.x) c = comp[c];
+        c -= (uint32_t)n;
+        keys[row.x] = c << kSlotBits | (2u * row.x + (tu && !tv ? 1u : 0u));
+        vals[row.x] = w;
+      }
+      warp_add(total, c, w, t < d1);
+    }
+    d0 = d1;
+    __syncthreads();
+  }
+  for (int q = m + tid; q < L.padded; q += threads) keys[q] = ~0u;
+  sort_words(keys, L.padded);
+  // running totals over all chains, and what lies before each chain
+  uint32_t *run = uf, *before = total, *child = reinterpret_cast<uint32_t *>(smem_raw + L.rest[0]);
+  const uint32_t slot_mask = (1u << kSlotBits) - 1u;
+  {
+    const int per = (m + threads - 1) / threads, q0 = tid * per, q1 = min(q0 + per, m);
+    uint32_t sum = 0;
+    for (int q = q0; q < q1; ++q) sum += vals[(keys[q] & slot_mask) >> 1];
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[tid >> 5] = x;
+    __syncthreads();
+    uint32_t at = x - sum;
+    for (int w = 0; w < tid >> 5; ++w) at += s_warp[w];
+    for (int q = q0; q < q1; ++q) {
+      const uint32_t key = keys[q];
+      if (q == 0 || keys[q - 1] >> kSlotBits != key >> kSlotBits) before[key >> kSlotBits] = at;
+      at += vals[(key & slot_mask) >> 1];
+      run[(key & slot_mask) >> 1] = at;
+    }
+  }
+  __syncthreads();
+  // every cluster: its size, and the cluster it merges into (k_dg_finish)
+  for (int q = tid; q < m; q += threads) {
+    const uint32_t key = keys[q], chain = key >> kSlotBits, rank = (key & slot_mask) >> 1;
+    const bool last = q + 1 >= m || keys[q + 1] >> kSlotBits != chain;
+    const uint32_t ps = last ? low[n + chain] : keys[q + 1] & slot_mask;
+    run[rank] -= before[chain];
+    if (out_parent) out_parent[n + rank] = ps == kInvalid ? kInvalid : (uint32_t)n + (ps >> 1);
+    if (ps != kInvalid) child[ps] = (uint32_t)n + rank;
+  }
+  for (int v = tid; v < n; v += threads) {
+    if (out_parent) out_parent[v] = (uint32_t)n + (low[v] >> 1);
+    child[low[v]] = (uint32_t)v;
+  }
+  __syncthreads();
+  if (link)
+    for (int k = tid; k < m; k += threads) {
+      const uint32_t a = child[2 * k], b = child[2 * k + 1];
+      link[k] = make_uint4(min(a, b), max(a, b), __float_as_uint(e[k].w), run[k]);
+    }
+  if (tid == 0) *status = 0u;
+}
+
+cudaError_t launch_one_cta(const emst_edge *e, int n, uint4 *link, uint32_t *out_parent, uint32_t *status,
+                           cudaStream_t s) {
+  static bool attr_set[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 64 || !attr_set[dev]) {
+    const cudaError_t rc = cudaFuncSetAttribute(k_dg_one_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                OneCtaLayout(kOneCtaEdges + 1).bytes);
+    if (rc != cudaSuccess) return rc;
+    if (dev < 64) attr_set[dev] = true;
+  }
+  const int threads = n - 1 < kOneCtaThreads ? (n - 1 + 31) & ~31 : kOneCtaThreads;  // one per edge
+  k_dg_one_cta<<<1, threads, OneCtaLayout(n).bytes, s>>>(e, n, link, out_parent, status);
+  return cudaPeekAtLastError();
+}
+
 }  // namespace
 
 int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t *out_parent,
@@ -523,18 +814,20 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     off += bytes > 0 ? bytes : 1;
     return at;
   };
+  const bool one_cta = m <= kOneCtaEdges;  // its arrays are in shared memory
   const int64_t tiles = (m + kScanTile - 1) / kScanTile;
   // counters, per-level counters and totals first: cleared together
   const size_t o_counters = take(256), o_levels = take(4 * kMaxLevels * sizeof(uint32_t));
-  const size_t o_total = take(4 * (size_t)n), clear = off;
-  const size_t o_node = take(8 * (size_t)(2 * n)), o_uf = take(4 * (size_t)(2 * n));
-  const size_t o_rest0 = take(16 * (size_t)(m / 2 + 1)), o_rest1 = take(16 * (size_t)(m / 2 + 1));
-  const size_t o_done = take(16 * (size_t)m);
-  const size_t o_k0 = take(8 * (size_t)m), o_k1 = take(8 * (size_t)m);
-  const size_t o_v0 = take(4 * (size_t)m), o_v1 = take(4 * (size_t)m);
-  const size_t o_sort = take(4 * (size_t)sort_state_words(m));
-  const size_t o_child = take(out_link ? 8 * (size_t)m : 0);
-  const size_t o_tiles = take(8 * (size_t)tiles);
+  auto take_big = [&](size_t bytes) { return take(one_cta ? 0 : bytes); };
+  const size_t o_total = take_big(4 * (size_t)n), clear = off;
+  const size_t o_node = take_big(8 * (size_t)(2 * n)), o_uf = take_big(4 * (size_t)(2 * n));
+  const size_t o_rest0 = take_big(16 * (size_t)(m / 2 + 1)), o_rest1 = take_big(16 * (size_t)(m / 2 + 1));
+  const size_t o_done = take_big(16 * (size_t)m);
+  const size_t o_k0 = take_big(8 * (size_t)m), o_k1 = take_big(8 * (size_t)m);
+  const size_t o_v0 = take_big(4 * (size_t)m), o_v1 = take_big(4 * (size_t)m);
+  const size_t o_sort = take_big(4 * (size_t)sort_state_words(m));
+  const size_t o_child = take_big(out_link ? 8 * (size_t)m : 0);
+  const size_t o_tiles = take_big(8 * (size_t)tiles);
   const size_t o_edges = edges_dev ? 0 : take(sizeof(emst_edge) * (size_t)m);
   const size_t o_link = (out_link && !link_dev) ? take(16 * (size_t)m) : 0;
   const size_t o_pout = (out_parent && !par_dev) ? take(4 * (size_t)(n + m)) : 0;
@@ -563,22 +856,23 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
   A.out_parent = pout;
   A.child = link ? U(o_child) : nullptr;
   uint32_t *status = A.counters + 1;
+  bool ok = true;
+  if (!edges_dev)
+    ok = cudaMemcpyAsync((void *)e, edges, sizeof(emst_edge) * (size_t)m, cudaMemcpyHostToDevice, s) == cudaSuccess;
   // a cooperative grid: what is resident at once, or less for few edges
   static int ctas_per_sm[64] = {0};  // by device, looked up once (every thread finds the same)
   int dev = 0;
   cudaGetDevice(&dev);
   int occ = dev >= 0 && dev < 64 ? ctas_per_sm[dev] : 0;
-  bool ok = true;
-  if (occ == 0) {
-    ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dg_contract, kContractThreads, 0) == cudaSuccess &&
+  if (one_cta) ok = ok && launch_one_cta(e, (int)n, link, pout, status, s) == cudaSuccess;
+  if (occ == 0 && !one_cta) {
+    ok = ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dg_contract, kContractThreads, 0) == cudaSuccess &&
          occ >= 1;
     if (ok && dev >= 0 && dev < 64) ctas_per_sm[dev] = occ;
   }
-  if (ok) {
+  if (ok && !one_cta) {
     cudaMemsetAsync(base, 0, clear, s);
     cudaMemsetAsync(A.node, 0xff, 8 * (size_t)(2 * n), s);
-    if (!edges_dev)
-      cudaMemcpyAsync((void *)e, edges, sizeof(emst_edge) * (size_t)m, cudaMemcpyHostToDevice, s);
     k_dg_check<<<grid_for(n, kDgBlock), kDgBlock, 0, s>>>(e, m, n, A.node, A.uf, A.counters);
     int64_t g = (int64_t)sm_count() * occ;
     if (g > (n + kContractThreads - 1) / kContractThreads) g = (n + kContractThreads - 1) / kContractThreads;
@@ -586,7 +880,7 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     ok = cudaLaunchCooperativeKernel(k_dg_contract, dim3((unsigned)g), dim3(kContractThreads), args, 0, s) ==
          cudaSuccess;
   }
-  if (ok) {
+  if (ok && !one_cta) {
     Problem P;  // the sort's buffers
     P.stream = s;
     P.counters = A.counters;
@@ -605,6 +899,8 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     if (link)
       launch_next(P, k_dg_rows, grid_for(m, kDgBlock), kDgBlock, 0, e, m, size, reinterpret_cast<const uint2 *>(A.child), link, status);
     ok = cudaPeekAtLastError() == cudaSuccess;
+  }
+  if (ok) {
     if (out_link && !link_dev)
       cudaMemcpyAsync(out_link, link, 16 * (size_t)m, cudaMemcpyDeviceToHost, s);
     if (out_parent && !par_dev)
