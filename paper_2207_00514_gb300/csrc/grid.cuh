@@ -6,6 +6,7 @@
 namespace emst {
 
 constexpr int kBarrierSpins = 1 << 22;
+constexpr int kAcquirePolls = 8;
 
 // Every CTA adds one to *bar and waits for all of this phase's additions
 // (*bar starts at zero; `phase` counts the barriers passed).  The launch is
@@ -25,14 +26,24 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t *status, ui
       asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(bar) : "memory");
       v += 1u;
       int spins = 0;
+      // An acquiring load empties the SM's L1, so a CTA that waits long polls
+      // without: it made every step of a chain walk of another CTA an L2 access
+      // (30,000 points on a line through emst_compute 10,060 -> 4,170 us).  The
+      // first polls, which see the end of most waits, acquire: a fence after
+      // them instead cost 0.4 us a barrier (333 points 121 -> 132 us).
       while (v < target) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        if (spins < kAcquirePolls)
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        else
+          asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         if (++spins > kBarrierSpins) {
           atomicOr(status, kErrSpin);
           ok = 0;
           break;
         }
       }
+      if (spins > kAcquirePolls)
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
     }
     s_ok = ok;
   }
