@@ -452,6 +452,7 @@ void *mapped_host(const void *p);
 // Streaming multiprocessors of the current device (queried once per device):
 // grid caps of grid-stride kernels are multiples of it.
 int sm_count();
+int stream_sm_count(cudaStream_t s);
 // Stream-ordered scratch from the library's pool on the current device
 // (release with cudaFreeAsync on the same stream).
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);

@@ -874,11 +874,13 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     cudaMemsetAsync(base, 0, clear, s);
     cudaMemsetAsync(A.node, 0xff, 8 * (size_t)(2 * n), s);
     k_dg_check<<<grid_for(n, kDgBlock), kDgBlock, 0, s>>>(e, m, n, A.node, A.uf, A.counters);
-    int64_t g = (int64_t)sm_count() * occ;
+    int64_t g = (int64_t)stream_sm_count(s) * occ;
     if (g > (n + kContractThreads - 1) / kContractThreads) g = (n + kContractThreads - 1) / kContractThreads;
     void *args[] = {&A};
-    ok = cudaLaunchCooperativeKernel(k_dg_contract, dim3((unsigned)g), dim3(kContractThreads), args, 0, s) ==
-         cudaSuccess;
+    auto launch = [&](unsigned ctas) {
+      return cudaLaunchCooperativeKernel(k_dg_contract, dim3(ctas), dim3(kContractThreads), args, 0, s);
+    };
+    ok = launch_cooperative(g, launch) == cudaSuccess;
   }
   if (ok && !one_cta) {
     Problem P;  // the sort's buffers

@@ -51,4 +51,18 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t *status, ui
   return s_ok != 0;
 }
 
+// A cooperative launch of at most `grid` CTAs: launch(g) launches g of them.
+// Refused as too large (the GPU holds fewer at once than the caller counted,
+// as where the SMs are shared out under it) it is made again with half the
+// CTAs, down to one; the kernels work with any number.
+template <class Launch>
+cudaError_t launch_cooperative(int64_t grid, Launch &&launch) {
+  for (;;) {
+    const cudaError_t e = launch((unsigned)grid);
+    if (e != cudaErrorCooperativeLaunchTooLarge || grid <= 1) return e;
+    cudaGetLastError();
+    grid = (grid + 1) / 2;
+  }
+}
+
 }  // namespace emst

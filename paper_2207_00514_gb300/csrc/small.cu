@@ -705,7 +705,7 @@ int small_emst(const float *points, int64_t n64, int dim, emst_edge *out, cudaSt
   }
   if (ok) {
     // a warp per query while the GPU holds that many
-    int grid = sm_count() * occ;
+    int grid = stream_sm_count(stream) * occ;
     const int want = (n + kWarpsPerCta - 1) / kWarpsPerCta;
     if (grid > want) grid = want;
     ok = cudaMemsetAsync(A.counters, 0, 256, stream) == cudaSuccess;
@@ -713,8 +713,10 @@ int small_emst(const float *points, int64_t n64, int dim, emst_edge *out, cudaSt
       ok = ok && cudaMemcpyAsync(copy, points, sizeof(float) * (size_t)n * dim, cudaMemcpyHostToDevice,
                                  stream) == cudaSuccess;
     void *args[] = {&A};
-    ok = ok && cudaLaunchCooperativeKernel(k_small, dim3((unsigned)grid), dim3(kThreads), args, smem, stream) ==
-                   cudaSuccess;
+    auto launch = [&](unsigned g) {
+      return cudaLaunchCooperativeKernel(k_small, dim3(g), dim3(kThreads), args, smem, stream);
+    };
+    ok = ok && launch_cooperative(grid, launch) == cudaSuccess;
     if (ok && out_staged)
       ok = cudaMemcpyAsync(out, A.out, sizeof(emst_edge) * (size_t)(n - 1), cudaMemcpyDeviceToHost,
                            stream) == cudaSuccess;
