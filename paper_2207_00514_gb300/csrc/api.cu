@@ -776,7 +776,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     P.log_every = ex->log_every < 1 ? 1 : ex->log_every;
   }
   int64_t reruns = 0;
-  const size_t need = layout(P, nullptr, !pts_dev, !out_dev && !out_map);
+  size_t need = layout(P, nullptr, !pts_dev, !out_dev && !out_map);
   char *base = nullptr;
   uint32_t host_counters[kMailWords] = {0};
   uint64_t prev_visits = 0, prev_queries = 0, prev_distinct = 0;
@@ -786,7 +786,14 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
   cudaEvent_t lev[2 * 40] = {nullptr};  // learned: around the proposed-cutoff search
   cudaEvent_t cev[2] = {nullptr, nullptr};  // mutual reachability: around the core distances
   int n_tev = 0;
-  if (cudaMallocFromPoolAsync((void **)&base, need, pool, stream) != cudaSuccess) {
+  cudaError_t got = cudaMallocFromPoolAsync((void **)&base, need, pool, stream);
+  if (got != cudaSuccess && P.want_near) {  // the lists (32 bytes a point) can be done without
+    cudaGetLastError();
+    P.want_near = false;
+    need = layout(P, nullptr, !pts_dev, !out_dev && !out_map);
+    got = cudaMallocFromPoolAsync((void **)&base, need, pool, stream);
+  }
+  if (got != cudaSuccess) {
     cudaGetLastError();
     return EMST_ERR_OOM;
   }
