@@ -88,12 +88,11 @@ int sm_count() {
 }
 
 // The SMs that kernels on stream s can use: fewer than the device's where the
-// stream or the current context owns a partition of it (a green context).
+// stream belongs to a partition of it (a green context).
 int stream_sm_count(cudaStream_t s) {
   struct Driver {
     PFN_cuStreamGetCtx_v12050 stream_ctx = nullptr;
     PFN_cuGreenCtxGetDevResource_v12040 green_resource = nullptr;
-    PFN_cuCtxGetDevResource_v12040 ctx_resource = nullptr;
     Driver() {
       auto find = [](const char *name, void **f, unsigned version) {
         cudaDriverEntryPointQueryResult found;
@@ -105,20 +104,17 @@ int stream_sm_count(cudaStream_t s) {
       };
       find("cuStreamGetCtx", reinterpret_cast<void **>(&stream_ctx), 12050);
       find("cuGreenCtxGetDevResource", reinterpret_cast<void **>(&green_resource), 12040);
-      find("cuCtxGetDevResource", reinterpret_cast<void **>(&ctx_resource), 12040);
     }
   };
   static const Driver D;
   const int all = sm_count();
   CUcontext ctx = nullptr;
   CUgreenCtx green = nullptr;
+  // (asking an ordinary context for its SMs as well made a small call 2 us longer)
+  if (!D.stream_ctx || !D.green_resource || D.stream_ctx(s, &ctx, &green) != CUDA_SUCCESS || !green) return all;
   CUdevResource r;
   std::memset(&r, 0, sizeof(r));
-  if (!D.stream_ctx || !D.green_resource || !D.ctx_resource || D.stream_ctx(s, &ctx, &green) != CUDA_SUCCESS)
-    return all;
-  const CUresult e = green ? D.green_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM)
-                           : D.ctx_resource(ctx, &r, CU_DEV_RESOURCE_TYPE_SM);
-  const int own = e == CUDA_SUCCESS ? (int)r.sm.smCount : 0;
+  const int own = D.green_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS ? (int)r.sm.smCount : 0;
   return own >= 1 && own < all ? own : all;
 }
 
