@@ -133,45 +133,64 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
-// The calling thread's mailbox: a page of mapped host memory into which a
-// call's kernels post the counters the host needs between rounds (post_mail in
-// rounds.cu), so that a round costs the host a wait on one word instead of a
-// copy and a stream synchronisation (about 10 us per round, which at a
-// million points is a tenth of the call).  One per host thread, freed with it;
-// a call uses it only while it runs, and its sequence numbers never repeat.
+// A call's mailbox: a page of mapped host memory into which its kernels post
+// the counters the host needs between rounds (post_mail in rounds.cu), so that
+// a round costs the host a wait on one word instead of a copy and a stream
+// synchronisation (about 10 us per round, which at a million points is a tenth
+// of the call).  A page holds kMailWords counters, the sequence number of the
+// last post and, the host's alone, of the last one asked for; the numbers of a
+// page never repeat.  Pages are kept for later calls, as many as there were
+// calls at once, and never freed: a thread that ends must make no call that
+// waits for the device or that another thread's stream capture forbids.
 namespace {
-struct Mailbox {
-  uint32_t *words = nullptr;  // kMailWords, then the sequence number of the last post
-  uint32_t seq = 0;
-  bool open() {
-    if (!words) {
-      // (another thread's stream may be under capture: the allocation is no part of it)
-      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-      cudaThreadExchangeStreamCaptureMode(&mode);
-      if (cudaHostAlloc((void **)&words, 4096, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-        cudaGetLastError();
-        words = nullptr;
+std::mutex g_mail_mu;
+std::vector<uint32_t *> &free_mail() {  // (outlives every thread)
+  static std::vector<uint32_t *> *pages = new std::vector<uint32_t *>;
+  return *pages;
+}
+
+struct MailLease {
+  uint32_t *page = nullptr;  // null: no mapped memory
+  MailLease() {
+    {
+      std::lock_guard<std::mutex> lock(g_mail_mu);
+      if (!free_mail().empty()) {
+        page = free_mail().back();
+        free_mail().pop_back();
+        return;
       }
-      cudaThreadExchangeStreamCaptureMode(&mode);
     }
-    if (words && seq == 0) std::memset(words, 0, 4096);
-    return words != nullptr;
+    // (another thread's stream may be under capture: the allocation is no part of it)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (cudaHostAlloc((void **)&page, 4096, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      page = nullptr;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (page) std::memset(page, 0, 4096);
   }
-  ~Mailbox() {
-    if (words) cudaFreeHost(words);
+  ~MailLease() {
+    if (!page) return;
+    std::lock_guard<std::mutex> lock(g_mail_mu);
+    free_mail().push_back(page);
   }
+  MailLease(const MailLease &) = delete;
+  MailLease &operator=(const MailLease &) = delete;
 };
-thread_local Mailbox t_mailbox;
+
+// The number of the next post.
+uint32_t next_post(Problem &P) { return P.mail_seq = ++P.mail[kMailWords + 1]; }
 
 // Waits for the post `P.mail_seq` and copies it; false when the stream ends
 // (or fails) without it.
 bool wait_mail(Problem &P, uint32_t *out) {
-  const uint32_t *flag = t_mailbox.words + kMailWords;
+  const uint32_t *flag = P.mail + kMailWords;
   auto arrived = [&]() { return __atomic_load_n(flag, __ATOMIC_ACQUIRE) == P.mail_seq; };
   for (;;) {
     for (int k = 0; k < 4096; ++k)
       if (arrived()) {
-        std::memcpy(out, t_mailbox.words, sizeof(uint32_t) * kMailWords);
+        std::memcpy(out, P.mail, sizeof(uint32_t) * kMailWords);
         return true;
       }
     const cudaError_t q = cudaStreamQuery(P.stream);
@@ -185,7 +204,7 @@ bool wait_mail(Problem &P, uint32_t *out) {
 // The counters as the work on the stream so far leaves them (kMailWords).
 bool read_counters(Problem &P, uint32_t *out) {
   if (P.mail) {
-    P.mail_seq = ++t_mailbox.seq;
+    next_post(P);
     launch_post_mail(P);
     return cudaPeekAtLastError() == cudaSuccess && wait_mail(P, out);
   }
@@ -359,7 +378,7 @@ bool run_build(Problem &P, uint32_t *counters) {
     // the tree follows at once, and the counters travel meanwhile
     const bool ahead = P.auto_wide && P.mail && P.n >= 2;
     if (ahead) {
-      P.mail_seq = ++t_mailbox.seq;
+      next_post(P);
       launch_post_mail(P);
       launch_build_tree(P, true);
     }
@@ -782,6 +801,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
   cudaEvent_t lev[2 * 40] = {nullptr};  // learned: around the proposed-cutoff search
   cudaEvent_t cev[2] = {nullptr, nullptr};  // mutual reachability: around the core distances
   int n_tev = 0;
+  MailLease lease;
   cudaError_t got = cudaMallocFromPoolAsync((void **)&base, need, pool, stream);
   if (got != cudaSuccess && P.want_near) {  // the lists (32 bytes a point) can be done without
     cudaGetLastError();
@@ -794,7 +814,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
     return EMST_ERR_OOM;
   }
   layout(P, base, !pts_dev, !out_dev && !out_map);
-  if (t_mailbox.open()) P.mail = t_mailbox.words;  // (one address for host and device)
+  P.mail = lease.page;  // (one address for host and device)
   if (stats) tm.start(stream);
   if (pts_map) P.points_mapped = pts_map;  // copied by the scene-box pass
   else if (!pts_dev)
@@ -872,7 +892,7 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
         n_tev = rounds + 1;
       }
       if (count) launch_count_seen(P);
-      if (P.mail) P.mail_seq = ++t_mailbox.seq;  // posted by the merge's last kernel
+      if (P.mail) next_post(P);  // posted by the merge's last kernel
       launch_merge(P);
       advance_round(P, 0);
       // the next round's first kernel, before this one's outcome is known: the
@@ -938,7 +958,8 @@ int compute_impl(const float *points, int64_t n, int dim, const int64_t *offsets
   }
 done:
   // (a call that fails half way leaves no kernel behind that could still post)
-  if (rc != EMST_OK && P.mail) cudaStreamSynchronize(stream);
+  // -- and if that cannot be known, the mailbox is not used again
+  if (rc != EMST_OK && P.mail && cudaStreamSynchronize(stream) != cudaSuccess) lease.page = nullptr;
   cudaFreeAsync(base, stream);
   if (rc == EMST_ERR_CUDA) cudaGetLastError();
   if (stats) {
