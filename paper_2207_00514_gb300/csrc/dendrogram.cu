@@ -166,7 +166,8 @@ struct Contract {
   uint32_t *vals;      // m, by rank: points the edge adds to its chain
   uint32_t *child;     // 2m or null: the cluster on each slot
   uint32_t *out_parent;  // n + m or null
-  uint32_t *counters;  // [1] status, [2] invalid input found before the contraction, [40] barrier
+  uint32_t *counters;  // [1] status, [2] invalid input found before the contraction, [40] barrier,
+                       // [41] tiles finished
   uint32_t *per_level; // 4 x kMaxLevels: components, edges left, edges done, errors
 };
 
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(kContractThreads, 3) k_dg_contract(Contract A)
 }
 
 // The sorted edges' running totals along their chains, in tiles: first each
-// tile's total since its last chain start (and whether it has one) ...
+// tile's total since its last chain start (and whether it has one),
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kDgBlock * kScanItems;
 
@@ -425,17 +426,62 @@ __device__ __forceinline__ Segment scan_segments(Segment s, Segment &before) {
   return join(base, x);
 }
 
+// and with many tiles, by the last CTA to finish, what the chain that reaches
+// into each tile gathered in the tiles before it (in place of the tile's
+// total).  Few tiles look for it on their own, back to the last chain start:
+// some steps at most, where the scan takes 6 us of the launch's tail (5,000
+// edges 117 -> 124 us a call); of all tiles it would be quadratic when one
+// chain holds most edges (a path of 100M edges of rising weights 30.6 ms by
+// walks, 16.3 by the scan; of 30M 11.3 and 11.1).
+constexpr int64_t kWalkTiles = 1024;
 __global__ void __launch_bounds__(kDgBlock) k_dg_tiles(const uint64_t *__restrict__ keys,
                                                        const uint32_t *__restrict__ vals, int64_t m,
-                                                       uint2 *__restrict__ tiles, const uint32_t *status) {
+                                                       uint2 *tiles, uint32_t *finished,
+                                                       const uint32_t *status) {
   wait_for_previous();
   if (*status != 0u) return;
+  __shared__ bool s_last;
   uint64_t k[kScanItems + 1];
   uint32_t v[kScanItems], heads;
   const int64_t q0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanItems;
   Segment before;
   const Segment s = scan_segments(load_items(keys, vals, m, q0, k, v, heads), before);
   if (threadIdx.x == kDgBlock - 1) tiles[blockIdx.x] = make_uint2(s.sum, s.head ? 1u : 0u);
+  if (gridDim.x <= kWalkTiles) return;
+  if (threadIdx.x == kDgBlock - 1) {
+    __threadfence();
+    s_last = atomicAdd(finished, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // a run of tiles per thread, read eight at a time (this is the launch's tail)
+  constexpr int kAtOnce = 8;
+  const int64_t count = gridDim.x;
+  const int64_t chunk = ((count + kDgBlock - 1) / kDgBlock + kAtOnce - 1) / kAtOnce * kAtOnce;
+  const int64_t lo = (int64_t)threadIdx.x * chunk, hi = lo + chunk < count ? lo + chunk : count;
+  auto load = [&](int64_t t, Segment (&x)[kAtOnce]) {
+#pragma unroll
+    for (int u = 0; u < kAtOnce; ++u) {
+      const uint2 w = t + u < hi ? __ldcg(tiles + t + u) : make_uint2(0u, 0u);
+      x[u] = Segment{w.x, w.y != 0u};
+    }
+  };
+  Segment x[kAtOnce], mine = {0u, false};
+  for (int64_t t = lo; t < hi; t += kAtOnce) {
+    load(t, x);
+#pragma unroll
+    for (int u = 0; u < kAtOnce; ++u) mine = join(mine, x[u]);
+  }
+  scan_segments(mine, before);
+  for (int64_t t = lo; t < hi; t += kAtOnce) {
+    load(t, x);
+#pragma unroll
+    for (int u = 0; u < kAtOnce; ++u) {
+      if (t + u < hi) tiles[t + u].x = before.sum;
+      before = join(before, x[u]);
+    }
+  }
 }
 
 // ... then every cluster: its size, and the cluster it merges into.
@@ -455,8 +501,10 @@ __global__ void __launch_bounds__(kDgBlock) k_dg_finish(const uint64_t *__restri
   const int64_t q0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanItems;
   const Segment mine = load_items(keys, vals, m, q0, k, v, heads);
   // what the chain that reaches into this tile gathered in the tiles before:
-  // back to the last one with a chain start
-  if (threadIdx.x < 32) {
+  // there already, or in those back to the last one with a chain start
+  if (gridDim.x > kWalkTiles) {
+    if (threadIdx.x == 0) s_carry = __ldg(&tiles[blockIdx.x].x);
+  } else if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     uint32_t sum = 0;
     for (int64_t t = (int64_t)blockIdx.x - 1; t >= 0; t -= 32) {
@@ -895,7 +943,8 @@ int dendrogram_impl(const emst_edge *edges, int64_t n, uint4 *out_link, uint32_t
     const int src = radix_sort_pairs(P, m, 0, (bits_for(n - 1) + 7) / 8, 0, 32);
     uint2 *tile = reinterpret_cast<uint2 *>(base + o_tiles);
     uint32_t *size = link ? P.vals[src ^ 1] : nullptr;  // the sort's other buffer is free again
-    launch_next(P, k_dg_tiles, (unsigned)tiles, kDgBlock, 0, P.keys[src], P.vals[src], m, tile, status);
+    launch_next(P, k_dg_tiles, (unsigned)tiles, kDgBlock, 0, P.keys[src], P.vals[src], m, tile,
+                A.counters + 41, status);
     launch_next(P, k_dg_finish, (unsigned)tiles, kDgBlock, 0, P.keys[src], P.vals[src], m, n, tile, A.node, size,
                                                      A.child, pout, status);
     if (link)

@@ -72,3 +72,9 @@ def test_not_a_tree():
     bad(lambda e: e["w"].__setitem__(11, np.nan))
     bad(lambda e: e["w"].__setitem__(200, -1.0))
     check(good, 500)
+
+
+def test_one_chain_over_many_tiles():
+    # a path of rising weights is one chain: every tile of the running totals
+    # continues it, over more tiles than the scan takes in one step per thread
+    check(synth.tree_edges(4_500_000, 9, "path_sorted"), 4_500_000)
