@@ -965,6 +965,23 @@ __global__ void __launch_bounds__(kActiveThreads) k_active_write(const uint8_t *
 
 using TravKernel = void (*)(TravArgs, const uint32_t *, const uint32_t *);
 
+// The CTAs of `block` threads of kernel K that the GPU holds at once.
+template <TravKernel K>
+static int resident_ctas(int block) {
+  static int per_sm[64][kTraverseMaxBlock / 32 + 1];  // by device and warps, looked up once (every thread finds the same)
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int b = dev >= 0 && dev < 64 ? per_sm[dev][block / 32] : 0;
+  if (b == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, K, block, 0) != cudaSuccess || b < 1) {
+      cudaGetLastError();
+      b = 1;
+    }
+    if (dev >= 0 && dev < 64) per_sm[dev][block / 32] = b;
+  }
+  return b * sm_count();
+}
+
 static void launch_trav(TravKernel k, int g, int block, const Problem &P, const TravArgs &A,
                         const uint32_t *list, const uint32_t *list_count) {
   launch_next(P, k, g, block, 0, A, list, list_count);
@@ -1064,10 +1081,13 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     }
     list = active;
     list_count = active_count;
-    g = sm_count() * (2048 / block);  // one resident wave
     A.queue = P.counters + kActiveQueue;  // warps take the list in order
   }
-#define EMST_LAUNCH(...) launch_trav(k_traverse<__VA_ARGS__>, g, block, P, A, list, list_count)
+// (a listed launch: the CTAs the GPU holds at once, so that each warp's first
+// entries are searched at once)
+#define EMST_LAUNCH(...)                                                                                       \
+  launch_trav(k_traverse<__VA_ARGS__>, A.queue ? resident_ctas<k_traverse<__VA_ARGS__>>(block) : g, block, P, A, \
+              list, list_count)
 // a host flag as a template argument
 #define EMST_IF(flag, B, ...)       \
   do {                              \
