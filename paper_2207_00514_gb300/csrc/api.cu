@@ -632,16 +632,20 @@ namespace {
 
 struct Timer {
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-  bool on = false;
+  bool on = false, marked[4] = {false, false, false, false};
   void start(cudaStream_t s) {
     on = true;
     for (auto &e : ev) cudaEventCreate(&e);
-    cudaEventRecord(ev[0], s);
+    mark(0, s);
   }
-  void mark(int k, cudaStream_t s) { if (on) cudaEventRecord(ev[k], s); }
+  void mark(int k, cudaStream_t s) {
+    if (on) marked[k] = cudaEventRecord(ev[k], s) == cudaSuccess;
+  }
+  // (0 where the call ended before one of the two: asked for, the time of such
+  // a pair would leave an error behind that the thread's next call reports)
   float ms(int a, int b) {
     float t = 0.f;
-    if (on) cudaEventElapsedTime(&t, ev[a], ev[b]);
+    if (marked[a] && marked[b]) cudaEventElapsedTime(&t, ev[a], ev[b]);
     return t;
   }
   ~Timer() { for (auto &e : ev) if (e) cudaEventDestroy(e); }

@@ -1,0 +1,67 @@
+"""The general path at sizes that emst_compute gives to the one-launch path:
+with options given every size takes it.  Non-finite coordinates, which the
+scene box reports (per CTA, on every way it reads the points) before the tree
+that was launched meanwhile is used, call after call."""
+from __future__ import annotations
+
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def words(edges):
+    import paper_2207_00514_gb300 as pkg
+    torch.cuda.synchronize()
+    return pkg.edges_numpy(edges).view(np.uint32).reshape(-1, 3)
+
+
+def want(pts):
+    e = oracle.prim(pts) if len(pts) <= 4000 else oracle.kd_boruvka(pts, threads=os.cpu_count() or 4)
+    return e.view(np.uint32).reshape(-1, 3)
+
+
+# 3 * 1,001 and 2 * 40,001 coordinates leave a tail behind the copy's 16-byte loads
+@pytest.mark.parametrize("dim,n", [(3, 1001), (2, 40_001), (3, 300_003)])
+@pytest.mark.parametrize("where", ["first", "last", "last_cta", "middle"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_non_finite(dim, n, where, bad):
+    import paper_2207_00514_gb300 as pkg
+    pts = synth.uniform(n, dim, 3)
+    at = {"first": (0, 0), "last": (n - 1, dim - 1), "last_cta": ((n - 1) // 256 * 256, 1), "middle": (n // 2, 0)}
+    broken = pts.copy()
+    broken[at[where]] = bad
+    t = torch.from_numpy(broken)
+    good = torch.from_numpy(pts).cuda()
+    for points in (t.cuda(), t.pin_memory(), t):
+        for kw in ({}, dict(morton_bits=64), dict(morton_bits=128)):
+            with pytest.raises(pkg.EmstError) as e:
+                pkg.emst_compute_ex(points, **kw)
+            assert e.value.status == -2
+    # the next call on the stream is not touched by it
+    assert np.array_equal(words(pkg.emst_compute_ex(good)[0]), words(pkg.emst_compute(good)))
+
+
+def test_non_finite_batched():
+    import paper_2207_00514_gb300 as pkg
+    pts = synth.uniform(9001, 3, 4)
+    offsets = np.array([0, 1, 3000, 3000, 9001], dtype=np.int64)
+    for row in (0, 2999, 9000):
+        broken = pts.copy()
+        broken[row, 2] = np.nan
+        for points in (torch.from_numpy(broken).cuda(), torch.from_numpy(broken).pin_memory()):
+            with pytest.raises(pkg.EmstError) as e:
+                pkg.emst_compute_batched(points, offsets)
+            assert e.value.status == -2
+    edges, at = pkg.emst_compute_batched(torch.from_numpy(pts).cuda(), offsets)
+    got = words(edges)
+    for k in range(4):
+        part = pts[offsets[k]:offsets[k + 1]]
+        if len(part) > 1:
+            assert np.array_equal(got[at[k]:at[k + 1]], want(part))
