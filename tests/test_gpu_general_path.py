@@ -1,7 +1,9 @@
 """The general path at sizes that emst_compute gives to the one-launch path:
-with options given every size takes it.  Non-finite coordinates, which the
-scene box reports (per CTA, on every way it reads the points) before the tree
-that was launched meanwhile is used, call after call."""
+with options given every size takes it.  Whole trees against the oracle,
+bit-exact, among them the output's order on runs of equal weights and the
+fallback on runs too long for it; host buffers; and non-finite coordinates,
+which the scene box reports (per CTA, on every way it reads the points) before
+the tree that was launched meanwhile is used."""
 from __future__ import annotations
 
 import os
@@ -11,6 +13,7 @@ import pytest
 
 import oracle
 import synth
+from test_gpu_parity import EMST_CASES
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -25,6 +28,27 @@ def words(edges):
 def want(pts):
     e = oracle.prim(pts) if len(pts) <= 4000 else oracle.kd_boruvka(pts, threads=os.cpu_count() or 4)
     return e.view(np.uint32).reshape(-1, 3)
+
+
+@pytest.mark.parametrize("name,make", EMST_CASES, ids=[c[0] for c in EMST_CASES])
+def test_emst_matches_oracle(name, make):
+    import paper_2207_00514_gb300 as pkg
+    pts = np.ascontiguousarray(make(), dtype=np.float32)
+    t = torch.from_numpy(pts).cuda()
+    w = want(pts)
+    assert np.array_equal(words(pkg.emst_compute_ex(t)[0]), w)
+    assert np.array_equal(words(pkg.emst_compute_ex(t, morton_bits=128)[0]), w)
+
+
+@pytest.mark.parametrize("n,dim", [(20_000, 3), (4_999, 2), (5, 3)])
+def test_host_buffers(n, dim):
+    import paper_2207_00514_gb300 as pkg
+    pts = synth.halos(n, 5) if dim == 3 else synth.blobs(n, 2, 5)
+    w = want(pts)
+    assert np.array_equal(words(pkg.emst_compute_ex(torch.from_numpy(pts).pin_memory())[0]), w)
+    out = torch.empty((n - 1, 3), dtype=torch.int32)  # pageable
+    pkg.emst_compute_ex(torch.from_numpy(pts.copy()), out_edges=out)
+    assert np.array_equal(words(out), w)
 
 
 # 3 * 1,001 and 2 * 40,001 coordinates leave a tail behind the copy's 16-byte loads
