@@ -161,16 +161,19 @@ def measured_peaks():
 #    outside label) minimum (16) -- and per distinct internal node visited its
 #    64-B record;
 #  later rounds: per point 12 B to decide whether to search at all -- its label
-#    (4) and previous result (8) (a skipped query rewrites its result only when
-#    it held a neighbour, not counted) -- per component its bound (4) and best
-#    so far (8), plus per query that searches 44 B -- its point (16), its
-#    previous neighbour's label (4), its new result (8), the minimum's update
-#    (16) -- and per distinct internal node visited 72 B: the record (64) and
-#    its child labels (8).
+#    (4) and result (8) -- per component its bound (4) and best so far (8), plus
+#    per query that searches 40 B -- its point (16), its new result (8), the
+#    minimum's update (16) -- and per distinct internal node visited 72 B: the
+#    record (64) and its child labels (8);
+#  rounds 1 to 3 also, per point whose earlier neighbour no longer stands, its
+#    list: four ids (16), their labels (16) and weights (16).  In round 1 that is
+#    every point; in rounds 2 and 3 at least every one that searches (how many
+#    others their lists settled is not counted).
 BYTES_FIRST_QUERY = 72
 BYTES_POINT = 12
 BYTES_COMPONENT = 12
-BYTES_SEARCH = 44
+BYTES_LIST = 48
+BYTES_SEARCH = 40
 BYTES_RECORD_FIRST = 64
 BYTES_RECORD = 72
 
@@ -181,7 +184,9 @@ def traversal_round_bytes(n: int, queries, distinct, components):
         if r == 0:
             out.append(float(q * BYTES_FIRST_QUERY + d * BYTES_RECORD_FIRST))
         else:
-            out.append(float(n * BYTES_POINT + c * BYTES_COMPONENT + q * BYTES_SEARCH + d * BYTES_RECORD))
+            listed = n if r == 1 else q if r <= 3 else 0
+            out.append(float(n * BYTES_POINT + c * BYTES_COMPONENT + listed * BYTES_LIST + q * BYTES_SEARCH
+                             + d * BYTES_RECORD))
     return out
 
 
@@ -679,7 +684,8 @@ def main():
                 "bytes_model": (f"round 0: {BYTES_FIRST_QUERY} B per query + {BYTES_RECORD_FIRST} B per distinct "
                                 f"internal node visited; later rounds: {BYTES_POINT} B per point + {BYTES_COMPONENT} B per component + "
                                 f"{BYTES_SEARCH} B per query that searches + {BYTES_RECORD} B per distinct "
-                                "internal node visited (counted by an instrumented call); time = the "
+                                f"internal node visited, rounds 1 to 3 also {BYTES_LIST} B per list read (every point in "
+                                "round 1, in 2 and 3 the points that search) (counted by an instrumented call); time = the "
                                 "round's traversal CUDA events in the timed calls"),
                 "per_round": per_round}
 
