@@ -17,7 +17,8 @@ capacity from the node records).
 
 Each candidate runs once to warm up and three times timed (whole-call device
 time from the library's CUDA events, best of three), with the tuning file
-ignored.  The fastest candidate of each class is written as one line of the
+ignored.  The fastest candidate of each class -- the default kernel unless one
+is faster by more than repeated runs differ -- is written as one line of the
 tuning file the library reads (see include/emst.h); every candidate's time is
 printed as a JSON line, so the choices are logged.
 
@@ -34,6 +35,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 DEFAULT_OUT = os.path.join(HERE, "emst_tuning.txt")
 BIG = 1 << 30
+DEFAULT = {"traversal": 1, "block_size": 128, "leaf_size": 1}
+# Repeated runs of one candidate differ by up to 1.5 % below a million points.
+MARGIN = 0.02
 
 # (dim, form, nmin, nmax, representative n or number of instances)
 CLASSES = [
@@ -86,6 +90,14 @@ def time_candidate(pkg, torch, pts, offs, opts, reps=3):
     return best
 
 
+def choose(results):
+    """The (ms, options) to write, of a class's measured candidates, and the
+    default kernel's time."""
+    default_ms = next(ms for ms, opts in results if opts == DEFAULT)
+    ms, opts = min(results, key=lambda r: r[0])
+    return (ms, opts, default_ms) if ms < (1.0 - MARGIN) * default_ms else (default_ms, DEFAULT, default_ms)
+
+
 def tune(out_path: str, quick: bool = False) -> list[dict]:
     import torch
     import paper_2207_00514_gb300 as pkg
@@ -106,10 +118,7 @@ def tune(out_path: str, quick: bool = False) -> list[dict]:
             results.append((ms, opts))
             print(json.dumps({"gpu": gpu, "dim": dim, "form": form, "n": len(pts_np), "ms": round(ms, 4),
                               **opts}), flush=True)
-        results.sort(key=lambda r: r[0])
-        ms, best = results[0]
-        default_ms = next(r[0] for r in results
-                          if r[1] == {"traversal": 1, "block_size": 128, "leaf_size": 1})
+        ms, best, default_ms = choose(results)
         rec = {"gpu": gpu, "dim": dim, "form": form, "nmin": nmin, "nmax": nmax, "n": len(pts_np),
                "best_ms": round(ms, 4), "default_ms": round(default_ms, 4), **best}
         chosen.append(rec)
@@ -123,7 +132,8 @@ def tune(out_path: str, quick: bool = False) -> list[dict]:
         torch.cuda.empty_cache()
     with open(out_path, "w") as f:
         f.write("# emst tuning file (written by paper_2207_00514_gb300/tune.py): per GPU, dimension,\n"
-                "# form and size range, the fastest exact traversal variant measured.\n")
+                "# form and size range, the fastest exact traversal variant measured, the default\n"
+                f"# kernel where none is faster by more than {100 * MARGIN:.0f} %.\n")
         for ln in lines:
             f.write(ln + "\n")
     return chosen
