@@ -24,8 +24,11 @@
  *  - output: exactly n-1 edges (i < j, original point indices), sorted by
  *    that same (w, i, j) order.
  *  - streams: `stream` is a cudaStream_t passed as void* (NULL = the legacy
- *    default stream).  Work is ordered on it; each call returns after that
- *    work has finished (it synchronises the stream once to read the status).
+ *    default stream).  Work is ordered on it; each call returns when its
+ *    result is complete and its status known.  The stream itself may then
+ *    still report work: a call may learn that from a word its last kernel
+ *    writes instead of synchronising the stream.  What the caller puts on the
+ *    stream next follows the call.
  *  - memory: the caller owns inputs and outputs.  Scratch memory is taken
  *    stream-ordered from a library-owned pool on the current device and
  *    returned to the pool before the call returns.
