@@ -12,7 +12,9 @@
 // The merge sequence is serial (its depth is the height of the hierarchy,
 // which single linkage makes long by chaining).  Here the tree is contracted
 // as Boruvka's algorithm would, and the contracted edges are put back into
-// chains (the idea of parallel dendrograms by recursive tree contraction):
+// chains, the idea of P. Sao, A. Prokopenko and D. Lebrun-Grandie, "PANDORA: A
+// Parallel Dendrogram Construction Algorithm for Single Linkage Clustering on
+// GPU" (2024):
 //  - Level 0 is the tree itself.  At every level, each vertex takes its
 //    lowest-ranked edge; the edges taken are contracted, the components they
 //    form are the vertices of the next level and the edges left are its
