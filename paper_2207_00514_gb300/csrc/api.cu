@@ -591,8 +591,8 @@ int run_output(Problem &P, emst_edge *out, uint32_t w_bits, uint32_t *counters) 
   if (P.num_inst == 1 && !P.ties && wb > 0) {
     launch_edge_keys_wi(P, m, L);
     const int s = radix_sort_pairs(P, m, 0, (wb + 7) / 8, 0, L, true);
-    // (the count of long runs is zero since the call's first kernel; the
-    // edges are written without waiting for it, and again below if need be)
+    // (the keys' kernel clears the count of long runs; the edges are written
+    // without waiting for it, and again below if need be)
     launch_edge_ties_w(P, m, s, L);
     launch_edge_from_keys(P, m, s, Lloc, wb, out);
     uint32_t long_runs = 0;

@@ -296,14 +296,15 @@ struct Problem {
   emst_edge *out_stage = nullptr;    // n-1: device staging of host outputs
   uint32_t *counters = nullptr;      // [0] edges emitted, [1] status bits, [2..3] node visits (u64),
                                      // [4..9] scene box (ordered), [10] long tie runs in the output, [28..29] identical curve neighbours (u64), [30..31] code collisions (u64), [32] a run of > 32 equal codes, [11] largest emitted
-                                     // weight bits, [16..23] sort tile counters,
+                                     // weight bits,
                                      // [12] next round's active components, [13] points
                                      // to rerun, [14..15] reruns / queries (learned radius),
                                      // [24] scan tiles finished, [34..35] queries that
                                      // searched (u64), [36..37] the work queue of the
                                      // persistent traversal (u64), [38..39] distinct internal
                                      // nodes visited (u64), [40] this round's active
-                                     // components, [41] rounds done (graph rounds)
+                                     // components, [41] rounds done (graph rounds), [50..52] the
+                                     // listing's (rounds.cu)
   uint32_t *count_dev = nullptr;     // graph rounds: counters + 40 (else nullptr)
   // The host's mailbox (device address of mapped host memory), or null: a
   // round's last kernel posts the counters there, then mail_seq.
@@ -412,7 +413,6 @@ void launch_merge(Problem &P);
 // posts the counters to the host's mailbox (P.mail, P.mail_seq)
 constexpr int kMailWords = 48;
 void launch_post_mail(Problem &P);
-void launch_fill_u32(Problem &P, uint32_t *p, uint32_t v, int64_t count);
 // count runs: adds the bits of the visited-node bitmap to counters[38..39]
 // and clears it for the next round
 void launch_count_seen(Problem &P);

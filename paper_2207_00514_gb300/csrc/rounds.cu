@@ -579,8 +579,8 @@ constexpr int kOrderedUntilRound = EMST_ORDERED_UNTIL_ROUND;  // exact curve ord
 // At 37M halo points the searches of rounds 1 / 2 / 3 fall from 32.4 / 24.7 /
 // 15.2M to 0.9 / 7.4 / 10.4M and the traversal from 29.3 to 22.8 ms (round 0
 // 6.6 -> 11.6, rounds 1-3 8.4 / 6.5 / 3.2 -> 1.4 / 2.5 / 2.4), the call from
-// 44.5 to 38 ms.  Bound, like the search it replaces, by the L1 data pipe and
-// divergence.  Lists read in rounds 1-2 / 1-3 / 1-4 / 1-5: 38.7 / 38.2 / 38.5
+// 44.5 to 38 ms.  Bound by the L1 data pipe (83 % of its wavefronts) and the
+// ALU (78 %: the insertions) together, with 12 of 32 lanes active (4M points).  Lists read in rounds 1-2 / 1-3 / 1-4 / 1-5: 38.7 / 38.2 / 38.5
 // / 38.8 ms; kNearSeed 2 / 3 / 6: round 0 12.18 / 11.86 / 11.56 ms; 40 and 36
 // instead of 32 registers: 12.36 and 12.2 ms.
 // ---------------------------------------------------------------------------
@@ -1289,18 +1289,6 @@ void launch_count_seen(Problem &P) {
   if (!P.seen || P.nc < 2) return;
   const int64_t words = (P.nc - 1 + 31) / 32;
   launch_next(P, k_count_seen, grid_for(words, kBlock), kBlock, 0, P.seen, words, reinterpret_cast<unsigned long long *>(P.counters + 38));
-  P.launches += 1;
-}
-
-__global__ void k_fill_u32(uint32_t *p, uint32_t v, int64_t count) {
-  wait_for_previous();
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < count) p[k] = v;
-}
-
-void launch_fill_u32(Problem &P, uint32_t *p, uint32_t v, int64_t count) {
-  if (count <= 0) return;
-  launch_next(P, k_fill_u32, grid_for(count, kBlock), kBlock, 0, p, v, count);
   P.launches += 1;
 }
 
