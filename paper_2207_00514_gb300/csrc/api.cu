@@ -144,19 +144,19 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
 // waits for the device or that another thread's stream capture forbids.
 namespace {
 std::mutex g_mail_mu;
-std::vector<uint32_t *> &free_mail() {  // (outlives every thread)
-  static std::vector<uint32_t *> *pages = new std::vector<uint32_t *>;
-  return *pages;
-}
+uint32_t *g_free_mail = nullptr;  // the first page, which holds the next one's address (no list to grow, nothing to throw)
+
+uint32_t *&next_page(uint32_t *page) { return *reinterpret_cast<uint32_t **>(page + 64); }
+static_assert(kMailWords + 2 <= 64, "the words of a page come before the address");
 
 struct MailLease {
   uint32_t *page = nullptr;  // null: no mapped memory
   MailLease() {
     {
       std::lock_guard<std::mutex> lock(g_mail_mu);
-      if (!free_mail().empty()) {
-        page = free_mail().back();
-        free_mail().pop_back();
+      if (g_free_mail) {
+        page = g_free_mail;
+        g_free_mail = next_page(page);
         return;
       }
     }
@@ -173,7 +173,8 @@ struct MailLease {
   ~MailLease() {
     if (!page) return;
     std::lock_guard<std::mutex> lock(g_mail_mu);
-    free_mail().push_back(page);
+    next_page(page) = g_free_mail;
+    g_free_mail = page;
   }
   MailLease(const MailLease &) = delete;
   MailLease &operator=(const MailLease &) = delete;
