@@ -430,12 +430,14 @@ __device__ __forceinline__ Segment scan_segments(Segment s, Segment &before) {
 
 // and with many tiles, by the last CTA to finish, what the chain that reaches
 // into each tile gathered in the tiles before it (in place of the tile's
-// total).  Few tiles look for it on their own, back to the last chain start:
-// some steps at most, where the scan takes 6 us of the launch's tail (5,000
-// edges 117 -> 124 us a call); of all tiles it would be quadratic when one
-// chain holds most edges (a path of 100M edges of rising weights 30.6 ms by
-// walks, 16.3 by the scan; of 30M 11.3 and 11.1).
-constexpr int64_t kWalkTiles = 1024;
+// total).  Fewer tiles look for it on their own, back to the last chain start,
+// which a chain of the usual length ends at once; the scan takes 6 to 10 us of
+// the launch's tail (random trees of 5,000 edges 190 -> 196 us a call, of 8M
+// 2,273 -> 2,283).  Of all tiles the walks would be quadratic when one chain
+// holds most edges (paths of rising weights, walks / scan: 8M edges 1,875 /
+// 1,828 us, 100M 30.6 / 16.2 ms), so the line lies where the scan's share is
+// below half a percent and the walks' worst below three.
+constexpr int64_t kWalkTiles = 4096;  // 8.4M edges
 __global__ void __launch_bounds__(kDgBlock) k_dg_tiles(const uint64_t *__restrict__ keys,
                                                        const uint32_t *__restrict__ vals, int64_t m,
                                                        uint2 *tiles, uint32_t *finished,

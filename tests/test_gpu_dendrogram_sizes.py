@@ -74,7 +74,8 @@ def test_not_a_tree():
     check(good, 500)
 
 
-def test_one_chain_over_many_tiles():
+@pytest.mark.parametrize("n", [4_500_000, 9_000_000])
+def test_one_chain_over_many_tiles(n):
     # a path of rising weights is one chain: every tile of the running totals
-    # continues it, over more tiles than the scan takes in one step per thread
-    check(synth.tree_edges(4_500_000, 9, "path_sorted"), 4_500_000)
+    # continues it, found tile by tile at the one size, by the scan at the other
+    check(synth.tree_edges(n, 9, "path_sorted"), n)
