@@ -89,3 +89,35 @@ def test_non_finite_batched():
         part = pts[offsets[k]:offsets[k + 1]]
         if len(part) > 1:
             assert np.array_equal(got[at[k]:at[k + 1]], want(part))
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_overflowing_weights(dim):
+    # nearly all pairs weigh +inf: every search's bounds tie with its best, and
+    # only the tie rule keeps it from visiting every point (4 to 60 times the
+    # time of the same points closer together without it)
+    import statistics
+    import time
+
+    import paper_2207_00514_gb300 as pkg
+    near = np.random.default_rng(dim).normal(size=(40_000, dim)).astype(np.float32)
+    far = near * np.float32(1e25)
+
+    def median_s(points):
+        t = torch.from_numpy(points).cuda()
+        times = []
+        for _ in range(8):
+            torch.cuda.synchronize()
+            a = time.perf_counter()
+            edges = pkg.emst_compute(t)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - a)
+        return statistics.median(times[1:]), words(edges)
+
+    far_s, got = median_s(far)
+    assert far_s < 4 * median_s(near)[0]
+    # (w, i, j): all weigh +inf but the pairs close enough, so nearly all edges meet point 0
+    e, _ = pkg.emst_compute_ex(torch.from_numpy(far).cuda(), traversal=2)  # another search
+    assert np.array_equal(got, words(e))
+    small = far[:3000]
+    assert np.array_equal(words(pkg.emst_compute_ex(torch.from_numpy(small).cuda())[0]), want(small))
