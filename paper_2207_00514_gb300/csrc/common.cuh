@@ -383,14 +383,16 @@ int radix_sort_pairs(Problem &P, int64_t n, int digit_begin, int digit_end, int 
                      bool cleared = false);
 int64_t sort_clear_words(int64_t n);
 // rounds.cu
-// Resident 256-thread CTAs the traversal's registers must allow.  While every
-// point searched, 8 (32 registers, some spilled) was best; over lists, 8 / 6 / 5
-// / 4 take (us per call): 1M 2D blobs 1,310 / 1,265 / 1,263 / 1,263, 3M host
+// Resident 256-thread CTAs the search kernels' registers must allow: few threads
+// with 48 registers each, or many with 32, some of them spilled.  A list of
+// queries fills its warps and is bound by each search's latency: 8 / 6 / 5 / 4
+// CTAs take (us per call) 1M 2D blobs 1,310 / 1,265 / 1,263 / 1,263, 3M host
 // 3,833 / 3,707 / 3,705 / 3,706, 2M dense 3,535 / 3,480 / 3,481 / 3,510, 300k
-// HDBSCAN 1,644 / 1,633 / 1,560 / 1,570, 37M halos (ms) 34.12 / 33.95 / 33.96 / 33.95.
-#ifndef EMST_TRAVERSE_MIN_BLOCKS
-#define EMST_TRAVERSE_MIN_BLOCKS 5
-#endif
+// HDBSCAN 1,644 / 1,633 / 1,560 / 1,570, 37M halos (ms) 34.12 / 33.95 / 33.96 /
+// 33.95.  Where one thread per point searches, where a leaf holds several points
+// and where every visit reads a core distance, warps in flight are what counts as
+// soon as the records exceed the L2 (launch_traverse has the line).
+constexpr int kTraverseFew = 5, kTraverseMany = 8;
 constexpr int kTraverseBlock = 128;     // default traversal CTA size (measured best)
 constexpr int kTraverseMaxBlock = 256;  // largest the traversal kernels are compiled for
 #ifndef EMST_PERSIST_BLOCK

@@ -357,9 +357,10 @@ void launch_upper_bounds(Problem &P) {
 
 // One thread per point, or (list != nullptr) a grid-stride pass over the
 // listed points (the certification reruns of the learned radius).
-template <bool CARRIED, bool RADIUS_IN, bool COUNT, bool SEEDED, bool CHUNKS, bool LEARNED,
+// CTAS: kTraverseFew or kTraverseMany.
+template <int CTAS, bool CARRIED, bool RADIUS_IN, bool COUNT, bool SEEDED, bool CHUNKS, bool LEARNED,
           bool FIRST, bool MRD, bool TIES = true, bool LBT = true, bool KEPT = true>
-__global__ void __launch_bounds__(kTraverseMaxBlock, EMST_TRAVERSE_MIN_BLOCKS) k_traverse(TravArgs A, const uint32_t *__restrict__ list,
+__global__ void __launch_bounds__(kTraverseMaxBlock, CTAS) k_traverse(TravArgs A, const uint32_t *__restrict__ list,
                                                      const uint32_t *__restrict__ list_count) {
   wait_for_previous();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -982,9 +983,12 @@ static int resident_ctas(int block) {
   return b * sm_count();
 }
 
-static void launch_trav(TravKernel k, int g, int block, const Problem &P, const TravArgs &A,
-                        const uint32_t *list, const uint32_t *list_count) {
-  launch_next(P, k, g, block, 0, A, list, list_count);
+// (a launch over the queue: the CTAs the GPU holds at once, so that each warp's
+// first entries are searched at once)
+template <TravKernel K>
+static void launch_trav(int g, int block, const Problem &P, const TravArgs &A, const uint32_t *list,
+                        const uint32_t *list_count) {
+  launch_next(P, K, A.queue ? resident_ctas<K>(block) : g, block, 0, A, list, list_count);
 }
 
 // The tighter lower bound of empty searches (traverse_one's LB) is tracked
@@ -1083,11 +1087,22 @@ void launch_traverse(Problem &P, bool carried, const float *radius_in, int block
     list_count = active_count;
     A.queue = P.counters + kActiveQueue;  // warps take the list in order
   }
-// (a listed launch: the CTAs the GPU holds at once, so that each warp's first
-// entries are searched at once)
-#define EMST_LAUNCH(...)                                                                                       \
-  launch_trav(k_traverse<__VA_ARGS__>, A.queue ? resident_ctas<k_traverse<__VA_ARGS__>>(block) : g, block, P, A, \
-              list, list_count)
+  // Which registers (kTraverseFew, kTraverseMany).  Many threads: chunk leaves
+  // (ms per call, few / many: 300k 3D, 4 points a leaf, 1.89 / 1.84, 3M 8.73 / 8.20,
+  // 37M 102.2 / 95.4); mutual reachability from kManyPoints on (k = 2, 1M 2.24 /
+  // 2.28, 3M 5.37 / 5.23, 37M 57.8 / 54.5); one thread per point from twice that
+  // on (graph rounds 1M 1.88 / 1.92, 3M 4.40 / 4.42, 8M 10.49 / 10.40, 37M 47.1 /
+  // 46.3; the learned form 3M 6.99 / 7.04, 8M 16.5 / 16.4, 37M 76.1 / 75.0).
+  const bool many = P.core2 ? P.n >= kManyPoints : !A.queue && P.n >= 2 * kManyPoints;
+#define EMST_LAUNCH(C1, R1, K1, S1, H1, ...)                                                            \
+  do {                                                                                                  \
+    if constexpr (H1)                                                                                   \
+      launch_trav<k_traverse<kTraverseMany, C1, R1, K1, S1, H1, __VA_ARGS__>>(g, block, P, A, list, list_count); \
+    else if (many)                                                                                      \
+      launch_trav<k_traverse<kTraverseMany, C1, R1, K1, S1, H1, __VA_ARGS__>>(g, block, P, A, list, list_count); \
+    else                                                                                                \
+      launch_trav<k_traverse<kTraverseFew, C1, R1, K1, S1, H1, __VA_ARGS__>>(g, block, P, A, list, list_count); \
+  } while (0)
 // a host flag as a template argument
 #define EMST_IF(flag, B, ...)       \
   do {                              \

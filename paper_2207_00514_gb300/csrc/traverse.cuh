@@ -499,7 +499,7 @@ __device__ __forceinline__ void finish_query(const TravArgs &A, int64_t i, Query
 
 // One query, start to finish (the one-thread-per-point form): the same
 // steps as start_query + explore + finish_query in one piece.  Registers are
-// few (EMST_TRAVERSE_MIN_BLOCKS), so nothing stays live through the search that
+// few (kTraverseFew, kTraverseMany), so nothing stays live through the search that
 // can be read again after it.
 // KEPT: a neighbour of an earlier round may still stand (keep_neighbour) and
 // settles the query; otherwise the caller has ruled that out (the listing
